@@ -5,8 +5,8 @@
 // processing time first). Each block of the persistent kernel then takes the
 // next instance from a device counter and solves it alone, synchronising
 // with __syncthreads only (no block ever waits on another block):
-//   lists   up to SMEM_ELEMS elements: loaded into shared memory and ranked by
-//           Wyllie's pointer jumping there (Sec. 3.1, single-block variant);
+//   lists   up to SMEM_ELEMS elements: loaded into shared memory and ranked
+//           there (block_rank.cuh);
 //           larger: a ruling set inside the block (Sec. 3.2): stratified
 //           splitters, in-place 8-byte walk words in global workspace, the
 //           splitter list held and ranked in shared memory, then the expand.
@@ -24,7 +24,7 @@
 // so the union's min-id labels minus voff[k] are each instance's labels.
 #include <algorithm>
 
-#include "block_wyllie.cuh"
+#include "block_rank.cuh"
 #include "cc_device.cuh"
 #include "common.cuh"
 #include "internal.h"
@@ -35,9 +35,9 @@ namespace {
 
 constexpr int BT = 512;                   // threads per batched block
 constexpr int SMEM_ELEMS = 8192;          // list elements / splitters held in shared memory
-constexpr int PER = SMEM_ELEMS / BT;      // per-thread share in block_wyllie
 constexpr int CC_SMEM_VERTS = 2 * SMEM_ELEMS;
-constexpr size_t SMEM_BYTES = 2 * sizeof(int) * SMEM_ELEMS;   // 64 KB, both kinds
+constexpr size_t CC_SMEM_BYTES = sizeof(int) * CC_SMEM_VERTS;                                   // 64 KB
+constexpr size_t LR_SMEM_BYTES = sizeof(uint64_t) * SMEM_ELEMS + 2 * sizeof(uint2) * BT;       // 72 KB
 constexpr int NCLASS = 33;
 constexpr int64_t CC_LARGE = int64_t(1) << 15;   // graphs above this many vertices go to the union path
 constexpr int SEG_BLOCK = 256;
@@ -90,26 +90,28 @@ __device__ __forceinline__ int64_t take_instance(int* s_k, int64_t count, DevCtl
 // ----------------------------------------------------------------- lists
 
 // Rank one list of n <= SMEM_ELEMS elements in shared memory.
-__device__ void list_in_smem(const int32_t* succ, int n, int head, int32_t* rank, int* val, int* nxt,
-                             DevCtl* ctl) {
+__device__ void list_in_smem(const int32_t* succ, int n, int head, int32_t* rank, uint64_t* W, uint2* sub,
+                             uint32_t seed, DevCtl* ctl) {
+#pragma unroll 4
     for (int i = threadIdx.x; i < n; i += BT) {
         const int s = succ[i];
         const bool tail = (s == -1) | (s == i);
         const bool bad = !tail && (s < 0 || s >= n);
         if (bad) record_error(ctl, LRCC_ERR_INVALID_INPUT, i);
-        nxt[i] = (tail || bad) ? (int)NIL : s;
-        val[i] = 1;
+        W[i] = pack((tail || bad) ? BR_NIL : (uint32_t)s, 1u);
     }
-    __syncthreads();
-    block_wyllie<PER, BT>(val, nxt, n, ctl);
-    for (int i = threadIdx.x; i < n; i += BT) rank[i] = val[i] - 1;
-    if (threadIdx.x == 0 && val[head] != n) record_error(ctl, LRCC_ERR_INVALID_INPUT, head);
+    bool whole;
+    const uint2* res = block_rank<BT>(W, sub, n, head, seed, &whole, ctl);
+    if (threadIdx.x == 0 && !whole) record_error(ctl, LRCC_ERR_INVALID_INPUT, head);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += BT) rank[i] = block_rank_sum<BT>(W[i], res) - 1;
 }
 
 // Rank one larger list with a ruling set inside the block; W is the list's
-// slice of the 8-byte word workspace.
+// slice of the 8-byte word workspace, R the splitters' packed words in shared
+// memory (next splitter, sublist length; before the walk: successor, 1).
 __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_t* rank, uint64_t* W,
-                                int* val, int* nxt, int* s_work, uint32_t seed, int min_logD, DevCtl* ctl) {
+                                uint64_t* R, uint2* sub, int* s_work, uint32_t seed, int min_logD, DevCtl* ctl) {
     // spacing: a power of two, at least 2^min_logD, with at most SMEM_ELEMS splitters
     int logD = max(2, min_logD);
     while (((n + (int64_t(1) << logD) - 1) >> logD) > SMEM_ELEMS) ++logD;
@@ -117,7 +119,7 @@ __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_
     const int r = (int)((n + D - 1) >> logD);
     const int64_t bh = head >> logD;
     const uint32_t head_off = (uint32_t)(head - (bh << logD));
-    // select (RS1+RS2): walk words, and each splitter's successor in nxt[j]
+    // select (RS1+RS2): walk words, and each splitter's successor in R[j]
     for (int64_t i = threadIdx.x; i < n; i += BT) {
         const int s = succ[i];
         const bool tail = (s == -1) | (s == i);
@@ -130,7 +132,7 @@ __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_
         if ((uint32_t)(i - (b << logD)) == off) {
             const int j = (int)(b >= bh ? b - bh : b - bh + r);
             W[i] = pack(nx | SPL, (uint32_t)j);
-            nxt[j] = (int)nx;
+            R[j] = pack(nx, 1);
         } else {
             W[i] = pack(nx, 1);
         }
@@ -141,7 +143,7 @@ __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_
     for (;;) {
         const int j = atomicAdd(s_work, 1);
         if (j >= r) break;
-        uint32_t cur = (uint32_t)nxt[j];
+        uint32_t cur = lo32(R[j]);
         uint32_t pre = 1;
         uint32_t next = NIL;
         int64_t steps = 0;
@@ -164,22 +166,23 @@ __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_
             pre += hi;
             cur = lo;
         }
-        nxt[j] = (int)next;
-        val[j] = (int)pre;
+        R[j] = pack(next == NIL ? BR_NIL : next, pre);
     }
+    // rank the splitters (RS4) in shared memory; their suffix sums replace their words
+    bool whole;
+    const uint2* res = block_rank<BT>(R, sub, r, 0, seed, &whole, ctl);
+    if (threadIdx.x == 0 && (!whole || (int64_t)res[0].y != n)) record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
+    for (int j = threadIdx.x; j < r; j += BT) R[j] = (uint64_t)(uint32_t)block_rank_sum<BT>(R[j], res);
     __syncthreads();
-    // rank the splitters (RS4) in shared memory
-    block_wyllie<PER, BT>(val, nxt, r, ctl);
-    if (threadIdx.x == 0 && val[0] != n) record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
     // expand (RS5)
     for (int64_t i = threadIdx.x; i < n; i += BT) {
         const uint64_t w = W[i];
         const uint32_t lo = lo32(w), hi = hi32(w);
         int out;
         if (lo & SPL) {
-            out = val[hi] - 1;
+            out = (int)lo32(R[hi]) - 1;
         } else if (hi & VIS) {
-            out = val[hi & ~VIS] - (int)lo - 1;
+            out = (int)lo32(R[hi & ~VIS]) - (int)lo - 1;
         } else {
             record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)i);
             out = -1;
@@ -192,9 +195,9 @@ __global__ void __launch_bounds__(BT)
     lr_batch_kernel(const int32_t* __restrict__ succ, const int64_t* __restrict__ off, const int32_t* __restrict__ heads,
                     int64_t count, const int32_t* __restrict__ order, int32_t* __restrict__ rank, uint64_t* W,
                     uint32_t seed, int min_logD, DevCtl* ctl) {
-    extern __shared__ int sm[];
-    int* val = sm;
-    int* nxt = sm + SMEM_ELEMS;
+    extern __shared__ __align__(16) unsigned char lb_raw[];
+    uint64_t* words = reinterpret_cast<uint64_t*>(lb_raw);
+    uint2* sub = reinterpret_cast<uint2*>(lb_raw + sizeof(uint64_t) * SMEM_ELEMS);
     __shared__ int s_k, s_work;
     for (;;) {
         const int64_t q = take_instance(&s_k, count, ctl);
@@ -205,9 +208,10 @@ __global__ void __launch_bounds__(BT)
         const int head = heads[k];
         if (head < 0 || head >= n) continue;
         if (n <= SMEM_ELEMS)
-            list_in_smem(succ + b, (int)n, head, rank + b, val, nxt, ctl);
+            list_in_smem(succ + b, (int)n, head, rank + b, words, sub, seed ^ (uint32_t)k, ctl);
         else
-            list_ruling_set(succ + b, n, head, rank + b, W + b, val, nxt, &s_work, seed ^ (uint32_t)k, min_logD, ctl);
+            list_ruling_set(succ + b, n, head, rank + b, W + b, words, sub, &s_work, seed ^ (uint32_t)k, min_logD,
+                            ctl);
     }
 }
 
@@ -690,8 +694,8 @@ __global__ void __launch_bounds__(SEG_BLOCK)
     }
 }
 
-lrcc_status set_smem(const void* k) {
-    return cuda_status(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+lrcc_status set_smem(const void* k, size_t bytes) {
+    return cuda_status(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
 }
 
 }  // namespace
@@ -725,13 +729,13 @@ lrcc_status lr_batched_run(Ctx* c, const int32_t* succ, const int64_t* off, cons
     phase_begin(c, s);
     batch_order<<<1, 1024, 0, s>>>(off, nullptr, heads, count, order, c->ctl);
     phase_end(c, s, PH_BATCH_PREP);
-    lrcc_status st = set_smem((const void*)lr_batch_kernel);
+    lrcc_status st = set_smem((const void*)lr_batch_kernel, LR_SMEM_BYTES);
     if (st != LRCC_OK) return st;
-    const int g = (int)std::min<int64_t>(count, persistent_grid(c, (const void*)lr_batch_kernel, BT, SMEM_BYTES));
+    const int g = (int)std::min<int64_t>(count, persistent_grid(c, (const void*)lr_batch_kernel, BT, LR_SMEM_BYTES));
     phase_begin(c, s);
     int min_logD = 2;
     while (min_logD < 20 && (1 << (min_logD + 1)) <= p.rs_spacing0) ++min_logD;
-    lr_batch_kernel<<<g, BT, SMEM_BYTES, s>>>(succ, off, heads, count, order, rank, W,
+    lr_batch_kernel<<<g, BT, LR_SMEM_BYTES, s>>>(succ, off, heads, count, order, rank, W,
                                               (uint32_t)(p.seed ^ (p.seed >> 32)), min_logD, c->ctl);
     phase_end(c, s, PH_LR_BATCH);
     return cuda_status(cudaGetLastError());
@@ -846,11 +850,11 @@ lrcc_status cc_batched_run(Ctx* c, const int32_t* src, const int32_t* dst, const
     phase_end(c, s, PH_CC_LOOP);
 
     // every other graph: one block each, largest first
-    lrcc_status st = set_smem((const void*)cc_batch_kernel);
+    lrcc_status st = set_smem((const void*)cc_batch_kernel, CC_SMEM_BYTES);
     if (st != LRCC_OK) return st;
-    const int g = (int)std::min<int64_t>(count, persistent_grid(c, (const void*)cc_batch_kernel, BT, SMEM_BYTES));
+    const int g = (int)std::min<int64_t>(count, persistent_grid(c, (const void*)cc_batch_kernel, BT, CC_SMEM_BYTES));
     phase_begin(c, s);
-    cc_batch_kernel<<<g, BT, SMEM_BYTES, s>>>(src, dst, eoff, voff, count, order, label, p.cc_max_rounds, c->ctl);
+    cc_batch_kernel<<<g, BT, CC_SMEM_BYTES, s>>>(src, dst, eoff, voff, count, order, label, p.cc_max_rounds, c->ctl);
     phase_end(c, s, PH_CC_BATCH);
     return cuda_status(cudaGetLastError());
 }

@@ -18,6 +18,7 @@
 #include <cmath>
 #include <type_traits>
 
+#include "block_rank.cuh"
 #include "block_wyllie.cuh"
 #include "common.cuh"
 #include "internal.h"
@@ -36,74 +37,82 @@ __device__ __forceinline__ void cta_wyllie(int* val, int* nxt, int r, DevCtl* ct
     block_wyllie<PER, FINAL_THREADS>(val, nxt, r, ctl);
 }
 
-// One block ranks a whole list of n <= PER * FINAL_THREADS elements. With
-// weights (w != nullptr) it writes the inclusive suffix sums of w instead of
-// the ranks, after a first pass with unit weights that checks the list.
+// lr_rank_wyllie of a list of n <= PER * FINAL_THREADS elements: pointer
+// jumping inside one block.
 template <int PER>
 __global__ void __launch_bounds__(FINAL_THREADS, 1)
-    lr_small_kernel(const int32_t* __restrict__ succ, const int32_t* __restrict__ w, int n, int head,
-                    int32_t* __restrict__ rank, DevCtl* ctl) {
+    wy_small_kernel(const int32_t* __restrict__ succ, int n, int head, int32_t* __restrict__ rank, DevCtl* ctl) {
     extern __shared__ int sm[];
     int* val = sm;
     int* nxt = sm + PER * FINAL_THREADS;
-    auto load = [&](bool weighted) {
-        for (int i = threadIdx.x; i < n; i += FINAL_THREADS) {
-            const int s = succ[i];
-            const bool tail = (s == -1) | (s == i);
-            const bool bad = !tail && (s < 0 || s >= n);
-            if (bad && !weighted) record_error(ctl, LRCC_ERR_INVALID_INPUT, i);
-            nxt[i] = (tail || bad) ? (int)NIL : s;
-            val[i] = weighted ? w[i] : 1;
-        }
-        __syncthreads();
-    };
-    load(false);
+    for (int i = threadIdx.x; i < n; i += FINAL_THREADS) {
+        const int s = succ[i];
+        const bool tail = (s == -1) | (s == i);
+        const bool bad = !tail && (s < 0 || s >= n);
+        if (bad) record_error(ctl, LRCC_ERR_INVALID_INPUT, i);
+        nxt[i] = (tail || bad) ? (int)NIL : s;
+        val[i] = 1;
+    }
+    __syncthreads();
     cta_wyllie<PER>(val, nxt, n, ctl);
     if (threadIdx.x == 0 && val[head] != n) record_error(ctl, LRCC_ERR_INVALID_INPUT, head);
-    if (w) {
-        __syncthreads();
-        load(true);
-        cta_wyllie<PER>(val, nxt, n, ctl);
+    for (int i = threadIdx.x; i < n; i += FINAL_THREADS) rank[i] = val[i] - 1;
+}
+
+// Shared memory of a one-block ranking of r elements: the packed words and the
+// splitters' two buffers.
+constexpr size_t BR_SUB_BYTES = 2 * sizeof(uint2) * FINAL_THREADS;
+constexpr size_t br_smem(int64_t r) { return sizeof(uint64_t) * (size_t)r + BR_SUB_BYTES; }
+
+// One block ranks a whole list (block_rank.cuh). With weights (w != nullptr)
+// it writes the inclusive suffix sums of w instead of the ranks.
+__global__ void __launch_bounds__(FINAL_THREADS, 1)
+    lr_small_kernel(const int32_t* __restrict__ succ, const int32_t* __restrict__ w, int n, int head,
+                    int32_t* __restrict__ rank, uint32_t seed, DevCtl* ctl) {
+    extern __shared__ __align__(16) unsigned char br_raw[];
+    uint2* sub = reinterpret_cast<uint2*>(br_raw);
+    uint64_t* W = reinterpret_cast<uint64_t*>(br_raw + BR_SUB_BYTES);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += FINAL_THREADS) {
+        const int s = succ[i];
+        const bool tail = (s == -1) | (s == i);
+        const bool bad = !tail && (s < 0 || s >= n);
+        if (bad) record_error(ctl, LRCC_ERR_INVALID_INPUT, i);
+        W[i] = pack((tail || bad) ? BR_NIL : (uint32_t)s, w ? (uint32_t)w[i] : 1u);
     }
+    bool whole;
+    const uint2* res = block_rank<FINAL_THREADS>(W, sub, n, head, seed, &whole, ctl);
+    if (threadIdx.x == 0 && !whole) record_error(ctl, LRCC_ERR_INVALID_INPUT, head);
     const int bias = w ? 0 : 1;
-    for (int i = threadIdx.x; i < n; i += FINAL_THREADS) rank[i] = val[i] - bias;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += FINAL_THREADS) rank[i] = block_rank_sum<FINAL_THREADS>(W[i], res) - bias;
 }
 
 // Last ruling-set level: one block ranks the weighted list of splitters held
 // in packed words R[j] = (next index or NIL, weight) and writes the inclusive
-// suffix weights S. The head splitter (index 0) must see the whole list.
-template <int PER>
+// suffix weights S. The splitters must form one list headed by splitter 0
+// (this also covers weighted sums, where the head's total says nothing about
+// the count), and the head splitter must see the whole list.
 __global__ void __launch_bounds__(FINAL_THREADS, 1)
-    rs_final_kernel(const uint64_t* __restrict__ R, int r, int32_t* __restrict__ S, int64_t expect,
+    rs_final_kernel(const uint64_t* __restrict__ R, int r, int32_t* __restrict__ S, int64_t expect, uint32_t seed,
                     DevCtl* ctl) {
     if (ctl->scan_bad) return;
-    extern __shared__ int sm[];
-    int* val = sm;
-    int* nxt = sm + PER * FINAL_THREADS;
-    // the splitters must form one list headed by splitter 0: every other
-    // splitter has exactly one predecessor, splitter 0 none (this also covers
-    // weighted sums, where the head's total says nothing about the count)
-    for (int j = threadIdx.x; j < r; j += FINAL_THREADS) val[j] = 0;
-    __syncthreads();
-    for (int j = threadIdx.x; j < r; j += FINAL_THREADS) {
-        const uint32_t nx = lo32(R[j]);
-        if (nx < (uint32_t)r) atomicAdd(&val[nx], 1);
-        else if (nx != NIL) record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
-    }
-    __syncthreads();
-    for (int j = threadIdx.x; j < r; j += FINAL_THREADS)
-        if (val[j] != (j == 0 ? 0 : 1)) record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
-    __syncthreads();
+    extern __shared__ __align__(16) unsigned char br_raw[];
+    uint2* sub = reinterpret_cast<uint2*>(br_raw);
+    uint64_t* W = reinterpret_cast<uint64_t*>(br_raw + BR_SUB_BYTES);
+#pragma unroll 4
     for (int j = threadIdx.x; j < r; j += FINAL_THREADS) {
         const uint64_t w = R[j];
-        nxt[j] = (int)lo32(w);
-        val[j] = (int)hi32(w);
+        const uint32_t nx = lo32(w);
+        if (nx >= (uint32_t)r && nx != NIL) record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
+        W[j] = pack(nx < (uint32_t)r ? nx : BR_NIL, hi32(w));
     }
-    __syncthreads();
-    cta_wyllie<PER>(val, nxt, r, ctl);
-    for (int j = threadIdx.x; j < r; j += FINAL_THREADS) S[j] = val[j];
-    if (threadIdx.x == 0 && expect >= 0 && val[0] != expect)
+    bool whole;
+    const uint2* res = block_rank<FINAL_THREADS>(W, sub, r, 0, seed, &whole, ctl);
+    if (threadIdx.x == 0 && (!whole || (expect >= 0 && (int64_t)res[0].y != expect)))
         record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
+#pragma unroll 4
+    for (int j = threadIdx.x; j < r; j += FINAL_THREADS) S[j] = block_rank_sum<FINAL_THREADS>(W[j], res);
 }
 
 // ------------------------------------------------------------ ruling set
@@ -1664,19 +1673,26 @@ __global__ void __launch_bounds__(BLOCK)
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-int small_per(int n) { return n <= 4096 ? 4 : (n <= 8192 ? 8 : 16); }
-
-lrcc_status launch_small(Ctx* c, cudaStream_t s, const int32_t* succ, int n, int head, int32_t* rank,
+lrcc_status launch_small(Ctx* c, cudaStream_t s, const int32_t* succ, int n, int head, int32_t* rank, uint32_t seed,
                          const int32_t* val = nullptr) {
-    const int per = small_per(n);
+    const size_t smem = br_smem(n);
+    cudaFuncSetAttribute((const void*)lr_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    phase_begin(c, s);
+    lr_small_kernel<<<1, FINAL_THREADS, smem, s>>>(succ, val, n, head, rank, seed, c->ctl);
+    phase_end(c, s, PH_SMALL);
+    return cuda_status(cudaGetLastError());
+}
+
+lrcc_status launch_small_wyllie(Ctx* c, cudaStream_t s, const int32_t* succ, int n, int head, int32_t* rank) {
+    const int per = n <= 4096 ? 4 : (n <= 8192 ? 8 : 16);
     const size_t smem = 2 * sizeof(int) * per * FINAL_THREADS;
-    const void* k = per == 4 ? (const void*)lr_small_kernel<4>
-                  : per == 8 ? (const void*)lr_small_kernel<8> : (const void*)lr_small_kernel<16>;
+    const void* k = per == 4 ? (const void*)wy_small_kernel<4>
+                  : per == 8 ? (const void*)wy_small_kernel<8> : (const void*)wy_small_kernel<16>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     phase_begin(c, s);
-    if (per == 4) lr_small_kernel<4><<<1, FINAL_THREADS, smem, s>>>(succ, val, n, head, rank, c->ctl);
-    else if (per == 8) lr_small_kernel<8><<<1, FINAL_THREADS, smem, s>>>(succ, val, n, head, rank, c->ctl);
-    else lr_small_kernel<16><<<1, FINAL_THREADS, smem, s>>>(succ, val, n, head, rank, c->ctl);
+    if (per == 4) wy_small_kernel<4><<<1, FINAL_THREADS, smem, s>>>(succ, n, head, rank, c->ctl);
+    else if (per == 8) wy_small_kernel<8><<<1, FINAL_THREADS, smem, s>>>(succ, n, head, rank, c->ctl);
+    else wy_small_kernel<16><<<1, FINAL_THREADS, smem, s>>>(succ, n, head, rank, c->ctl);
     phase_end(c, s, PH_SMALL);
     return cuda_status(cudaGetLastError());
 }
@@ -1852,7 +1868,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         rs_scan_verdict<<<1, 1, 0, s>>>(c->ctl);
         phase_end(c, s, PH_SELECT0);
     }
-    if (n <= p.rs_small || L.levels == 0) return launch_small(c, s, succ, (int)n, head, rank, val);
+    if (n <= p.rs_small || L.levels == 0) return launch_small(c, s, succ, (int)n, head, rank, (uint32_t)p.seed, val);
     char* base = static_cast<char*>(c->ws);
     auto R = [&](int l) { return reinterpret_cast<uint64_t*>(base + L.off_R[l]); };
     auto SN = [&](int l) { return reinterpret_cast<int32_t*>(base + L.off_snext[l]); };
@@ -2000,19 +2016,10 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     {
         const int lf = L.levels;
         const int r = (int)L.size[lf];
-        const int per = small_per(r);
-        const size_t smem = 2 * sizeof(int) * per * FINAL_THREADS;
+        const size_t smem = br_smem(r);
         phase_begin(c, s);
-        if (per == 4) {
-            cudaFuncSetAttribute((const void*)rs_final_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            rs_final_kernel<4><<<1, FINAL_THREADS, smem, s>>>(R(lf), r, S(lf), val ? -1 : n, ctl);
-        } else if (per == 8) {
-            cudaFuncSetAttribute((const void*)rs_final_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            rs_final_kernel<8><<<1, FINAL_THREADS, smem, s>>>(R(lf), r, S(lf), val ? -1 : n, ctl);
-        } else {
-            cudaFuncSetAttribute((const void*)rs_final_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            rs_final_kernel<16><<<1, FINAL_THREADS, smem, s>>>(R(lf), r, S(lf), val ? -1 : n, ctl);
-        }
+        cudaFuncSetAttribute((const void*)rs_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        rs_final_kernel<<<1, FINAL_THREADS, smem, s>>>(R(lf), r, S(lf), val ? -1 : n, seed0, ctl);
         phase_end(c, s, PH_FINAL);
     }
     for (int l = L.levels - 1; l >= 1; --l) {
@@ -2169,7 +2176,7 @@ lrcc_status lr_enqueue_scan_forest(Ctx* c, cudaStream_t s, const int32_t* succ, 
 
 lrcc_status lr_enqueue_wyllie(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n, int32_t head,
                               int32_t* rank, const Plan& p) {
-    if (n <= p.rs_small) return launch_small(c, s, succ, (int)n, head, rank);
+    if (n <= p.rs_small) return launch_small_wyllie(c, s, succ, (int)n, head, rank);
     uint64_t* W0 = static_cast<uint64_t*>(c->ws);
     uint64_t* W1 = reinterpret_cast<uint64_t*>(static_cast<char*>(c->ws) +
                                                align_up(sizeof(uint64_t) * (size_t)n, 256));
