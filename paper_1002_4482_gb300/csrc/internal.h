@@ -50,8 +50,9 @@ struct RsLayout {
                                     // size[l+1] = ceil(size[l] / 2^logD[l]) splitters at level l
     int64_t size[MAX_LEVELS + 1];   // element bound of each level (size[0] = n)
     int logD[MAX_LEVELS];           // log2 of the splitter spacing of each walked level
-    size_t off_R[MAX_LEVELS + 1], off_snext[MAX_LEVELS + 1], off_sw[MAX_LEVELS + 1],
-        off_S[MAX_LEVELS + 1];
+    // level l >= 1: packed words, per-element records of the walked levels, suffix weights;
+    // level 1 also holds each splitter's successor and weight when level 0 packs walk words
+    size_t off_R[MAX_LEVELS + 1], off_P[MAX_LEVELS + 1], off_S[MAX_LEVELS + 1], off_snext = 0, off_sw = 0;
     size_t off_W0 = 0;
     bool readonly = false;          // level 0 by the read-only walk (chunks, scan, scatter, place)
     bool split = false;             // level 0 over split mark / local-rank arrays

@@ -9,8 +9,8 @@
 //            word is overwritten IN PLACE with (prefix weight, owner | VIS),
 //            so a step costs one random sector read plus its write-back;
 //   recurse  (RS4) the list of splitters, weighted by sublist size, is again
-//            cut by splitters until it fits one thread block, where Wyllie
-//            runs in shared memory (Sec. 3.1, single-block variant);
+//            cut by splitters and walked (rs_chase) until it fits one thread
+//            block, which ranks it in shared memory (block_rank.cuh);
 //   expand   (RS5) streaming passes turn (prefix, owner) into ranks.
 // Every level stores the inclusive suffix weight S (elements from a node to
 // the tail, itself included); the final rank is S - 1.
@@ -222,25 +222,70 @@ __global__ void __launch_bounds__(BLOCK)
     }
 }
 
-// Select at level >= 1: the elements are the previous level's splitters,
-// whose packed words R[j] = (next, weight) are already walk words; the head
-// is element 0. One thread per block rewrites its splitter's word as
-// (next | SPL, block) and records its successor and weight.
-__global__ void __launch_bounds__(BLOCK)
-    rs_select(uint64_t* __restrict__ R, int64_t nl, int32_t* __restrict__ snext, int32_t* __restrict__ sw,
-              int logD, int64_t nb, uint32_t seed, const DevCtl* ctl) {
-    if (ctl->scan_bad) return;
-    const int64_t D = int64_t(1) << logD;
-    for (int64_t b = static_cast<int64_t>(blockIdx.x) * BLOCK + threadIdx.x; b < nb;
-         b += static_cast<int64_t>(gridDim.x) * BLOCK) {
-        const uint32_t size = (uint32_t)min(D, nl - (b << logD));
-        const uint32_t off = b == 0 ? 0u : block_offset((uint32_t)b, size, seed);
-        const int64_t sidx = (b << logD) + off;
-        const uint64_t w = R[sidx];
-        R[sidx] = pack(lo32(w) | SPL, (uint32_t)b);
-        snext[b] = (int32_t)lo32(w);
-        sw[b] = (int32_t)hi32(w);
+// Brent's cycle detection for a walk that only reads: the anchor moves to the
+// current element after 64, 128, 256, ... steps, so a walk caught in a cycle
+// meets its anchor after at most three times the cycle's and its lead's length.
+struct CycleGuard {
+    uint32_t anchor, steps = 0, limit = 64;
+    __device__ __forceinline__ explicit CycleGuard(uint32_t start) : anchor(start) {}
+    // true when `cur` was visited before
+    __device__ __forceinline__ bool seen(uint32_t cur) {
+        if (cur == anchor) return true;
+        if (++steps == limit) {
+            anchor = cur;
+            limit *= 2;
+        }
+        return false;
     }
+};
+
+// Sublist walk at level >= 1 (RS2 and RS3 in one kernel): the elements are the
+// previous level's splitters with packed words R[i] = (next, weight), the head
+// is element 0. Thread j starts at the splitter of block j, steps until the
+// next element is a splitter (recognised by its hashed offset, so nothing has
+// to be marked first), and stores P[i] = (prefix weight, owner) for every
+// element it visits and Rout[j] = (next splitter, weight of its sublist).
+//
+// These levels are L2-resident and bound by the latency of the longest sublist
+// (about D ln r steps), so a step is one dependent read of 304 cycles and
+// little else: the splitter test of the next element runs while its word is on
+// the way, one thread takes one sublist (no hand-out between steps), and the
+// words read are not the words written. The form before marked the splitters
+// in a pass of their own and overwrote R in place; a store to a line that was
+// just read costs the L2 far more than a store elsewhere (read-then-store runs
+// at 29-65 G/s, reads alone at 290, stores alone at 180-206).
+__global__ void __launch_bounds__(BLOCK)
+    rs_chase(const uint64_t* __restrict__ R, uint32_t nl, uint64_t* __restrict__ P, uint64_t* __restrict__ Rout,
+             uint32_t r, int logD, uint32_t seed, DevCtl* ctl) {
+    if (ctl->scan_bad) return;
+    const uint32_t j = blockIdx.x * BLOCK + threadIdx.x;
+    if (j >= r) return;
+    const uint32_t D = 1u << logD;
+    auto offset = [&](uint32_t b) {
+        return b == 0 ? 0u : block_offset(b, min(D, nl - (b << logD)), seed);
+    };
+    const uint32_t start = (j << logD) + offset(j);
+    uint64_t w = R[start];
+    P[start] = pack(0, j);
+    uint32_t cur = lo32(w), pre = hi32(w);
+    CycleGuard guard(start);
+    uint32_t next = NIL;
+    while (cur != NIL) {
+        if (cur >= nl || guard.seen(cur)) {
+            record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)cur);
+            break;
+        }
+        w = R[cur];
+        const uint32_t b = cur >> logD;
+        if ((cur & (D - 1)) == offset(b)) {
+            next = b;
+            break;
+        }
+        P[cur] = pack(pre, j);
+        pre += hi32(w);
+        cur = lo32(w);
+    }
+    Rout[j] = pack(next, pre);
 }
 
 // Sublist walk (RS3). Each thread keeps K walks in flight so that K
@@ -999,22 +1044,15 @@ __global__ void __launch_bounds__(BLOCK)
 
 // Expand at level >= 1: S[c] = S_next[owner] - prefix (RS5).
 __global__ void __launch_bounds__(BLOCK)
-    rs_expand(const uint64_t* __restrict__ W, int r, const int32_t* __restrict__ Snext, int rnext,
+    rs_expand(const uint64_t* __restrict__ P, uint32_t r, const int32_t* __restrict__ Snext, uint32_t rnext,
               int32_t* __restrict__ S, DevCtl* ctl) {
     if (ctl->scan_bad) return;
-    for (int c = blockIdx.x * BLOCK + threadIdx.x; c < r; c += gridDim.x * BLOCK) {
-        const uint64_t w = W[c];
-        const uint32_t lo = lo32(w), hi = hi32(w);
-        // indices are checked so that a malformed input can only give wrong
-        // values (with an error recorded), never an access outside Snext
-        if ((lo & SPL) && hi < (uint32_t)rnext) {
-            S[c] = Snext[hi];
-        } else if (!(lo & SPL) && (hi & VIS) && (hi & ~VIS) < (uint32_t)rnext) {
-            S[c] = (int32_t)((uint32_t)Snext[hi & ~VIS] - lo);
-        } else {
-            record_error(ctl, LRCC_ERR_INVALID_INPUT, c);
-            S[c] = 0;
-        }
+    for (uint32_t c = blockIdx.x * BLOCK + threadIdx.x; c < r; c += gridDim.x * BLOCK) {
+        const uint64_t p = P[c];
+        // an element no walk reached holds an old word: its owner is checked, so
+        // that a malformed input can only give wrong values (the last level has
+        // recorded it), never an access outside Snext
+        S[c] = hi32(p) < rnext ? (int32_t)((uint32_t)Snext[hi32(p)] - lo32(p)) : 0;
     }
 }
 
@@ -1765,12 +1803,15 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
         ++lvl;
         L.size[lvl] = nb;
         L.off_R[lvl] = take(sizeof(uint64_t) * (size_t)nb);
-        L.off_snext[lvl] = take(sizeof(int32_t) * (size_t)nb);
-        L.off_sw[lvl] = take(sizeof(int32_t) * (size_t)nb);
+        if (lvl == 1) {
+            L.off_snext = take(sizeof(int32_t) * (size_t)nb);
+            L.off_sw = take(sizeof(int32_t) * (size_t)nb);
+        }
         L.off_S[lvl] = take(sizeof(int32_t) * (size_t)nb);
         cur = nb;
     }
     L.levels = lvl;
+    for (int l = 1; l < lvl; ++l) L.off_P[l] = take(sizeof(uint64_t) * (size_t)L.size[l]);
     L.readonly = p.rs_level0 == 2 && lvl > 0 && walk_grid > 0;
     L.split = p.rs_level0 == 3 && lvl > 0;
     if (L.readonly) {
@@ -1871,8 +1912,9 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     if (n <= p.rs_small || L.levels == 0) return launch_small(c, s, succ, (int)n, head, rank, (uint32_t)p.seed, val);
     char* base = static_cast<char*>(c->ws);
     auto R = [&](int l) { return reinterpret_cast<uint64_t*>(base + L.off_R[l]); };
-    auto SN = [&](int l) { return reinterpret_cast<int32_t*>(base + L.off_snext[l]); };
-    auto SW = [&](int l) { return reinterpret_cast<int32_t*>(base + L.off_sw[l]); };
+    auto P = [&](int l) { return reinterpret_cast<uint64_t*>(base + L.off_P[l]); };
+    int32_t* SN = reinterpret_cast<int32_t*>(base + L.off_snext);
+    int32_t* SW = reinterpret_cast<int32_t*>(base + L.off_sw);
     auto S = [&](int l) { return reinterpret_cast<int32_t*>(base + L.off_S[l]); };
     uint64_t* W0 = reinterpret_cast<uint64_t*>(base + L.off_W0);
     DevCtl* ctl = c->ctl;
@@ -1886,14 +1928,14 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         const int g = stream_grid(c, groups, k);
         phase_begin(c, s);
         if (vec)
-            rs_select0<true><<<g, BLOCK, 0, s>>>(succ, val, n, head, W0, SN(1), SW(1), L.logD[0], L.size[1],
+            rs_select0<true><<<g, BLOCK, 0, s>>>(succ, val, n, head, W0, SN, SW, L.logD[0], L.size[1],
                                                  seed0, ctl, given == nullptr);
         else
-            rs_select0<false><<<g, BLOCK, 0, s>>>(succ, val, n, head, W0, SN(1), SW(1), L.logD[0], L.size[1],
+            rs_select0<false><<<g, BLOCK, 0, s>>>(succ, val, n, head, W0, SN, SW, L.logD[0], L.size[1],
                                                   seed0, ctl, given == nullptr);
         if (given) {
             const int gm = stream_grid(c, given_r, (const void*)rs_mark_given);
-            rs_mark_given<<<gm, BLOCK, 0, s>>>(W0, n, head, given, given_r, SN(1), SW(1), ctl);
+            rs_mark_given<<<gm, BLOCK, 0, s>>>(W0, n, head, given, given_r, SN, SW, ctl);
         }
         phase_end(c, s, PH_SELECT0);
     }
@@ -1926,10 +1968,10 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         phase_begin(c, s);
         if (mark16) {
             const int g = stream_grid(c, n, (const void*)rs_select0s<uint16_t>);
-            rs_select0s<uint16_t><<<g, BLOCK, 0, s>>>(succ, (uint16_t*)mark, lrank, SN(1), SW(1), L0, ctl);
+            rs_select0s<uint16_t><<<g, BLOCK, 0, s>>>(succ, (uint16_t*)mark, lrank, SN, SW, L0, ctl);
         } else {
             const int g = stream_grid(c, n, (const void*)rs_select0s<uint32_t>);
-            rs_select0s<uint32_t><<<g, BLOCK, 0, s>>>(succ, (uint32_t*)mark, lrank, SN(1), SW(1), L0, ctl);
+            rs_select0s<uint32_t><<<g, BLOCK, 0, s>>>(succ, (uint32_t*)mark, lrank, SN, SW, L0, ctl);
         }
         phase_end(c, s, PH_SELECT0);
     }
@@ -1949,21 +1991,21 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     while ((int64_t(1) << lg) < n) ++lg;
     C.shift = std::max(0, lg - NBK_LOG);
     C.careful = int64_t(32) << L.logD[0];
-    auto walk = [&](int l, uint64_t* Wl, int64_t nl) {
-        const int r = (int)L.size[l + 1];
-        int* work = &ctl->work[l];
+    auto walk0 = [&] {
+        const int r = (int)L.size[1];
+        int* work = &ctl->work[0];
         phase_begin(c, s);
         if (p.rs_chains >= 4) {
             const int g = persistent_grid(c, (const void*)rs_walk<4>, BLOCK);
-            rs_walk<4><<<g, BLOCK, 0, s>>>(Wl, SN(l + 1), SW(l + 1), R(l + 1), r, work, nl, ctl);
+            rs_walk<4><<<g, BLOCK, 0, s>>>(W0, SN, SW, R(1), r, work, n, ctl);
         } else if (p.rs_chains == 2) {
             const int g = persistent_grid(c, (const void*)rs_walk<2>, BLOCK);
-            rs_walk<2><<<g, BLOCK, 0, s>>>(Wl, SN(l + 1), SW(l + 1), R(l + 1), r, work, nl, ctl);
+            rs_walk<2><<<g, BLOCK, 0, s>>>(W0, SN, SW, R(1), r, work, n, ctl);
         } else {
             const int g = persistent_grid(c, (const void*)rs_walk<1>, BLOCK);
-            rs_walk<1><<<g, BLOCK, 0, s>>>(Wl, SN(l + 1), SW(l + 1), R(l + 1), r, work, nl, ctl);
+            rs_walk<1><<<g, BLOCK, 0, s>>>(W0, SN, SW, R(1), r, work, n, ctl);
         }
-        phase_end(c, s, l == 0 ? PH_WALK0 : PH_WALK);
+        phase_end(c, s, PH_WALK0);
     };
     if (L.readonly) {
         cudaMemsetAsync(C.vis, 0, sizeof(uint32_t) * (size_t)((n + 31) / 32), s);
@@ -1989,7 +2031,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
             using MT = decltype(mt);
             constexpr int K = decltype(k)::value;
             const int g = persistent_grid(c, (const void*)rs_walk0s<MT, K>, BLOCK);
-            rs_walk0s<MT, K><<<g, BLOCK, 0, s>>>(succ, (MT*)mark, lrank, SN(1), R(1), &ctl->work[0], L0, ctl);
+            rs_walk0s<MT, K><<<g, BLOCK, 0, s>>>(succ, (MT*)mark, lrank, SN, R(1), &ctl->work[0], L0, ctl);
         };
         phase_begin(c, s);
         if (mark16) {
@@ -2003,15 +2045,15 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         }
         phase_end(c, s, PH_WALK0);
     } else {
-        walk(0, W0, n);
+        walk0();
     }
     for (int l = 1; l < L.levels; ++l) {
         const uint32_t seed = mix32(seed0 + 0x9E3779B9u * (uint32_t)l);
-        const int g = stream_grid(c, L.size[l + 1], (const void*)rs_select);
+        const unsigned g = (unsigned)((L.size[l + 1] + BLOCK - 1) / BLOCK);
         phase_begin(c, s);
-        rs_select<<<g, BLOCK, 0, s>>>(R(l), L.size[l], SN(l + 1), SW(l + 1), L.logD[l], L.size[l + 1], seed, ctl);
-        phase_end(c, s, PH_SELECT);
-        walk(l, R(l), L.size[l]);
+        rs_chase<<<g, BLOCK, 0, s>>>(R(l), (uint32_t)L.size[l], P(l), R(l + 1), (uint32_t)L.size[l + 1], L.logD[l], seed,
+                                     ctl);
+        phase_end(c, s, PH_WALK);
     }
     {
         const int lf = L.levels;
@@ -2025,7 +2067,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     for (int l = L.levels - 1; l >= 1; --l) {
         const int g = stream_grid(c, L.size[l], (const void*)rs_expand);
         phase_begin(c, s);
-        rs_expand<<<g, BLOCK, 0, s>>>(R(l), (int)L.size[l], S(l + 1), (int)L.size[l + 1], S(l), ctl);
+        rs_expand<<<g, BLOCK, 0, s>>>(P(l), (uint32_t)L.size[l], S(l + 1), (uint32_t)L.size[l + 1], S(l), ctl);
         phase_end(c, s, PH_EXPAND);
     }
     if (U) {
