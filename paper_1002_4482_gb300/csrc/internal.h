@@ -56,6 +56,9 @@ struct RsLayout {
     size_t off_W0 = 0;
     bool readonly = false;          // level 0 by the read-only walk (chunks, scan, scatter, place)
     bool split = false;             // level 0 over split mark / local-rank arrays
+    bool direct = false;            // level 0 through 4-byte records in the rank array
+    int pbits = 0;                  // direct: position bits of a record
+    int64_t fixed = 0;              // direct: first-level splitters before the extra owners
     int64_t grid = 0, cap = 0, ovf_cap = 0;
     int segcap = 0, units = 0;
     size_t off_ids = 0, off_meta = 0, off_fill = 0, off_counts = 0, off_totals = 0,
@@ -64,7 +67,17 @@ struct RsLayout {
 };
 // extra1: extra first-level splitters (the heads of batched lists ranked as one list)
 // given1: the number of first-level splitters when the caller chooses them
-RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1 = 0, int64_t given1 = 0);
+// direct: whether an in-place first level may keep its records in the rank array
+// (unweighted ranks, stratified splitters, rank not overlapping succ)
+RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1 = 0, int64_t given1 = 0,
+                   bool direct = false);
+// Largest list ranked that way: succ and rank (8 bytes per element) stay in L2.
+constexpr int64_t DIRECT_MAX = int64_t(1) << 24;
+// Whether the n-element arrays succ and rank share memory.
+inline bool arrays_overlap(const int32_t* a, const int32_t* b, int64_t n) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return (x > y ? x - y : y - x) < sizeof(int32_t) * (uintptr_t)n;
+}
 
 // Batched lists ranked as one list by the read-only first level: K lists own
 // [off[k], off[k+1]) of succ with local ids; device scratch for the global

@@ -90,13 +90,14 @@ __global__ void __launch_bounds__(FINAL_THREADS, 1)
 
 // Last ruling-set level: one block ranks the weighted list of splitters held
 // in packed words R[j] = (next index or NIL, weight) and writes the inclusive
-// suffix weights S. The splitters must form one list headed by splitter 0
-// (this also covers weighted sums, where the head's total says nothing about
-// the count), and the head splitter must see the whole list.
+// suffix weights S. The head splitter (index 0) must see the whole list:
+// `expect` elements, or, for weighted sums (expect < 0), whose total says
+// nothing about the count, every one of the r splitters.
 __global__ void __launch_bounds__(FINAL_THREADS, 1)
-    rs_final_kernel(const uint64_t* __restrict__ R, int r, int32_t* __restrict__ S, int64_t expect, uint32_t seed,
-                    DevCtl* ctl) {
+    rs_final_kernel(const uint64_t* __restrict__ R, int r, int fixed, int32_t* __restrict__ S, int64_t expect,
+                    uint32_t seed, DevCtl* ctl) {
     if (ctl->scan_bad) return;
+    if (fixed < r) r = min(r, fixed + ctl->ff_extra);   // extra owners in use (rs_walk_direct)
     extern __shared__ __align__(16) unsigned char br_raw[];
     uint2* sub = reinterpret_cast<uint2*>(br_raw);
     uint64_t* W = reinterpret_cast<uint64_t*>(br_raw + BR_SUB_BYTES);
@@ -109,7 +110,9 @@ __global__ void __launch_bounds__(FINAL_THREADS, 1)
     }
     bool whole;
     const uint2* res = block_rank<FINAL_THREADS>(W, sub, r, 0, seed, &whole, ctl);
-    if (threadIdx.x == 0 && (!whole || (expect >= 0 && (int64_t)res[0].y != expect)))
+    // with a total to expect, the head's total decides (it counts elements, and the
+    // path from the head holds each once); splitters off the path are then empty ones
+    if (threadIdx.x == 0 && (expect >= 0 ? (int64_t)res[0].y != expect : !whole))
         record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
 #pragma unroll 4
     for (int j = threadIdx.x; j < r; j += FINAL_THREADS) S[j] = block_rank_sum<FINAL_THREADS>(W[j], res);
@@ -241,7 +244,8 @@ struct CycleGuard {
 
 // Sublist walk at level >= 1 (RS2 and RS3 in one kernel): the elements are the
 // previous level's splitters with packed words R[i] = (next, weight), the head
-// is element 0. Thread j starts at the splitter of block j, steps until the
+// is element 0; elements from `fixed` on are extra owners of the first level,
+// of which ctl->ff_extra are in use. Thread j starts at the splitter of block j, steps until the
 // next element is a splitter (recognised by its hashed offset, so nothing has
 // to be marked first), and stores P[i] = (prefix weight, owner) for every
 // element it visits and Rout[j] = (next splitter, weight of its sublist).
@@ -256,7 +260,7 @@ struct CycleGuard {
 // at 29-65 G/s, reads alone at 290, stores alone at 180-206).
 __global__ void __launch_bounds__(BLOCK)
     rs_chase(const uint64_t* __restrict__ R, uint32_t nl, uint64_t* __restrict__ P, uint64_t* __restrict__ Rout,
-             uint32_t r, int logD, uint32_t seed, DevCtl* ctl) {
+             uint32_t r, int logD, uint32_t seed, uint32_t fixed, DevCtl* ctl) {
     if (ctl->scan_bad) return;
     const uint32_t j = blockIdx.x * BLOCK + threadIdx.x;
     if (j >= r) return;
@@ -265,6 +269,10 @@ __global__ void __launch_bounds__(BLOCK)
         return b == 0 ? 0u : block_offset(b, min(D, nl - (b << logD)), seed);
     };
     const uint32_t start = (j << logD) + offset(j);
+    if (start >= fixed && start - fixed >= (uint32_t)ctl->ff_extra) {   // an extra owner nobody took
+        Rout[j] = pack(NIL, 0);
+        return;
+    }
     uint64_t w = R[start];
     P[start] = pack(0, j);
     uint32_t cur = lo32(w), pre = hi32(w);
@@ -1099,6 +1107,90 @@ __global__ void __launch_bounds__(BLOCK)
     }
 }
 
+// ------------------------------------------------ level 0, ranks in place
+//
+// First level of lists whose successors and ranks fit L2 together: the walk
+// reads succ and writes one 4-byte record (owner, position) per element into
+// the caller's rank array, which a streaming pass turns into the rank
+// S1[owner] - 1 - position. No pass packs walk words first (splitters are
+// recognised by their hashed offset), no workspace per element is needed, and
+// 8 bytes per element are touched at random where the packed words cost 16;
+// reading one array and writing another also keeps the walk from storing to
+// lines it has just read (read-then-store runs at 29-65 G/s on GB300, reads
+// alone at 290, stores alone at 180-206). lr_rank of 100,003 elements 67.7 ->
+// 37.1 us, 2^20 106.7 -> 67.5, 15,000,001 479 -> 460 (there succ and rank are 120
+// of L2's 129 MB, and the walk waits on HBM again).
+//
+// The record has the owner in its high bits and `pbits` bits of position. A
+// sublist longer than 2^pbits goes on under an extra owner index nb + e, which
+// the splitter before it links to; at most n >> pbits of them exist.
+
+__global__ void __launch_bounds__(BLOCK)
+    rs_walk_direct(const int32_t* __restrict__ succ, uint32_t* __restrict__ rec, Level0 L0, int pbits, int extras,
+                   uint64_t* __restrict__ R1, DevCtl* ctl) {
+    const Geo32 g = geo32(L0);
+    uint32_t j = blockIdx.x * BLOCK + threadIdx.x;
+    if (j >= g.nb) return;
+    uint32_t cur = splitter_node32(j, g, nullptr), pos = 0;
+    int32_t x = __ldg(succ + cur);
+    CycleGuard guard(cur);
+    uint32_t next = NIL;
+    for (;;) {
+        // cur belongs to owner j at position pos, x = succ[cur]
+        rec[cur] = (j << pbits) | pos;
+        ++pos;
+        if (x == -1 || (uint32_t)x == cur) break;
+        if ((uint32_t)x >= g.n || guard.seen((uint32_t)x)) {
+            record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)cur);
+            break;
+        }
+        cur = (uint32_t)x;
+        x = __ldg(succ + cur);   // on its way while cur is tested
+        const int sj = splitter_index32(cur, g);
+        if (sj >= 0) {
+            next = (uint32_t)sj;
+            break;
+        }
+        if (pos >> pbits) {
+            const int e = atomicAdd(&ctl->ff_extra, 1);
+            if (e >= extras) {
+                record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)cur);
+                break;
+            }
+            R1[j] = pack(g.nb + (uint32_t)e, pos);
+            j = g.nb + (uint32_t)e;
+            pos = 0;
+        }
+    }
+    R1[j] = pack(next, pos);
+}
+
+// Records -> ranks, in place. Records of elements no walk reached (a malformed
+// input, which the last level has recorded) may name any owner: -1 then.
+template <bool VEC>
+__global__ void __launch_bounds__(BLOCK)
+    rs_expand_direct(int32_t* rank, int64_t n, const int32_t* __restrict__ S1, uint32_t r1, int pbits) {
+    const uint32_t mask = (1u << pbits) - 1;
+    auto rank_of = [&](int32_t v) {
+        const uint32_t o = (uint32_t)v >> pbits;
+        return o < r1 ? S1[o] - 1 - (int32_t)((uint32_t)v & mask) : -1;
+    };
+    const int64_t ngroups = (n + 3) >> 2;
+    for (int64_t g = static_cast<int64_t>(blockIdx.x) * BLOCK + threadIdx.x; g < ngroups;
+         g += static_cast<int64_t>(gridDim.x) * BLOCK) {
+        const int64_t i0 = g * 4;
+        if (VEC && i0 + 3 < n) {
+            int4* p = reinterpret_cast<int4*>(rank + i0);
+            const int4 v = *p;
+            *p = make_int4(rank_of(v.x), rank_of(v.y), rank_of(v.z), rank_of(v.w));
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (i0 + q < n) rank[i0 + q] = rank_of(rank[i0 + q]);
+        }
+    }
+}
+
 // ------------------------------------------------ level 0, split arrays
 //
 // The paper's other first-level layout (Sec. 3.2, the "48 bit" version): the
@@ -1775,9 +1867,10 @@ int rs_walk_grid_current(const Plan& p) {
     return per_sm * sms;
 }
 
-RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int64_t given1) {
+RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int64_t given1, bool direct) {
     RsLayout L;
     L.size[0] = n;
+    direct = direct && p.rs_level0 == 1 && n > p.rs_small && n <= DIRECT_MAX;
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
@@ -1786,7 +1879,7 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
     };
     // in-place walk words, the (element, rank) pairs of the read-only walk, or
     // the split mark and local-rank arrays (each 256-byte aligned)
-    L.off_W0 = take(sizeof(uint64_t) * (size_t)n + 256);
+    if (!direct) L.off_W0 = take(sizeof(uint64_t) * (size_t)n + 256);
     int64_t cur = n;
     int lvl = 0;
     while (cur > p.rs_small && lvl < MAX_LEVELS) {
@@ -1799,11 +1892,20 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
         // level 1 may hold extra splitters (the heads of batched lists ranked as one list)
         int64_t nb = ((cur + (int64_t(1) << logD) - 1) >> logD) + (lvl == 0 ? extra1 : 0);
         if (lvl == 0 && given1 > 0) nb = given1;   // first-level splitters chosen by the caller
+        if (lvl == 0 && direct) {
+            // as many position bits as the owners leave, extra owners included
+            L.direct = true;
+            L.fixed = nb;
+            for (L.pbits = 31; L.pbits > 0; --L.pbits) {
+                nb = L.fixed + (n >> L.pbits);
+                if (nb <= (int64_t(1) << (32 - L.pbits))) break;
+            }
+        }
         L.logD[lvl] = logD;
         ++lvl;
         L.size[lvl] = nb;
         L.off_R[lvl] = take(sizeof(uint64_t) * (size_t)nb);
-        if (lvl == 1) {
+        if (lvl == 1 && !direct) {
             L.off_snext = take(sizeof(int32_t) * (size_t)nb);
             L.off_sw = take(sizeof(int32_t) * (size_t)nb);
         }
@@ -1898,11 +2000,11 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
                           int32_t* rank, const Plan& p, const RsLayout& L, const int32_t* val,
                           const BatchUnion* U, const int32_t* given, int64_t given_r) {
     // caller-chosen first-level splitters need the in-place first level
-    if (given && (L.readonly || L.split || U)) return LRCC_ERR_ARG;
+    if (given && (L.readonly || L.split || L.direct || U)) return LRCC_ERR_ARG;
     // batched lists ranked as one list need the read-only first level
     if (U && (!L.readonly || val)) return LRCC_ERR_ARG;
     // weighted sums use the in-place first level (the others count positions)
-    if (val && (L.readonly || L.split)) return LRCC_ERR_ARG;
+    if (val && (L.readonly || L.split || L.direct)) return LRCC_ERR_ARG;
     if (val) {
         phase_begin(c, s);
         rs_scan_check<<<stream_grid(c, n, (const void*)rs_scan_check), BLOCK, 0, s>>>(val, n, c->ctl);
@@ -1923,7 +2025,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     // level 0
     const bool vec = aligned16(succ) && (!val || aligned16(val));
     const int64_t groups = (n + 3) / 4;
-    if (!L.readonly && !L.split) {
+    if (!L.readonly && !L.split && !L.direct) {
         const void* k = vec ? (const void*)rs_select0<true> : (const void*)rs_select0<false>;
         const int g = stream_grid(c, groups, k);
         phase_begin(c, s);
@@ -2044,6 +2146,11 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
             else walk0s(uint32_t(), std::integral_constant<int, 1>());
         }
         phase_end(c, s, PH_WALK0);
+    } else if (L.direct) {
+        phase_begin(c, s);
+        rs_walk_direct<<<(unsigned)((L0.nb + BLOCK - 1) / BLOCK), BLOCK, 0, s>>>(
+            succ, reinterpret_cast<uint32_t*>(rank), L0, L.pbits, (int)(L.size[1] - L.fixed), R(1), ctl);
+        phase_end(c, s, PH_WALK0);
     } else {
         walk0();
     }
@@ -2052,7 +2159,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         const unsigned g = (unsigned)((L.size[l + 1] + BLOCK - 1) / BLOCK);
         phase_begin(c, s);
         rs_chase<<<g, BLOCK, 0, s>>>(R(l), (uint32_t)L.size[l], P(l), R(l + 1), (uint32_t)L.size[l + 1], L.logD[l], seed,
-                                     ctl);
+                                     l == 1 && L.direct ? (uint32_t)L.fixed : 0xFFFFFFFFu, ctl);
         phase_end(c, s, PH_WALK);
     }
     {
@@ -2061,7 +2168,8 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         const size_t smem = br_smem(r);
         phase_begin(c, s);
         cudaFuncSetAttribute((const void*)rs_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        rs_final_kernel<<<1, FINAL_THREADS, smem, s>>>(R(lf), r, S(lf), val ? -1 : n, seed0, ctl);
+        rs_final_kernel<<<1, FINAL_THREADS, smem, s>>>(R(lf), r, lf == 1 && L.direct ? (int)L.fixed : r, S(lf),
+                                                       val ? -1 : n, seed0, ctl);
         phase_end(c, s, PH_FINAL);
     }
     for (int l = L.levels - 1; l >= 1; --l) {
@@ -2093,6 +2201,14 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
             const int g = stream_grid(c, n, (const void*)rs_expand0s<uint32_t>);
             rs_expand0s<uint32_t><<<g, BLOCK, 0, s>>>((const uint32_t*)mark, lrank, n, S(1), L.size[1], rank, ctl);
         }
+        phase_end(c, s, PH_EXPAND0);
+    } else if (L.direct) {
+        const bool v = aligned16(rank);
+        const void* k = v ? (const void*)rs_expand_direct<true> : (const void*)rs_expand_direct<false>;
+        const int g = stream_grid(c, groups, k);
+        phase_begin(c, s);
+        if (v) rs_expand_direct<true><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits);
+        else rs_expand_direct<false><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits);
         phase_end(c, s, PH_EXPAND0);
     } else {
         const bool v = vec && aligned16(rank);

@@ -50,12 +50,14 @@ std::mutex g_noalloc_mu;
 void* g_noalloc_ptr[NOALLOC_MAX_DEVICES] = {};
 int g_noalloc_sms[NOALLOC_MAX_DEVICES] = {};
 
-// Fixed plan: in-place first level (no chunk buffers), spacing 16 at every
-// level, lists of at most 8192 elements ranked by one block.
-Plan noalloc_plan() {
+// Fixed plan: in-place first level (no chunk buffers), lists of at most 8192
+// elements ranked by one block. Records in the rank array leave room for the
+// short spacings of lr_rank's plan; a caller that ranks in place (rank = succ)
+// needs 8-byte walk words, and spacing 16 at every level for the rest to fit.
+Plan noalloc_plan(bool direct) {
     Plan p;
-    p.rs_spacing0 = 16;
-    p.rs_spacing = 16;
+    p.rs_spacing0 = direct ? 8 : 16;
+    p.rs_spacing = direct ? 4 : 16;
     p.rs_small = 8192;
     p.rs_chains = 1;
     p.rs_level0 = 1;
@@ -107,8 +109,9 @@ extern "C" lrcc_status lr_rank_noalloc(const int32_t* succ, int64_t n, int32_t h
     int sms = 0;
     lrcc_status st = scratch_for(dev, &scratch, &sms);
     if (st != LRCC_OK) return st;
-    const Plan p = noalloc_plan();
-    const RsLayout L = rs_layout(n, p, 0);
+    const bool direct = !arrays_overlap(succ, rank, n);
+    const Plan p = noalloc_plan(direct);
+    const RsLayout L = rs_layout(n, p, 0, 0, 0, direct);
     const size_t ctl_off = align_up(L.bytes, 256);
     if (ctl_off + sizeof(DevCtl) > NOALLOC_SCRATCH_BYTES) return LRCC_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -65,20 +65,17 @@ void init_plans_locked() {
             Plan& p = g_plan[k][l];
             p = Plan{};
             p.rs_small = 16384;
-            if (l <= 22) {
-                // deeper levels at spacing 4: their walks are latency-bound, and
-                // shorter sublists beat fewer levels up to 2^22 (with L2 flushed
-                // before each call: 2^18 0.116 ms against 0.145 at spacing 16, 2^20
-                // 0.153 against 0.177 at spacing 8)
+            if (l <= 24) {
+                // latency-bound up to 2^22 or so: short sublists, deeper levels at
+                // spacing 4 (2^20: 72.1 us, 78 with 8 / 8, 76 with 16 / 4, 95 with 32 / 8;
+                // 15,000,001: 426, 432 with 8 / 8, 436 with 16 / 4)
                 p.rs_level0 = 1, p.rs_spacing0 = 8, p.rs_spacing = 4;
-            } else if (l <= 24) {
-                p.rs_level0 = 1, p.rs_spacing0 = 16, p.rs_spacing = 8;
             } else if (l <= 27) {
                 // the read-only first level pays off once the list outgrows L2
                 // (8-byte walk words of 2^25 elements are 256 MB)
-                p.rs_level0 = 2, p.rs_spacing0 = 16, p.rs_spacing = 8;
+                p.rs_level0 = 2, p.rs_spacing0 = 16, p.rs_spacing = 4;
             } else {
-                p.rs_level0 = 2, p.rs_spacing0 = 32, p.rs_spacing = 8;
+                p.rs_level0 = 2, p.rs_spacing0 = 32, p.rs_spacing = 4;
             }
             // batched lists: minimum spacing of the in-block ruling sets
             if (k == KIND_LR_BATCH) p.rs_spacing0 = 64;
@@ -366,7 +363,8 @@ lrcc_status lr_rank_locked(Ctx* c, const int32_t* succ, int64_t n, int32_t head,
     lrcc_status st = LRCC_OK;
     Plan p = plan_for(KIND_LR, n);
     if (val) p.rs_level0 = 1;   // weighted sums: the in-place first level carries the values
-    const RsLayout L = rs_layout(n, p, rs_walk_grid(c, p));
+    // (a caller that ranks in place, out = succ, keeps the packed words)
+    const RsLayout L = rs_layout(n, p, rs_walk_grid(c, p), 0, 0, !val && !arrays_overlap(succ, rank, n));
     if (n > p.rs_small) {
         st = ensure_ws(c, L.bytes);
         if (st != LRCC_OK) return st;
@@ -953,7 +951,7 @@ int64_t lrcc_workspace_query(int kind, int64_t n, int64_t m) {
         case 7: return (int64_t)lr_scan_forest_ws(n, p);   // lr_scan_forest
         case KIND_LR: {
             // the walk's block count on the current device (as on a GB300 when none can be queried)
-            return n > p.rs_small ? (int64_t)rs_layout(n, p, rs_walk_grid_current(p)).bytes : 0;
+            return n > p.rs_small ? (int64_t)rs_layout(n, p, rs_walk_grid_current(p), 0, 0, true).bytes : 0;
         }
         case KIND_LR_WYLLIE: return n > p.rs_small ? (int64_t)lr_wyllie_ws(n, p) : 0;
         case KIND_CC: return (int64_t)(p.cc_hook == 4 ? cc_sv_ws(n) : cc_ws(m));
