@@ -1913,7 +1913,9 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
         cur = nb;
     }
     L.levels = lvl;
-    for (int l = 1; l < lvl; ++l) L.off_P[l] = take(sizeof(uint64_t) * (size_t)L.size[l]);
+    // level 1's records take over the successors and weights, which only the first level's walk reads
+    for (int l = 1; l < lvl; ++l)
+        L.off_P[l] = l == 1 && !direct ? L.off_snext : take(sizeof(uint64_t) * (size_t)L.size[l]);
     L.readonly = p.rs_level0 == 2 && lvl > 0 && walk_grid > 0;
     L.split = p.rs_level0 == 3 && lvl > 0;
     if (L.readonly) {
