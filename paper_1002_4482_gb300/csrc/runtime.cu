@@ -357,12 +357,21 @@ int lrcc_version(void) { return 101; }
 
 namespace {
 
+// Weighted sums: the in-place first level carries the values in packed words.
+// Above 2^22 elements its splitters are at least 16 apart: as fast as 8 apart
+// (15,000,000 elements: 491 us both), in 9.7 bytes per element instead of 11.3.
+Plan scan_plan(int64_t n) {
+    Plan p = plan_for(KIND_LR, n);
+    p.rs_level0 = 1;
+    if (n > (int64_t(1) << 22)) p.rs_spacing0 = std::max(p.rs_spacing0, 16);
+    return p;
+}
+
 // lr_rank on device buffers, with the context's lock held.
 lrcc_status lr_rank_locked(Ctx* c, const int32_t* succ, int64_t n, int32_t head, int32_t* rank,
                            const int32_t* val = nullptr) {
     lrcc_status st = LRCC_OK;
-    Plan p = plan_for(KIND_LR, n);
-    if (val) p.rs_level0 = 1;   // weighted sums: the in-place first level carries the values
+    const Plan p = val ? scan_plan(n) : plan_for(KIND_LR, n);
     // (a caller that ranks in place, out = succ, keeps the packed words)
     const RsLayout L = rs_layout(n, p, rs_walk_grid(c, p), 0, 0, !val && !arrays_overlap(succ, rank, n));
     if (n > p.rs_small) {
@@ -944,8 +953,7 @@ int64_t lrcc_workspace_query(int kind, int64_t n, int64_t m) {
     const Plan p = kind == KIND_CC ? plan_for(cc_plan_kind(m, n), n) : plan_for(kind > 5 ? KIND_LR : kind, n);
     switch (kind) {
         case 6: {   // lr_scan: the in-place first level
-            Plan ps = p;
-            ps.rs_level0 = 1;
+            const Plan ps = scan_plan(n);
             return n > ps.rs_small ? (int64_t)rs_layout(n, ps, rs_walk_grid_current(ps)).bytes : 0;
         }
         case 7: return (int64_t)lr_scan_forest_ws(n, p);   // lr_scan_forest
