@@ -167,7 +167,8 @@ lrcc_status lr_scan_forest(const int32_t* succ, const int32_t* val, int64_t n, i
  * endpoints have different roots, atomicMin links the larger root below the
  * smaller) and shortcutting (pointer jumping until every tree is a star),
  * until a hook pass finds no edge joining two roots. The round count is
- * capped; reaching the cap records LRCC_ERR_NOT_CONVERGED.
+ * capped; reaching the cap records LRCC_ERR_NOT_CONVERGED. Workspace: about 3
+ * bytes per edge (2 above 2^26 edges).
  */
 lrcc_status cc_label(const int32_t* src, const int32_t* dst, int64_t m, int64_t n,
                      int32_t* label, void* stream);
@@ -309,7 +310,9 @@ typedef struct lrcc_plan {
     int32_t rs_spacing;      /* mean sublist length at deeper levels */
     int32_t rs_small;        /* lists of at most this many elements are ranked by one block */
     int32_t rs_chains;       /* sublist walks interleaved per thread: 1, 2 or 4 */
-    int32_t cc_hook;         /* 1 = one atomicMin per edge and pass, 2 = re-link until joined,
+    int32_t cc_hook;         /* 1 = one atomicMin per edge and pass (all passes in one launch, or
+                                one block, unless cc_max_rounds or use_graphs = 2 asks for a
+                                launch per pass), 2 = re-link until joined,
                                 3 = rule 1 in the first pass, rule 2 after, 4 = the
                                 Shiloach-Vishkin rounds themselves (shortcut, mark, conditional
                                 and stagnant-tree hooking, shortcut, check; Sec. 4 SV0-SV5),
@@ -333,8 +336,9 @@ typedef struct lrcc_plan {
     int32_t cc_sample;       /* components: before the first pass over all edges, one hook pass
                                 and shortcut over the first m / cc_sample edges (a sample that
                                 forms most of the large components cheaply); 1 = no sample pass,
-                                -1 = automatic (about one sampled edge per vertex on graphs with
-                                at least 8 edges per vertex, two with 4 to 7, no sample below) */
+                                -1 = automatic (hook rule 1: about one sampled edge per vertex
+                                from 2 edges per vertex up; the other rules: one from 8 edges
+                                per vertex up, two with 4 to 7, no sample below) */
 } lrcc_plan;
 
 /* kind: 1 = list ranking, 2 = its Wyllie form, 3 = connected components of

@@ -25,7 +25,9 @@
 // edge links its endpoints with atomicMin and carries every link the atomic
 // displaces on to the next pair (link_direct), so that pass joins every edge
 // it reads, and rule 1 after it. All give the same labels. Rule 4, the
-// paper's own round structure, is in cc_sv.cu.
+// paper's own round structure, is in cc_sv.cu. Rule 1 runs here only when the
+// plan asks for plain launches or caps the passes; otherwise cc_gang.cu takes
+// it, with all rounds in one launch.
 //
 // Before the loop, an optional sample pass (plan.cc_sample) hooks and
 // shortcuts a prefix of the edge list, which forms most of a large component

@@ -184,6 +184,12 @@ int64_t cc_active_cap(int64_t m);
 lrcc_status cc_gather_probe_run(Ctx* c, const int32_t* src, const int32_t* dst, int64_t m, const int32_t* table,
                                 int64_t n, int64_t* out);
 size_t cc_ws(int64_t m);
+// Rule 1 in one launch (cc_gang.cu): whether the plan takes it, its workspace, the run.
+bool cc_gang_applies(const Plan& p);
+bool cc_one_block_applies(int64_t m, int64_t n);
+size_t cc_gang_ws(int64_t m, int64_t n, int sms);
+lrcc_status cc_run_gang(Ctx* c, const int32_t* src, const int32_t* dst, int64_t m, int64_t n, int32_t* label,
+                        const Plan& p);
 // The Shiloach-Vishkin round structure (plan.cc_hook = 4): workspace, run, round bound.
 size_t cc_sv_ws(int64_t n);
 lrcc_status cc_run_sv(Ctx* c, const int32_t* src, const int32_t* dst, int64_t m, int64_t n, int32_t* label,

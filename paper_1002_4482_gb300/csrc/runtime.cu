@@ -396,10 +396,13 @@ lrcc_status lr_rank_locked(Ctx* c, const int32_t* succ, int64_t n, int32_t head,
 lrcc_status cc_label_locked(Ctx* c, const int32_t* src, const int32_t* dst, int64_t m, int64_t n, int32_t* label) {
     const Plan p = plan_for(cc_plan_kind(m, n), n);
     const bool sv = p.cc_hook == 4;
-    lrcc_status st = ensure_ws(c, sv ? cc_sv_ws(n) : cc_ws(m));
+    const bool gang = cc_gang_applies(p);
+    lrcc_status st = ensure_ws(c, sv ? cc_sv_ws(n) : gang ? cc_gang_ws(m, n, c->sms) : cc_ws(m));
     if (st != LRCC_OK) return st;
     reset_ctl(c, c->stream);
-    st = sv ? cc_run_sv(c, src, dst, m, n, label, p) : cc_run(c, src, dst, m, n, label, p);
+    st = sv     ? cc_run_sv(c, src, dst, m, n, label, p)
+         : gang ? cc_run_gang(c, src, dst, m, n, label, p)
+                : cc_run(c, src, dst, m, n, label, p);
     c->last_kind = KIND_CC;
     return st;
 }
@@ -849,6 +852,17 @@ void release_device_stream(int dev, void* stream) {
     delete c;
 }
 
+// SMs of the current device (a GB300's when none can be queried).
+int sms_current() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
+        cudaGetLastError();
+        return 152;
+    }
+    return sms;
+}
+
 int64_t ctx_bytes(const Ctx* c) { return (int64_t)(c->ws_bytes + c->io_bytes) + (int64_t)sizeof(DevCtl); }
 
 }  // namespace lrcc
@@ -962,7 +976,8 @@ int64_t lrcc_workspace_query(int kind, int64_t n, int64_t m) {
             return n > p.rs_small ? (int64_t)rs_layout(n, p, rs_walk_grid_current(p), 0, 0, true).bytes : 0;
         }
         case KIND_LR_WYLLIE: return n > p.rs_small ? (int64_t)lr_wyllie_ws(n, p) : 0;
-        case KIND_CC: return (int64_t)(p.cc_hook == 4 ? cc_sv_ws(n) : cc_ws(m));
+        case KIND_CC:
+            return (int64_t)(p.cc_hook == 4 ? cc_sv_ws(n) : cc_gang_applies(p) ? cc_gang_ws(m, n, sms_current()) : cc_ws(m));
         case KIND_LR_BATCH: {   // n = total elements, m = lists
             const Plan pb = plan_for(KIND_LR_BATCH, n);
             if (!batch_union_applies(n, pb)) return (int64_t)lr_batched_ws(n, m);
