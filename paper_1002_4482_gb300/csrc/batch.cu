@@ -22,6 +22,8 @@
 // disjoint union in global ids (voff[k] + local id), by grid-wide hook and
 // shortcut kernels looped on the device; components never cross instances,
 // so the union's min-id labels minus voff[k] are each instance's labels.
+// (Graphs under hook rule 1 are labelled by cc_batch.cu instead; this file's
+// graph kernels serve the other rules, plain launches and capped passes.)
 #include <algorithm>
 
 #include "block_rank.cuh"

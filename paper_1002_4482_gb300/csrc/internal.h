@@ -201,6 +201,11 @@ lrcc_status lr_batched_run(Ctx* c, const int32_t* succ, const int64_t* off, cons
                            int64_t count, int32_t* rank, int64_t total_nodes, const Plan& p);
 lrcc_status cc_batched_run(Ctx* c, const int32_t* src, const int32_t* dst, const int64_t* eoff,
                            const int64_t* voff, int64_t count, int64_t total_edges, int32_t* label, const Plan& p);
+// Rule 1 (cc_batch.cu): whether the plan takes it, its workspace, the run.
+bool cc_batch_gang_applies(const Plan& p);
+size_t cc_batch_gang_ws(int64_t count, int64_t total_edges, int sms);
+lrcc_status cc_batch_gang_run(Ctx* c, const int32_t* src, const int32_t* dst, const int64_t* eoff, const int64_t* voff,
+                              int64_t count, int64_t total_edges, int32_t* label);
 size_t lr_batched_ws(int64_t total_nodes, int64_t count);
 // Batched lists of at least 2^22 elements in all whose batched plan (looked up
 // by the total) has the read-only first level are ranked together as one list.

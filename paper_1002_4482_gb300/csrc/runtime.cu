@@ -631,10 +631,12 @@ lrcc_status cc_label_batched_sized(const int32_t* src, const int32_t* dst, const
     if (st != LRCC_OK) return st;
     std::lock_guard<std::mutex> lk(c->mu);
     const Plan p = plan_for(KIND_CC_BATCH, 0);
-    st = ensure_ws(c, cc_batched_ws(num_graphs, total_edges));
+    const bool gang = cc_batch_gang_applies(p);
+    st = ensure_ws(c, gang ? cc_batch_gang_ws(num_graphs, total_edges, c->sms) : cc_batched_ws(num_graphs, total_edges));
     if (st != LRCC_OK) return st;
     reset_ctl(c, c->stream);
-    st = cc_batched_run(c, src, dst, edge_off, vert_off, num_graphs, total_edges, label, p);
+    st = gang ? cc_batch_gang_run(c, src, dst, edge_off, vert_off, num_graphs, total_edges, label)
+              : cc_batched_run(c, src, dst, edge_off, vert_off, num_graphs, total_edges, label, p);
     c->last_kind = KIND_CC_BATCH;
     return st;
 }
@@ -987,7 +989,8 @@ int64_t lrcc_workspace_query(int kind, int64_t n, int64_t m) {
             // global successors, two int32 per list
             return (int64_t)(rs_layout(n, pu, rs_walk_grid_current(pu), m).bytes + 4 * (size_t)n + 8 * (size_t)m + 1024);
         }
-        case KIND_CC_BATCH: return (int64_t)cc_batched_ws(m, n);   // n = total edges, m = graphs
+        case KIND_CC_BATCH:   // n = total edges, m = graphs
+            return (int64_t)(cc_batch_gang_applies(p) ? cc_batch_gang_ws(m, n, sms_current()) : cc_batched_ws(m, n));
         default: return -1;
     }
 }
