@@ -197,7 +197,9 @@ lrcc_status cc_label_host(const int32_t* src, const int32_t* dst, int64_t m, int
 /*
  * Batched list ranking: num_lists independent lists in one launch (a
  * persistent kernel takes the lists from a device work queue, largest first;
- * each list is ranked by one thread block).
+ * each list is ranked by one thread block), or, when the lists are long on
+ * average (2^12 elements) or many (2^25 in all) and the batched plan's rs_level0
+ * is 2, by the whole GPU as one list.
  * List k owns elements [node_off[k], node_off[k+1]) of succ and rank;
  * succ values and heads[k] are LOCAL ids (0-based within list k), and the
  * ranks are local too. node_off is int64[num_lists + 1] on the device,
@@ -216,8 +218,8 @@ lrcc_status lr_rank_batched_sized(const int32_t* succ, const int64_t* node_off, 
                                   int64_t num_lists, int64_t total_nodes, int32_t* rank, void* stream);
 
 /*
- * Batched connected components: num_graphs independent graphs in one launch
- * (a persistent kernel, one thread block per graph, largest first).
+ * Batched connected components: num_graphs independent graphs (largest first;
+ * a gang of blocks takes each large graph, one block each small one).
  * Graph k owns edges [edge_off[k], edge_off[k+1]) of src/dst and vertices
  * [vert_off[k], vert_off[k+1]) of label; edge endpoints and labels are LOCAL
  * ids. Offsets are int64[num_graphs + 1] on the device, non-decreasing, 0 first.
@@ -324,8 +326,10 @@ typedef struct lrcc_plan {
                                 re-link until joined whatever the rule */
     int32_t cc_max_rounds;   /* cap on hook passes (-1 = back to the automatic cap) */
     int32_t use_graphs;      /* 1 = replay captured CUDA graphs, 2 = plain launches */
-    int32_t rs_level0;       /* first ruling-set level: 1 = the walk rewrites 8-byte words in
-                                place; 2 = the walk only reads succ and writes what it visits
+    int32_t rs_level0;       /* first ruling-set level: 1 = in place: up to 2^24 elements the walk
+                                keeps 4-byte records in the rank array, above that (and for
+                                weighted ranks, given splitters and rank = succ) it rewrites
+                                8-byte words in a workspace; 2 = the walk only reads succ and writes what it visits
                                 as 32-byte chunks, which are turned into ranks by a scatter
                                 into id-range buckets and a placement pass; 3 = the walk
                                 reads succ and keeps an ownership mark (16 bits below 65,535

@@ -5,8 +5,8 @@
 // processing time first). Each block of the persistent kernel then takes the
 // next instance from a device counter and solves it alone, synchronising
 // with __syncthreads only (no block ever waits on another block):
-//   lists   up to SMEM_ELEMS elements: loaded into shared memory and ranked
-//           there (block_rank.cuh);
+//   lists   up to 24,576 elements: loaded into shared memory and ranked there
+//           (block_rank.cuh);
 //           larger: a ruling set inside the block (Sec. 3.2): stratified
 //           splitters, in-place 8-byte walk words in global workspace, the
 //           splitter list held and ranked in shared memory, then the expand.
@@ -37,14 +37,19 @@ namespace {
 
 constexpr int BT = 512;                   // threads per batched block
 constexpr int SMEM_ELEMS = 8192;          // list elements / splitters held in shared memory
+constexpr int SMEM_CLASS = 13;            // the size class that ends with SMEM_ELEMS
+constexpr int BT_LARGE = 1024;            // the same for lists above SMEM_ELEMS
+constexpr int SMEM_ELEMS_LARGE = 24576;
 constexpr int CC_SMEM_VERTS = 2 * SMEM_ELEMS;
 constexpr size_t CC_SMEM_BYTES = sizeof(int) * CC_SMEM_VERTS;                                   // 64 KB
 constexpr size_t LR_SMEM_BYTES = sizeof(uint64_t) * SMEM_ELEMS + 2 * sizeof(uint2) * BT;       // 72 KB
+constexpr size_t LR_SMEM_LARGE = sizeof(uint64_t) * SMEM_ELEMS_LARGE + 2 * sizeof(uint2) * BT_LARGE;   // 208 KB
 constexpr int NCLASS = 33;
 constexpr int64_t CC_LARGE = int64_t(1) << 15;   // graphs above this many vertices go to the union path
 constexpr int SEG_BLOCK = 256;
 
-// Order instances by size class (floor(log2 size)), largest first.
+// Order instances by size class (floor(log2(size - 1))), largest first; order[count]
+// = how many have more than SMEM_ELEMS elements (they come first).
 __global__ void __launch_bounds__(1024)
     batch_order(const int64_t* __restrict__ off_a, const int64_t* __restrict__ off_b, const int32_t* heads,
                 int64_t count, int32_t* __restrict__ order, DevCtl* ctl) {
@@ -67,7 +72,7 @@ __global__ void __launch_bounds__(1024)
             record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)k);
             return 0;
         }
-        return size <= 1 ? 0 : min(63 - __clzll((unsigned long long)size), NCLASS - 1);
+        return size <= 1 ? 0 : min(64 - __clzll((unsigned long long)(size - 1)), NCLASS - 1);
     };
     for (int64_t k = threadIdx.x; k < count; k += blockDim.x) atomicAdd(&s_hist[klass(k)], 1);
     __syncthreads();
@@ -76,26 +81,28 @@ __global__ void __launch_bounds__(1024)
         for (int c = NCLASS - 1; c >= 0; --c) {
             s_start[c] = run;
             run += s_hist[c];
+            if (c == SMEM_CLASS + 1) order[count] = run;
         }
     }
     __syncthreads();
     for (int64_t k = threadIdx.x; k < count; k += blockDim.x) order[atomicAdd(&s_start[klass(k)], 1)] = (int32_t)k;
 }
 
-__device__ __forceinline__ int64_t take_instance(int* s_k, int64_t count, DevCtl* ctl) {
+__device__ __forceinline__ int64_t take_instance(int* s_k, int* next, int64_t count) {
     __syncthreads();
-    if (threadIdx.x == 0) *s_k = atomicAdd(&ctl->batch_next, 1);
+    if (threadIdx.x == 0) *s_k = atomicAdd(next, 1);
     __syncthreads();
     return *s_k < count ? *s_k : -1;
 }
 
 // ----------------------------------------------------------------- lists
 
-// Rank one list of n <= SMEM_ELEMS elements in shared memory.
+// Rank one list in shared memory.
+template <int T>
 __device__ void list_in_smem(const int32_t* succ, int n, int head, int32_t* rank, uint64_t* W, uint2* sub,
                              uint32_t seed, DevCtl* ctl) {
 #pragma unroll 4
-    for (int i = threadIdx.x; i < n; i += BT) {
+    for (int i = threadIdx.x; i < n; i += T) {
         const int s = succ[i];
         const bool tail = (s == -1) | (s == i);
         const bool bad = !tail && (s < 0 || s >= n);
@@ -103,26 +110,27 @@ __device__ void list_in_smem(const int32_t* succ, int n, int head, int32_t* rank
         W[i] = pack((tail || bad) ? BR_NIL : (uint32_t)s, 1u);
     }
     bool whole;
-    const uint2* res = block_rank<BT>(W, sub, n, head, seed, &whole, ctl);
+    const uint2* res = block_rank<T>(W, sub, n, head, seed, &whole, ctl);
     if (threadIdx.x == 0 && !whole) record_error(ctl, LRCC_ERR_INVALID_INPUT, head);
 #pragma unroll 4
-    for (int i = threadIdx.x; i < n; i += BT) rank[i] = block_rank_sum<BT>(W[i], res) - 1;
+    for (int i = threadIdx.x; i < n; i += T) rank[i] = block_rank_sum<T>(W[i], res) - 1;
 }
 
 // Rank one larger list with a ruling set inside the block; W is the list's
 // slice of the 8-byte word workspace, R the splitters' packed words in shared
 // memory (next splitter, sublist length; before the walk: successor, 1).
+template <int T, int CAP>
 __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_t* rank, uint64_t* W,
                                 uint64_t* R, uint2* sub, int* s_work, uint32_t seed, int min_logD, DevCtl* ctl) {
-    // spacing: a power of two, at least 2^min_logD, with at most SMEM_ELEMS splitters
+    // spacing: a power of two, at least 2^min_logD, with at most CAP splitters
     int logD = max(2, min_logD);
-    while (((n + (int64_t(1) << logD) - 1) >> logD) > SMEM_ELEMS) ++logD;
+    while (((n + (int64_t(1) << logD) - 1) >> logD) > CAP) ++logD;
     const int64_t D = int64_t(1) << logD;
     const int r = (int)((n + D - 1) >> logD);
     const int64_t bh = head >> logD;
     const uint32_t head_off = (uint32_t)(head - (bh << logD));
     // select (RS1+RS2): walk words, and each splitter's successor in R[j]
-    for (int64_t i = threadIdx.x; i < n; i += BT) {
+    for (int64_t i = threadIdx.x; i < n; i += T) {
         const int s = succ[i];
         const bool tail = (s == -1) | (s == i);
         const bool bad = !tail && (s < 0 || s >= n);
@@ -172,12 +180,12 @@ __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_
     }
     // rank the splitters (RS4) in shared memory; their suffix sums replace their words
     bool whole;
-    const uint2* res = block_rank<BT>(R, sub, r, 0, seed, &whole, ctl);
+    const uint2* res = block_rank<T>(R, sub, r, 0, seed, &whole, ctl);
     if (threadIdx.x == 0 && (!whole || (int64_t)res[0].y != n)) record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
-    for (int j = threadIdx.x; j < r; j += BT) R[j] = (uint64_t)(uint32_t)block_rank_sum<BT>(R[j], res);
+    for (int j = threadIdx.x; j < r; j += T) R[j] = (uint64_t)(uint32_t)block_rank_sum<T>(R[j], res);
     __syncthreads();
     // expand (RS5)
-    for (int64_t i = threadIdx.x; i < n; i += BT) {
+    for (int64_t i = threadIdx.x; i < n; i += T) {
         const uint64_t w = W[i];
         const uint32_t lo = lo32(w), hi = hi32(w);
         int out;
@@ -193,27 +201,35 @@ __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_
     }
 }
 
-__global__ void __launch_bounds__(BT)
+// Lists of at most CAP elements in shared memory, larger ones by a ruling set
+// inside the block. Two launches share the lists: those above SMEM_ELEMS
+// elements (order[0 .. *split)) with 1024 threads and room for 24,576 elements,
+// the others with 512 threads and three blocks per SM. 2000 lists of 2^8 to 2^14
+// elements: 83 us with the second size, 344 us when the lists above 8192 elements
+// were walked in global memory.
+template <int T, int CAP, bool LARGE>
+__global__ void __launch_bounds__(T)
     lr_batch_kernel(const int32_t* __restrict__ succ, const int64_t* __restrict__ off, const int32_t* __restrict__ heads,
-                    int64_t count, const int32_t* __restrict__ order, int32_t* __restrict__ rank, uint64_t* W,
-                    uint32_t seed, int min_logD, DevCtl* ctl) {
+                    int64_t count, const int32_t* __restrict__ order, const int32_t* __restrict__ split,
+                    int32_t* __restrict__ rank, uint64_t* W, uint32_t seed, int min_logD, DevCtl* ctl) {
     extern __shared__ __align__(16) unsigned char lb_raw[];
     uint64_t* words = reinterpret_cast<uint64_t*>(lb_raw);
-    uint2* sub = reinterpret_cast<uint2*>(lb_raw + sizeof(uint64_t) * SMEM_ELEMS);
+    uint2* sub = reinterpret_cast<uint2*>(lb_raw + sizeof(uint64_t) * CAP);
     __shared__ int s_k, s_work;
+    const int64_t first = LARGE ? 0 : *split, last = LARGE ? *split : count;
     for (;;) {
-        const int64_t q = take_instance(&s_k, count, ctl);
+        const int64_t q = take_instance(&s_k, LARGE ? &ctl->batch_next : &ctl->seg_next, last - first);
         if (q < 0) break;
-        const int64_t k = order[q];
+        const int64_t k = order[first + q];
         const int64_t b = off[k], n = off[k + 1] - b;
         if (n <= 0 || n > 0x7FFFFFFELL) continue;
         const int head = heads[k];
         if (head < 0 || head >= n) continue;
-        if (n <= SMEM_ELEMS)
-            list_in_smem(succ + b, (int)n, head, rank + b, words, sub, seed ^ (uint32_t)k, ctl);
+        if (n <= CAP)
+            list_in_smem<T>(succ + b, (int)n, head, rank + b, words, sub, seed ^ (uint32_t)k, ctl);
         else
-            list_ruling_set(succ + b, n, head, rank + b, W + b, words, sub, &s_work, seed ^ (uint32_t)k, min_logD,
-                            ctl);
+            list_ruling_set<T, CAP>(succ + b, n, head, rank + b, W + b, words, sub, &s_work, seed ^ (uint32_t)k,
+                                    min_logD, ctl);
     }
 }
 
@@ -322,7 +338,7 @@ __global__ void __launch_bounds__(BT)
     extern __shared__ int sm[];
     __shared__ int s_k;
     for (;;) {
-        const int64_t q = take_instance(&s_k, count, ctl);
+        const int64_t q = take_instance(&s_k, &ctl->batch_next, count);
         if (q < 0) break;
         const int64_t k = order[q];
         const int64_t eb = eoff[k], m = eoff[k + 1] - eb;
@@ -704,7 +720,7 @@ lrcc_status set_smem(const void* k, size_t bytes) {
 
 size_t lr_batched_ws(int64_t total_nodes, int64_t count) {
     return align_up(sizeof(uint64_t) * (size_t)std::max<int64_t>(total_nodes, 1), 256) +
-           align_up(sizeof(int32_t) * (size_t)std::max<int64_t>(count, 1), 256);
+           align_up(sizeof(int32_t) * (size_t)(std::max<int64_t>(count, 1) + 1), 256);
 }
 
 // Active-edge buffers of the union path: a quarter of all edges each. On the
@@ -718,7 +734,7 @@ int64_t cc_batched_active_cap(int64_t total_edges) {
 size_t cc_batched_ws(int64_t count, int64_t total_edges) {
     const size_t c = (size_t)std::max<int64_t>(count, 1);
     const int64_t acap = cc_batched_active_cap(total_edges);
-    return 2 * align_up(sizeof(int32_t) * c, 256) + 2 * align_up(sizeof(int64_t) * (c + 1), 256) + 256 +
+    return 2 * align_up(sizeof(int32_t) * (c + 1), 256) + 2 * align_up(sizeof(int64_t) * (c + 1), 256) + 256 +
            (acap > 0 ? 2 * align_up(sizeof(int2) * (size_t)acap, 256) : 0);
 }
 
@@ -731,14 +747,23 @@ lrcc_status lr_batched_run(Ctx* c, const int32_t* succ, const int64_t* off, cons
     phase_begin(c, s);
     batch_order<<<1, 1024, 0, s>>>(off, nullptr, heads, count, order, c->ctl);
     phase_end(c, s, PH_BATCH_PREP);
-    lrcc_status st = set_smem((const void*)lr_batch_kernel, LR_SMEM_BYTES);
+    auto small_k = lr_batch_kernel<BT, SMEM_ELEMS, false>;
+    auto large_k = lr_batch_kernel<BT_LARGE, SMEM_ELEMS_LARGE, true>;
+    lrcc_status st = set_smem((const void*)small_k, LR_SMEM_BYTES);
+    if (st == LRCC_OK) st = set_smem((const void*)large_k, LR_SMEM_LARGE);
     if (st != LRCC_OK) return st;
-    const int g = (int)std::min<int64_t>(count, persistent_grid(c, (const void*)lr_batch_kernel, BT, LR_SMEM_BYTES));
-    phase_begin(c, s);
     int min_logD = 2;
     while (min_logD < 20 && (1 << (min_logD + 1)) <= p.rs_spacing0) ++min_logD;
-    lr_batch_kernel<<<g, BT, LR_SMEM_BYTES, s>>>(succ, off, heads, count, order, rank, W,
-                                              (uint32_t)(p.seed ^ (p.seed >> 32)), min_logD, c->ctl);
+    const uint32_t seed = (uint32_t)(p.seed ^ (p.seed >> 32));
+    phase_begin(c, s);
+    if (total_nodes > SMEM_ELEMS) {
+        const int64_t most = std::min<int64_t>(count, total_nodes / SMEM_ELEMS);   // lists above SMEM_ELEMS at most
+        const int g = (int)std::min<int64_t>(most, persistent_grid(c, (const void*)large_k, BT_LARGE, LR_SMEM_LARGE));
+        large_k<<<g, BT_LARGE, LR_SMEM_LARGE, s>>>(succ, off, heads, count, order, order + count, rank, W, seed, min_logD,
+                                                   c->ctl);
+    }
+    const int g = (int)std::min<int64_t>(count, persistent_grid(c, (const void*)small_k, BT, LR_SMEM_BYTES));
+    small_k<<<g, BT, LR_SMEM_BYTES, s>>>(succ, off, heads, count, order, order + count, rank, W, seed, min_logD, c->ctl);
     phase_end(c, s, PH_LR_BATCH);
     return cuda_status(cudaGetLastError());
 }
@@ -749,7 +774,7 @@ lrcc_status cc_batched_run(Ctx* c, const int32_t* src, const int32_t* dst, const
     const size_t cnt = (size_t)std::max<int64_t>(count, 1);
     char* w = static_cast<char*>(c->ws);
     int32_t* order = reinterpret_cast<int32_t*>(w);
-    w += align_up(sizeof(int32_t) * cnt, 256);
+    w += align_up(sizeof(int32_t) * (cnt + 1), 256);
     LargeSet L;
     L.ids = reinterpret_cast<int32_t*>(w);
     w += align_up(sizeof(int32_t) * cnt, 256);

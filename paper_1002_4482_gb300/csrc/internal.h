@@ -207,12 +207,13 @@ size_t cc_batch_gang_ws(int64_t count, int64_t total_edges, int sms);
 lrcc_status cc_batch_gang_run(Ctx* c, const int32_t* src, const int32_t* dst, const int64_t* eoff, const int64_t* voff,
                               int64_t count, int64_t total_edges, int32_t* label);
 size_t lr_batched_ws(int64_t total_nodes, int64_t count);
-// Batched lists of at least 2^22 elements in all whose batched plan (looked up
-// by the total) has the read-only first level are ranked together as one list.
-bool batch_union_applies(int64_t total, const Plan& batch_plan);
-size_t lr_batched_union_ws(Ctx* c, int64_t total, int64_t K);
+// How batched lists are ranked: one block per list, all of them together as one
+// list with records in the rank array, or together by the read-only first level.
+enum BatchMode { BATCH_BLOCKS, BATCH_DIRECT, BATCH_READONLY };
+BatchMode lr_batch_mode(int64_t total, int64_t K, const Plan& batch_plan, bool overlap);
+size_t lr_batched_union_ws(int walk_grid, int64_t total, int64_t K, BatchMode mode);
 lrcc_status lr_batched_union(Ctx* c, cudaStream_t s, const int32_t* succ, const int64_t* off, const int32_t* heads,
-                             int64_t K, int64_t total, int32_t* rank);
+                             int64_t K, int64_t total, int32_t* rank, BatchMode mode);
 size_t cc_batched_ws(int64_t count, int64_t total_edges);
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

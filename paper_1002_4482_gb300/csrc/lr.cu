@@ -1515,7 +1515,8 @@ __global__ void __launch_bounds__(BLOCK)
     }
 }
 
-// One block: the first list's head, and the head splitter of every list.
+// One block: the first list's head (head_dev[0]) and the head splitter of every
+// list; head_dev[1] = the heads that became extra splitters.
 __global__ void __launch_bounds__(1024)
     bl_heads(const int64_t* __restrict__ off, const int32_t* __restrict__ heads, int64_t K, int64_t n, int logD,
              int64_t nb, uint32_t seed, int32_t* __restrict__ head_spl, int32_t* __restrict__ extra_elem,
@@ -1596,7 +1597,10 @@ __global__ void __launch_bounds__(1024)
             ++e;
         }
     }
-    if (t == 0) ctl->ff_extra = total;
+    if (t == 0) {
+        ctl->ff_extra = total;
+        head_dev[1] = total;
+    }
 }
 
 // After the first-level walk: the splitter that ends list k (its word names no
@@ -1642,6 +1646,102 @@ __global__ void __launch_bounds__(BLOCK)
         if (e < 0 || e >= n) continue;
         const int64_t k = find_list(off, K, e);
         S1[j] = (int32_t)((uint32_t)S1[j] - (uint32_t)(n - off[k + 1]));
+    }
+}
+
+// The lists ranked together with their records in the rank array (as
+// rs_walk_direct does for one list), for lists that L2 holds one after another:
+// walkers take the splitters in id order, so those in flight stay in a few
+// lists whose successors and records are in L2. The walk reads the local ids
+// itself, and the splitter that ends a list is linked to the next list's head
+// on the spot. 2048 lists of 2^8 to 2^20 elements: 3.58 ms, against 5.87 through
+// global successors, chunks, scatter and placement; the walk (2.6 ms, 96 G
+// steps/s) is bound by its two L2 requests per element, the expansion (0.8 ms) by
+// one gather each.
+constexpr int LISTS_BLOCK = 128;   // short blocks: one lasts as long as its longest sublist
+__global__ void __launch_bounds__(LISTS_BLOCK)
+    rs_walk_lists(const int32_t* __restrict__ succ, uint32_t* __restrict__ rec, Level0 L0,
+                  const int64_t* __restrict__ off, int64_t K, const int32_t* __restrict__ head_spl, int pbits,
+                  int extras, uint64_t* __restrict__ R1, DevCtl* ctl) {
+    const int64_t gh = L0.head_dev[0];
+    L0.bh = gh >> L0.logD;
+    L0.head_off = (uint32_t)(gh - (L0.bh << L0.logD));
+    const Geo32 g = geo32(L0);
+    uint32_t j = blockIdx.x * LISTS_BLOCK + threadIdx.x;
+    if (j >= g.nb + (uint32_t)L0.head_dev[1]) return;
+    uint32_t cur = splitter_node32(j, g, L0.extra), pos = 0;
+    int64_t k = find_list(off, K, cur);
+    const uint32_t base = (uint32_t)off[k], len = (uint32_t)(off[k + 1] - off[k]);
+    int32_t x = __ldg(succ + cur);
+    CycleGuard guard(cur);
+    uint32_t next = NIL;
+    for (;;) {
+        // cur (a global id) belongs to owner j at position pos, x is its local successor
+        rec[cur] = (j << pbits) | pos;
+        ++pos;
+        if (x == -1 || (uint32_t)x == cur - base) {
+            // the end of list k: on to the next list's head
+            for (++k; k < K && off[k + 1] == off[k];) ++k;
+            if (k < K) next = (uint32_t)head_spl[k];
+            break;
+        }
+        if ((uint32_t)x >= len || guard.seen(base + (uint32_t)x)) {
+            record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)cur);
+            break;
+        }
+        cur = base + (uint32_t)x;
+        x = __ldg(succ + cur);   // on its way while cur is tested
+        const int sj = splitter_index32(cur, g);
+        if (sj >= 0) {
+            next = (uint32_t)sj;
+            break;
+        }
+        if (pos >> pbits) {
+            const int e = atomicAdd(&ctl->ff_extra, 1);
+            if (e >= extras) {
+                record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)cur);
+                break;
+            }
+            R1[j] = pack(g.nb + (uint32_t)e, pos);
+            j = g.nb + (uint32_t)e;
+            pos = 0;
+        }
+    }
+    R1[j] = pack(next, pos);
+}
+
+// Records -> local ranks: the rank along all lists less the elements of the
+// later ones. A block takes one stretch of the elements and every thread keeps
+// the list it is in.
+template <bool VEC>
+__global__ void __launch_bounds__(BLOCK)
+    rs_expand_lists(int32_t* rank, int64_t n, const int32_t* __restrict__ S1, uint32_t r1, int pbits,
+                    const int64_t* __restrict__ off, int64_t K) {
+    const uint32_t mask = (1u << pbits) - 1;
+    const int64_t per = ((n + gridDim.x - 1) / gridDim.x + 4 * BLOCK - 1) / (4 * BLOCK) * (4 * BLOCK);
+    const int64_t b = per * blockIdx.x, e = min(n, b + per);
+    if (b >= e) return;
+    int64_t k = find_list(off, K, min(b + (int64_t)threadIdx.x * 4, n - 1));
+    int64_t end = off[k + 1];
+    auto rank_of = [&](int64_t i, int32_t v) {
+        while (i >= end) end = off[++k + 1];
+        const uint32_t o = (uint32_t)v >> pbits;
+        return o < r1 ? (int32_t)((uint32_t)S1[o] - 1u - ((uint32_t)v & mask) - (uint32_t)(n - end)) : -1;
+    };
+    for (int64_t i = b + threadIdx.x * 4; i < e; i += 4 * BLOCK) {
+        if (VEC && i + 3 < e) {
+            int4* p = reinterpret_cast<int4*>(rank + i);
+            const int4 v = __ldcs(p);
+            int4 r;
+            r.x = rank_of(i, v.x);
+            r.y = rank_of(i + 1, v.y);
+            r.z = rank_of(i + 2, v.z);
+            r.w = rank_of(i + 3, v.w);
+            __stcs(p, r);
+        } else {
+            for (int q = 0; q < 4; ++q)
+                if (i + q < e) rank[i + q] = rank_of(i + q, rank[i + q]);
+        }
     }
 }
 
@@ -1870,7 +1970,8 @@ int rs_walk_grid_current(const Plan& p) {
 RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int64_t given1, bool direct) {
     RsLayout L;
     L.size[0] = n;
-    direct = direct && p.rs_level0 == 1 && n > p.rs_small && n <= DIRECT_MAX;
+    // (batched lists, extra1 > 0, stay in L2 one after another at any total)
+    direct = direct && p.rs_level0 == 1 && n > p.rs_small && (extra1 > 0 || n <= DIRECT_MAX);
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
@@ -1894,10 +1995,11 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
         if (lvl == 0 && given1 > 0) nb = given1;   // first-level splitters chosen by the caller
         if (lvl == 0 && direct) {
             // as many position bits as the owners leave, extra owners included
+            const int64_t heads = nb;   // with the heads of batched lists
             L.direct = true;
-            L.fixed = nb;
+            L.fixed = nb - extra1;
             for (L.pbits = 31; L.pbits > 0; --L.pbits) {
-                nb = L.fixed + (n >> L.pbits);
+                nb = heads + (n >> L.pbits);
                 if (nb <= (int64_t(1) << (32 - L.pbits))) break;
             }
         }
@@ -1946,11 +2048,27 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
     return L;
 }
 
-// Batched lists as one list: the plan, the layout and the workspace.
-constexpr int64_t BATCH_UNION_MIN = int64_t(1) << 22;
+// Batched lists ranked together as one list: whether, the plan, the layout and
+// the workspace. One block ranks a list of up to 24,576 elements in some 30 us
+// and needs 270 us and more for a longer one, where the whole GPU takes 60 to 100
+// for all of them; the host only knows the total and the count, so the mean
+// decides: lists of 2^12 elements on average go together (16 lists of up to 2^17:
+// 62 us, 269 by blocks; 64 of up to 2^20: 166 against 2618), of 2^13 when they
+// total less than 2^17, shorter ones by blocks (2000 of up to 2^14: 83 us), and a
+// large total is not left to single blocks. Lists of 2^22 elements and less on
+// average keep their records in the rank array, longer ones outgrow L2 and take
+// the read-only first level (chunks, scatter, placement) when they total 2^25.
+constexpr int64_t UNION_MIN = int64_t(1) << 15;
+constexpr int64_t UNION_DIRECT_MEAN = int64_t(1) << 22;
+constexpr int64_t UNION_READONLY_MIN = int64_t(1) << 25;
+constexpr int64_t UNION_MAX = int64_t(0x7FFFFFFE);   // global ids are int32
 
-bool batch_union_applies(int64_t total, const Plan& batch_plan) {
-    return total >= BATCH_UNION_MIN && batch_plan.rs_level0 == 2;
+BatchMode lr_batch_mode(int64_t total, int64_t K, const Plan& batch_plan, bool overlap) {
+    if (batch_plan.rs_level0 != 2 || total < UNION_MIN || total > UNION_MAX - K) return BATCH_BLOCKS;
+    const int64_t min_mean = int64_t(1) << (total < (int64_t(1) << 17) ? 13 : 12);
+    if (total <= UNION_DIRECT_MEAN * K && !overlap)
+        return total >= min_mean * K || total >= UNION_READONLY_MIN ? BATCH_DIRECT : BATCH_BLOCKS;
+    return total >= UNION_READONLY_MIN ? BATCH_READONLY : BATCH_BLOCKS;
 }
 
 struct UnionPlan {
@@ -1959,14 +2077,16 @@ struct UnionPlan {
     size_t off_gsucc, off_head_spl, off_extra, off_head_dev, bytes;
 };
 
-UnionPlan union_plan(Ctx* c, int64_t total, int64_t K) {
+UnionPlan union_plan(int walk_grid, int64_t total, int64_t K, BatchMode mode) {
     UnionPlan U;
+    const bool direct = mode == BATCH_DIRECT;
     U.p = plan_for(KIND_LR, total);
-    U.p.rs_level0 = 2;
-    U.L = rs_layout(total, U.p, rs_walk_grid(c, U.p), K);
+    U.p.rs_level0 = direct ? 1 : 2;
+    U.p.rs_small = std::min(U.p.rs_small, 16384);
+    U.L = rs_layout(total, U.p, walk_grid, K, 0, direct);
     size_t off = align_up(U.L.bytes, 256);
     U.off_gsucc = off;
-    off = align_up(off + sizeof(int32_t) * (size_t)total, 256);
+    if (!direct) off = align_up(off + sizeof(int32_t) * (size_t)total, 256);
     U.off_head_spl = off;
     off = align_up(off + sizeof(int32_t) * (size_t)K, 256);
     U.off_extra = off;
@@ -1976,12 +2096,14 @@ UnionPlan union_plan(Ctx* c, int64_t total, int64_t K) {
     return U;
 }
 
-size_t lr_batched_union_ws(Ctx* c, int64_t total, int64_t K) { return union_plan(c, total, K).bytes; }
+size_t lr_batched_union_ws(int walk_grid, int64_t total, int64_t K, BatchMode mode) {
+    return union_plan(walk_grid, total, K, mode).bytes;
+}
 
 lrcc_status lr_batched_union(Ctx* c, cudaStream_t s, const int32_t* succ, const int64_t* off, const int32_t* heads,
-                             int64_t K, int64_t total, int32_t* rank) {
-    const UnionPlan P = union_plan(c, total, K);
-    if (!P.L.readonly || P.L.levels == 0 || c->ws_bytes < P.bytes) return LRCC_ERR_ARG;
+                             int64_t K, int64_t total, int32_t* rank, BatchMode mode) {
+    const UnionPlan P = union_plan(rs_walk_grid(c, plan_for(KIND_LR, total)), total, K, mode);
+    if (!(P.L.readonly || P.L.direct) || P.L.levels == 0 || c->ws_bytes < P.bytes) return LRCC_ERR_ARG;
     char* base = static_cast<char*>(c->ws);
     BatchUnion U;
     U.off = off;
@@ -2003,8 +2125,8 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
                           const BatchUnion* U, const int32_t* given, int64_t given_r) {
     // caller-chosen first-level splitters need the in-place first level
     if (given && (L.readonly || L.split || L.direct || U)) return LRCC_ERR_ARG;
-    // batched lists ranked as one list need the read-only first level
-    if (U && (!L.readonly || val)) return LRCC_ERR_ARG;
+    // batched lists ranked as one list need the read-only first level or records in the rank array
+    if (U && (!(L.readonly || L.direct) || val)) return LRCC_ERR_ARG;
     // weighted sums use the in-place first level (the others count positions)
     if (val && (L.readonly || L.split || L.direct)) return LRCC_ERR_ARG;
     if (val) {
@@ -2053,11 +2175,11 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     if (U) {
         const int g = stream_grid(c, (n + BL_TILE - 1) / BL_TILE * BLOCK, (const void*)bl_gsucc);
         phase_begin(c, s);
-        bl_gsucc<<<g, BLOCK, 0, s>>>(succ, U->off, U->K, n, U->gsucc, ctl);
+        if (L.readonly) bl_gsucc<<<g, BLOCK, 0, s>>>(succ, U->off, U->K, n, U->gsucc, ctl);
         bl_heads<<<1, 1024, 0, s>>>(U->off, U->heads, U->K, n, L0.logD, L0.nb, seed0, U->head_spl, U->extra_elem,
                                     U->head_dev, ctl);
         phase_end(c, s, PH_BATCH_PREP);
-        succ = U->gsucc;
+        if (L.readonly) succ = U->gsucc;
         L0.head_dev = U->head_dev;
         L0.extra = U->extra_elem;
         L0.extra_count = &ctl->ff_extra;
@@ -2148,6 +2270,12 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
             else walk0s(uint32_t(), std::integral_constant<int, 1>());
         }
         phase_end(c, s, PH_WALK0);
+    } else if (L.direct && U) {
+        phase_begin(c, s);
+        rs_walk_lists<<<(unsigned)((L0.nb + U->K + LISTS_BLOCK - 1) / LISTS_BLOCK), LISTS_BLOCK, 0, s>>>(
+            succ, reinterpret_cast<uint32_t*>(rank), L0, U->off, U->K, U->head_spl, L.pbits, (int)(L.size[1] - L.fixed),
+            R(1), ctl);
+        phase_end(c, s, PH_WALK0);
     } else if (L.direct) {
         phase_begin(c, s);
         rs_walk_direct<<<(unsigned)((L0.nb + BLOCK - 1) / BLOCK), BLOCK, 0, s>>>(
@@ -2180,7 +2308,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         rs_expand<<<g, BLOCK, 0, s>>>(P(l), (uint32_t)L.size[l], S(l + 1), (uint32_t)L.size[l + 1], S(l), ctl);
         phase_end(c, s, PH_EXPAND);
     }
-    if (U) {
+    if (U && L.readonly) {
         phase_begin(c, s);
         bl_adjust<<<stream_grid(c, L.size[1], (const void*)bl_adjust), BLOCK, 0, s>>>(S(1), U->off, U->K, n, L0);
         phase_end(c, s, PH_BATCH_PREP);
@@ -2203,6 +2331,14 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
             const int g = stream_grid(c, n, (const void*)rs_expand0s<uint32_t>);
             rs_expand0s<uint32_t><<<g, BLOCK, 0, s>>>((const uint32_t*)mark, lrank, n, S(1), L.size[1], rank, ctl);
         }
+        phase_end(c, s, PH_EXPAND0);
+    } else if (L.direct && U) {
+        const bool v = aligned16(rank);
+        const void* k = v ? (const void*)rs_expand_lists<true> : (const void*)rs_expand_lists<false>;
+        const int g = stream_grid(c, groups, k);
+        phase_begin(c, s);
+        if (v) rs_expand_lists<true><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off, U->K);
+        else rs_expand_lists<false><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off, U->K);
         phase_end(c, s, PH_EXPAND0);
     } else if (L.direct) {
         const bool v = aligned16(rank);

@@ -77,8 +77,12 @@ void init_plans_locked() {
             } else {
                 p.rs_level0 = 2, p.rs_spacing0 = 32, p.rs_spacing = 4;
             }
-            // batched lists: minimum spacing of the in-block ruling sets
-            if (k == KIND_LR_BATCH) p.rs_spacing0 = 64;
+            // batched lists: minimum spacing of the in-block ruling sets; from 2^15
+            // elements in all they may be ranked together (lr_batch_mode)
+            if (k == KIND_LR_BATCH) {
+                p.rs_spacing0 = 64;
+                if (l >= 15) p.rs_level0 = 2;
+            }
             // sparse graphs whose parent array outgrows L2 (uniform random graphs of
             // 4 edges per vertex, 2^26 vertices: 13.6 ms against 15.6 with rule 1 and
             // no sample): a sample pass over an eighth of the edges, then re-linking
@@ -587,12 +591,13 @@ lrcc_status lr_rank_batched_sized(const int32_t* succ, const int64_t* node_off, 
     // the batched plan is looked up by the total element count: its first-level
     // mode decides between one block per list and the lists ranked as one list
     const Plan p = plan_for(KIND_LR_BATCH, total_nodes);
-    if (batch_union_applies(total_nodes, p)) {
-        // the lists ranked together as one list by the read-only first level
-        st = ensure_ws(c, lr_batched_union_ws(c, total_nodes, num_lists));
+    const BatchMode mode = lr_batch_mode(total_nodes, num_lists, p, arrays_overlap(succ, rank, total_nodes));
+    if (mode != BATCH_BLOCKS) {
+        const int grid = rs_walk_grid(c, plan_for(KIND_LR, total_nodes));
+        st = ensure_ws(c, lr_batched_union_ws(grid, total_nodes, num_lists, mode));
         if (st != LRCC_OK) return st;
         reset_ctl(c, c->stream);
-        st = lr_batched_union(c, c->stream, succ, node_off, heads, num_lists, total_nodes, rank);
+        st = lr_batched_union(c, c->stream, succ, node_off, heads, num_lists, total_nodes, rank, mode);
     } else {
         st = ensure_ws(c, lr_batched_ws(total_nodes, num_lists));
         if (st != LRCC_OK) return st;
@@ -982,12 +987,16 @@ int64_t lrcc_workspace_query(int kind, int64_t n, int64_t m) {
             return (int64_t)(p.cc_hook == 4 ? cc_sv_ws(n) : cc_gang_applies(p) ? cc_gang_ws(m, n, sms_current()) : cc_ws(m));
         case KIND_LR_BATCH: {   // n = total elements, m = lists
             const Plan pb = plan_for(KIND_LR_BATCH, n);
-            if (!batch_union_applies(n, pb)) return (int64_t)lr_batched_ws(n, m);
-            Plan pu = plan_for(KIND_LR, n);
-            pu.rs_level0 = 2;
-            // the lists ranked as one list: the one-list layout with m extra splitters,
-            // global successors, two int32 per list
-            return (int64_t)(rs_layout(n, pu, rs_walk_grid_current(pu), m).bytes + 4 * (size_t)n + 8 * (size_t)m + 1024);
+            // the most that a call of this size takes (one with rank = succ keeps its
+            // records elsewhere)
+            size_t need = 0;
+            for (const bool overlap : {false, true}) {
+                const BatchMode mode = lr_batch_mode(n, m, pb, overlap);
+                need = std::max(need, mode == BATCH_BLOCKS
+                                          ? lr_batched_ws(n, m)
+                                          : lr_batched_union_ws(rs_walk_grid_current(plan_for(KIND_LR, n)), n, m, mode));
+            }
+            return (int64_t)need;
         }
         case KIND_CC_BATCH:   // n = total edges, m = graphs
             return (int64_t)(cc_batch_gang_applies(p) ? cc_batch_gang_ws(m, n, sms_current()) : cc_batched_ws(m, n));
