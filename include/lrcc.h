@@ -145,11 +145,10 @@ lrcc_status lr_scan(const int32_t* succ, const int32_t* val, int64_t n, int32_t 
  * given), and out[i] is the sum of val from i to the tail of i's own list,
  * modulo 2^32. The heads (elements no successor names) become extra splitters
  * of the ruling set's first level, and the much smaller forest of splitters is
- * summed by pointer jumping (Sec. 3.1). When a value is negative or the values
- * total 2^31 or more, the whole forest is summed by pointer jumping instead
- * (O(n log n) work, any values). An element named by two successors, a cycle
- * or a successor out of range records LRCC_ERR_INVALID_INPUT. Workspace: 37 to
- * 40 bytes per element (the first level is sized for every element a head).
+ * summed by pointer jumping (Sec. 3.1). Any values are accepted. An element
+ * named by two successors, a cycle or a successor out of range records
+ * LRCC_ERR_INVALID_INPUT. Workspace: 37 to 40 bytes per element (the first level
+ * is sized for every element a head).
  */
 lrcc_status lr_scan_forest(const int32_t* succ, const int32_t* val, int64_t n, int32_t* out, void* stream);
 

@@ -34,7 +34,9 @@ struct DevCtl {
     int pad[1];
     unsigned long long scan_total;   // weighted ranks: sum of the values
     unsigned long long edges_read;   // component loop: edges read by all hook passes
-    alignas(128) unsigned gang[64];  // cc_gang.cuh: the single gang's GangCtl
+    unsigned long long links, named, visited;   // weighted ranks: elements with a successor, elements
+                                                // named by one, elements the walks reached
+    alignas(128) unsigned gang[64];  // gang.cuh: the GangCtl of a launch that is one gang
 };
 
 __device__ __forceinline__ void record_error(DevCtl* c, int code, int where = -1) {

@@ -57,6 +57,8 @@ struct RsLayout {
     bool readonly = false;          // level 0 by the read-only walk (chunks, scan, scatter, place)
     bool split = false;             // level 0 over split mark / local-rank arrays
     bool direct = false;            // level 0 through 4-byte records in the rank array
+    bool values = false;            // weighted ranks with records apart from the walk words
+    size_t off_P0 = 0;              // values: those records
     int pbits = 0;                  // direct: position bits of a record
     int64_t fixed = 0;              // direct: first-level splitters before the extra owners
     int64_t grid = 0, cap = 0, ovf_cap = 0;
@@ -69,8 +71,9 @@ struct RsLayout {
 // given1: the number of first-level splitters when the caller chooses them
 // direct: whether an in-place first level may keep its records in the rank array
 // (unweighted ranks, stratified splitters, rank not overlapping succ)
+// values: weighted ranks
 RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1 = 0, int64_t given1 = 0,
-                   bool direct = false);
+                   bool direct = false, bool values = false);
 // Largest list ranked that way: succ and rank (8 bytes per element) stay in L2.
 constexpr int64_t DIRECT_MAX = int64_t(1) << 24;
 // Whether the n-element arrays succ and rank share memory.

@@ -16,11 +16,13 @@
 // the tail, itself included); the final rank is S - 1.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <type_traits>
 
 #include "block_rank.cuh"
 #include "block_wyllie.cuh"
 #include "common.cuh"
+#include "gang.cuh"
 #include "internal.h"
 
 namespace lrcc {
@@ -92,10 +94,11 @@ __global__ void __launch_bounds__(FINAL_THREADS, 1)
 // in packed words R[j] = (next index or NIL, weight) and writes the inclusive
 // suffix weights S. The head splitter (index 0) must see the whole list:
 // `expect` elements, or, for weighted sums (expect < 0), whose total says
-// nothing about the count, every one of the r splitters.
+// nothing about the count, every one of the r splitters, whose walks must have
+// reached `visited` elements (0: walks that mark what they visit).
 __global__ void __launch_bounds__(FINAL_THREADS, 1)
     rs_final_kernel(const uint64_t* __restrict__ R, int r, int fixed, int32_t* __restrict__ S, int64_t expect,
-                    uint32_t seed, DevCtl* ctl) {
+                    unsigned long long visited, uint32_t seed, DevCtl* ctl) {
     if (ctl->scan_bad) return;
     if (fixed < r) r = min(r, fixed + ctl->ff_extra);   // extra owners in use (rs_walk_direct)
     extern __shared__ __align__(16) unsigned char br_raw[];
@@ -112,7 +115,8 @@ __global__ void __launch_bounds__(FINAL_THREADS, 1)
     const uint2* res = block_rank<FINAL_THREADS>(W, sub, r, 0, seed, &whole, ctl);
     // with a total to expect, the head's total decides (it counts elements, and the
     // path from the head holds each once); splitters off the path are then empty ones
-    if (threadIdx.x == 0 && (expect >= 0 ? (int64_t)res[0].y != expect : !whole))
+    if (threadIdx.x == 0 &&
+        (expect >= 0 ? (int64_t)res[0].y != expect : !whole || (visited && ctl->visited != visited)))
         record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
 #pragma unroll 4
     for (int j = threadIdx.x; j < r; j += FINAL_THREADS) S[j] = block_rank_sum<FINAL_THREADS>(W[j], res);
@@ -303,10 +307,8 @@ __global__ void __launch_bounds__(BLOCK)
 template <int K>
 __global__ void __launch_bounds__(BLOCK)
     rs_walk(uint64_t* __restrict__ W, const int32_t* __restrict__ snext, const int32_t* __restrict__ sw,
-            uint64_t* __restrict__ Rout, int r, int* work, int64_t nlevel, DevCtl* ctl,
-            const int* r_extra = nullptr) {
+            uint64_t* __restrict__ Rout, int r, int* work, int64_t nlevel, DevCtl* ctl) {
     if (ctl->scan_bad) return;
-    if (r_extra) r += *r_extra;   // splitters added on the device (forest heads)
     constexpr int CHUNK = 64;
     const int lane = threadIdx.x & 31;
     int pool = 0, pool_end = 0;
@@ -1775,129 +1777,216 @@ __global__ void rs_scan_verdict(DevCtl* ctl) {
     }
 }
 
+// ------------------------------------------- weighted ranks, separate records
+
+// First level of weighted ranks: W[i] = (next or NIL, value) is read and
+// P[i] = (prefix sum, owner) written, one thread per splitter, the splitters
+// recognised by their hashed offset. Sums are plain 32-bit words (modulo 2^32):
+// nothing is marked in them. For one list the geometry's head is the list's; a
+// forest has the heads as extra splitters (L0.extra, after the stratified ones).
+// P is an array of its own (APART) or W itself: when both outgrow L2 a record
+// written where its word was read costs one line where two arrays cost two, while
+// inside L2 a store to a line just read costs more than one elsewhere (see
+// rs_chase). lr_scan: 10^6 elements 89 us apart against 119, 4 * 10^6 147 against
+// 184, 15 * 10^6 841 against 491. The loads matter: apart, read-only ones (50,000
+// elements: 35.5 us, 42 with plain loads); in place, past L1, where a plain load
+// leaves the line that the store then hits (a forest of 10^7 elements: walk 227 us,
+// 1676 with plain loads).
+template <bool APART>
+__global__ void __launch_bounds__(BLOCK)
+    rs_walk_values(const uint64_t* W, uint64_t* P, Level0 L0, uint64_t* __restrict__ R1, DevCtl* ctl) {
+    if (ctl->scan_bad) return;
+    auto load = [](const uint64_t* p) {
+        return APART ? (uint64_t)__ldg(reinterpret_cast<const unsigned long long*>(p)) : ld_cg_u64(p);
+    };
+    const Geo32 g = geo32(L0);
+    const uint32_t r = g.nb + (L0.extra_count ? (uint32_t)*L0.extra_count : 0u);
+    unsigned long long visited = 0;
+    for (uint32_t j = blockIdx.x * BLOCK + threadIdx.x; j < r; j += gridDim.x * BLOCK) {
+        uint32_t cur = splitter_node32(j, g, L0.extra);
+        uint64_t w = load(W + cur);
+        P[cur] = pack(0, j);
+        uint32_t pre = hi32(w), steps = 1, next = NIL;
+        CycleGuard guard(cur);
+        cur = lo32(w);
+        while (cur != NIL) {
+            if (cur >= g.n || guard.seen(cur)) {
+                record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)cur);
+                break;
+            }
+            w = load(W + cur);
+            const int sj = splitter_index32(cur, g);
+            if (sj >= 0) {
+                next = (uint32_t)sj;
+                break;
+            }
+            P[cur] = pack(pre, j);
+            pre += hi32(w);
+            ++steps;
+            cur = lo32(w);
+        }
+        R1[j] = pack(next, pre);
+        visited += steps;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) visited += __shfl_xor_sync(0xffffffffu, visited, o);
+    if ((threadIdx.x & 31) == 0 && visited) atomicAdd(&ctl->visited, visited);
+}
+
+// out = (owner's sum) - prefix. The sums are words S[o * stride + at].
+template <bool VEC>
+__global__ void __launch_bounds__(BLOCK)
+    rs_expand_values(const uint64_t* __restrict__ P, int64_t n, const uint32_t* __restrict__ S, int stride, int at,
+                     int64_t r, int32_t* __restrict__ out, DevCtl* ctl) {
+    if (ctl->scan_bad) return;
+    auto sum_of = [&](uint64_t p) {
+        const uint32_t o = hi32(p);   // an element no walk reached (reported already) may name any owner
+        return o < r ? (int32_t)(S[(int64_t)o * stride + at] - lo32(p)) : 0;
+    };
+    const int64_t ngroups = (n + 3) >> 2;
+    for (int64_t g = static_cast<int64_t>(blockIdx.x) * BLOCK + threadIdx.x; g < ngroups;
+         g += static_cast<int64_t>(gridDim.x) * BLOCK) {
+        const int64_t i0 = g * 4;
+        if (i0 + 3 < n) {
+            const ulonglong2* s = reinterpret_cast<const ulonglong2*>(P + i0);
+            const ulonglong2 a = __ldcs(s), b = __ldcs(s + 1);
+            const int4 r4 = make_int4(sum_of(a.x), sum_of(a.y), sum_of(b.x), sum_of(b.y));
+            if (VEC) {
+                __stcs(reinterpret_cast<int4*>(out + i0), r4);
+            } else {
+                out[i0] = r4.x; out[i0 + 1] = r4.y; out[i0 + 2] = r4.z; out[i0 + 3] = r4.w;
+            }
+        } else {
+            for (int64_t i = i0; i < n; ++i) out[i] = sum_of(P[i]);
+        }
+    }
+}
+
 // ------------------------------------------- weighted ranks of a forest
 
 // A forest of lists has no single head. Its weighted ranks take the ruling
 // set with every list head as an extra first-level splitter (the heads are the
 // elements no successor names, found with one bit per element in a bitmap L2
-// holds, which also catches an element named twice); the first level walks
-// as for one list, and the splitters, a much smaller forest, are summed by
-// pointer jumping (Sec. 3.1): words (next or NIL, value), rounds of (next,
-// value) <- (next[next], value + value[next]); a splitter still linked after
-// the last round lies on a cycle. When the values rule out the 31-bit fields
-// of the first level (a negative value, or a total of 2^31 or more), the
-// whole forest is summed by pointer jumping instead (fs_pack).
+// holds); the first level walks as for one list, and the splitters, a much
+// smaller forest, are summed by pointer jumping (Sec. 3.1): words (next or NIL,
+// value), rounds of (next, value) <- (next[next], value + value[next]), inside
+// one launch that stops when no link is left. What makes the input invalid:
+// an element named twice (more links than named elements), a cycle without a
+// splitter (elements no walk reached), a cycle with one (links left after the
+// last round).
 __global__ void __launch_bounds__(BLOCK)
-    ff_indeg(const int32_t* __restrict__ succ, int64_t n, uint32_t* has_pred, DevCtl* ctl) {
+    ff_links(const int32_t* __restrict__ succ, int64_t n, uint32_t* has_pred, DevCtl* ctl) {
     const uint64_t pol = policy_evict_first();
-    for (int64_t i = (int64_t)blockIdx.x * BLOCK + threadIdx.x; i < n; i += (int64_t)gridDim.x * BLOCK) {
-        const int32_t sx = ld_stream(succ + i, pol);
-        const bool tail = (sx == -1) | (sx == i);
-        if (tail) continue;
-        if (sx < 0 || sx >= n) {
-            record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)i);
-            continue;
+    const int64_t stride = (int64_t)gridDim.x * BLOCK;
+    unsigned long long links = 0;
+    for (int64_t i0 = (int64_t)blockIdx.x * BLOCK + threadIdx.x; i0 < n; i0 += 4 * stride) {
+        int32_t sx[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sx[q] = i0 + q * stride < n ? ld_stream(succ + i0 + q * stride, pol) : -1;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int64_t i = i0 + q * stride;
+            if (i >= n || sx[q] == -1 || sx[q] == i) continue;
+            if (sx[q] < 0 || sx[q] >= n) {
+                record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)i);
+                continue;
+            }
+            // no answer is waited for: elements named twice show in the count
+            atomicOr(has_pred + (sx[q] >> 5), 1u << (sx[q] & 31));
+            ++links;
         }
-        const uint32_t bit = 1u << (sx & 31);
-        if (atomicOr(has_pred + (sx >> 5), bit) & bit) record_error(ctl, LRCC_ERR_INVALID_INPUT, sx);
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) links += __shfl_xor_sync(0xffffffffu, links, o);
+    if ((threadIdx.x & 31) == 0 && links) atomicAdd(&ctl->links, links);
 }
 
-// Forest first level: the stratified splitter of every block of D ids keeps
-// its block number as index; every other head takes an index from nb on (one
-// counter atomic per warp). Walk words as in rs_select0, with the value as
-// weight.
+// Walk words, and the heads that are not stratified splitters as extra ones
+// (indices nb, nb + 1, ... in no particular order: one counter atomic per warp
+// and iteration).
 __global__ void __launch_bounds__(BLOCK)
-    ff_select0(const int32_t* __restrict__ succ, const int32_t* __restrict__ val, int64_t n,
-               const uint32_t* __restrict__ has_pred, uint64_t* __restrict__ W, int32_t* __restrict__ snext,
-               int32_t* __restrict__ sw, int logD, int64_t nb, int64_t r1_max, uint32_t seed, DevCtl* ctl) {
-    if (ctl->scan_bad) return;
+    ff_select(const int32_t* __restrict__ succ, const int32_t* __restrict__ val, int64_t n,
+              const uint32_t* __restrict__ has_pred, uint64_t* __restrict__ W, int32_t* __restrict__ extra, Level0 L0,
+              DevCtl* ctl) {
+    constexpr int U = 4;   // groups of 32 elements per warp and iteration
     const uint64_t pol = policy_evict_first();
-    const int64_t D = int64_t(1) << logD;
+    const Geo32 g = geo32(L0);
     const int lane = threadIdx.x & 31;
-    // warp-uniform trip count for the ballot
-    for (int64_t base = (int64_t)blockIdx.x * BLOCK + (threadIdx.x & ~31); base < n; base += (int64_t)gridDim.x * BLOCK) {
-        const int64_t i = base + lane;
-        const bool in = i < n;
-        int32_t sx = -1, v = 0;
-        if (in) {
-            sx = ld_stream(succ + i, pol);
-            v = ld_stream(val + i, pol);
+    unsigned long long named = 0;
+    const int64_t warp = ((int64_t)blockIdx.x * BLOCK + threadIdx.x) >> 5, warps = (int64_t)gridDim.x * (BLOCK / 32);
+    for (int64_t b = warp * 32 * U; b < n; b += warps * 32 * U) {
+        int32_t sx[U], v[U];
+        uint32_t pw[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int64_t i = b + q * 32 + lane;
+            sx[q] = i < n ? ld_stream(succ + i, pol) : -1;
+            v[q] = i < n ? ld_stream(val + i, pol) : 0;
+            pw[q] = b + q * 32 < n ? has_pred[(b >> 5) + q] : 0xFFFFFFFFu;
         }
-        const bool tail = (sx == -1) | (sx == i);
-        const uint32_t nx = (tail || sx < 0 || sx >= n) ? NIL : (uint32_t)sx;
-        const int64_t b = i >> logD;
-        const uint32_t size = in ? (uint32_t)min(D, n - (b << logD)) : 1u;
-        const bool strat = in && (uint32_t)(i - (b << logD)) == block_offset((uint32_t)b, size, seed);
-        const bool head = in && !((has_pred[i >> 5] >> (i & 31)) & 1u);
-        const bool extra = head && !strat;
-        const unsigned m = __ballot_sync(0xffffffffu, extra);
-        int first = 0;
-        if (lane == 0 && m) first = atomicAdd(&ctl->ff_extra, __popc(m));
-        first = __shfl_sync(0xffffffffu, first, 0);
-        if (!in) continue;
-        int64_t j = -1;
-        if (strat) j = b;
-        else if (extra) j = nb + first + __popc(m & lanemask_lt());
-        if (j >= r1_max) {
-            record_error(ctl, LRCC_ERR_INVALID_INPUT, -7);
-            j = -1;
-        }
-        if (j >= 0) {
-            W[i] = pack(nx | SPL, (uint32_t)j);
-            snext[j] = (int32_t)nx;
-            sw[j] = v;
-        } else {
-            W[i] = pack(nx, (uint32_t)v);
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int64_t i = b + q * 32 + lane;
+            const bool in = i < n;
+            if (b + q * 32 < n && lane == 0) named += __popc(pw[q]);
+            const bool head = in && !(pw[q] >> lane & 1);
+            const bool more = head && splitter_index32((uint32_t)i, g) < 0;
+            const unsigned m = __ballot_sync(0xffffffffu, more);
+            if (m) {
+                int first = 0;
+                if (lane == 0) first = atomicAdd(&ctl->ff_extra, __popc(m));
+                first = __shfl_sync(0xffffffffu, first, 0);
+                if (more) extra[first + __popc(m & lanemask_lt())] = (int32_t)i;
+            }
+            const bool tail = (sx[q] == -1) | (sx[q] == i) | (sx[q] < 0) | (sx[q] >= n);
+            if (in) W[i] = pack(tail ? NIL : (uint32_t)sx[q], (uint32_t)v[q]);
         }
     }
+    if (lane == 0 && named) atomicAdd(&ctl->named, named);
 }
 
-// Verdict for the forest: values outside the first level's range select the
-// pointer-jumping form (no error; that form takes any values).
-__global__ void ff_verdict(DevCtl* ctl) {
-    if (ctl->scan_bad || ctl->scan_total >= (1ull << 31)) ctl->scan_bad = 1;
-}
-
-__global__ void __launch_bounds__(BLOCK)
-    fs_pack(const int32_t* __restrict__ succ, const int32_t* __restrict__ val, int64_t n, uint64_t* __restrict__ W,
-            uint32_t* named, DevCtl* ctl) {
-    if (!ctl->scan_bad) return;   // only when the ruling-set form cannot take the values
-    const uint64_t pol = policy_evict_first();
-    for (int64_t i = (int64_t)blockIdx.x * BLOCK + threadIdx.x; i < n; i += (int64_t)gridDim.x * BLOCK) {
-        const int32_t sx = ld_stream(succ + i, pol);
-        const bool tail = (sx == -1) | (sx == i);
-        const bool bad = !tail && (sx < 0 || sx >= n);
-        W[i] = pack((tail || bad) ? NIL : (uint32_t)sx, (uint32_t)ld_stream(val + i, pol));
-    }
-}
-
-__global__ void __launch_bounds__(BLOCK)
-    fs_jump(const uint64_t* __restrict__ Win, uint64_t* __restrict__ Wout, int64_t n, const int* extra,
-            const DevCtl* ctl) {
-    // two uses: the whole forest when the values rule out the ruling set
-    // (extra == nullptr), or the forest of first-level splitters (n + *extra of them)
-    if (extra ? ctl->scan_bad : !ctl->scan_bad) return;
-    if (extra) n += *extra;
-    for (int64_t i = (int64_t)blockIdx.x * BLOCK + threadIdx.x; i < n; i += (int64_t)gridDim.x * BLOCK) {
-        uint64_t w = Win[i];
-        const uint32_t nx = lo32(w);
-        if (nx != NIL) {
-            const uint64_t x = Win[nx];
-            w = pack(lo32(x), hi32(w) + hi32(x));
+// The splitter forest's sums by pointer jumping in place: every word (next, sum
+// up to next) is read and written whole, and a word that another block has
+// already taken further only lengthens the jump, so no second buffer and no
+// copying of finished words is needed. Rounds end when no link is left, where a
+// launch per round had to make as many as the longest possible list needs.
+__global__ void __launch_bounds__(GANG_THREADS, 1)
+    ff_rounds(uint64_t* R, int64_t n, int64_t nb, GangCtl* gc, DevCtl* ctl) {
+    __shared__ int s_flag;
+    Gang G{gc, &gc->arrived[0], (int)gridDim.x, (int)blockIdx.x, 0, ctl, &s_flag};
+    const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    const int64_t r = nb + ctl->ff_extra;
+    const int64_t stride = (int64_t)gridDim.x * GANG_THREADS;
+    if (lead && (ctl->links != ctl->named || ctl->visited != (unsigned long long)n))
+        record_error(ctl, LRCC_ERR_INVALID_INPUT, -7);
+    int cap = 2;
+    while ((int64_t(1) << (cap - 2)) < r) ++cap;
+    for (int round = 0;; ++round) {
+        bool any = false;
+        for (int64_t i0 = (int64_t)blockIdx.x * GANG_THREADS + threadIdx.x; i0 < r; i0 += 4 * stride) {
+            uint64_t w[4], x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) w[q] = i0 + q * stride < r ? ld_cg_u64(R + i0 + q * stride) : pack(NIL, 0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = lo32(w[q]) < (uint64_t)r ? ld_cg_u64(R + lo32(w[q])) : pack(NIL, 0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (lo32(w[q]) == NIL) continue;
+                R[i0 + q * stride] = pack(lo32(x[q]), hi32(w[q]) + hi32(x[q]));
+                any |= lo32(x[q]) != NIL;
+            }
         }
-        Wout[i] = w;
-    }
-}
-
-__global__ void __launch_bounds__(BLOCK)
-    fs_final(const uint64_t* __restrict__ W, int64_t n, int32_t* __restrict__ out, const int* extra, DevCtl* ctl) {
-    if (extra ? ctl->scan_bad : !ctl->scan_bad) return;
-    if (extra) n += *extra;
-    for (int64_t i = (int64_t)blockIdx.x * BLOCK + threadIdx.x; i < n; i += (int64_t)gridDim.x * BLOCK) {
-        const uint64_t w = W[i];
-        if (lo32(w) != NIL) record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)i);
-        out[i] = (int32_t)hi32(w);
+        if (__syncthreads_or(any) && threadIdx.x == 0) atomicAdd(&gc->kept[round % 3], 1ull);
+        if (lead) gc->kept[(round + 1) % 3] = 0;
+        if (!G.sync()) return;
+        const bool more = *reinterpret_cast<volatile unsigned long long*>(&gc->kept[round % 3]) != 0;
+        if (!more || round >= cap) {
+            if (lead) {
+                if (more) record_error(ctl, LRCC_ERR_INVALID_INPUT, -2);
+                ctl->jump_rounds = round + 1;
+            }
+            return;
+        }
     }
 }
 
@@ -1931,6 +2020,21 @@ int stream_grid(Ctx* c, int64_t groups, const void* kernel) {
     const int pg = persistent_grid(c, kernel, BLOCK);
     const int64_t need = (groups + BLOCK - 1) / BLOCK;
     return (int)std::max<int64_t>(1, std::min<int64_t>(need, pg));
+}
+
+// Weighted ranks up to this size keep their records apart from the walk words
+// (16 bytes per element, within L2 up to about here).
+constexpr int64_t WALK_NEAR = int64_t(1) << 22;
+
+void enqueue_expand_values(Ctx* c, cudaStream_t s, const uint64_t* P, int64_t n, const uint32_t* S, int stride, int at,
+                           int64_t r, int32_t* out) {
+    const bool v = aligned16(out);
+    const void* k = v ? (const void*)rs_expand_values<true> : (const void*)rs_expand_values<false>;
+    const int g = stream_grid(c, (n + 3) / 4, k);
+    phase_begin(c, s);
+    if (v) rs_expand_values<true><<<g, BLOCK, 0, s>>>(P, n, S, stride, at, r, out, c->ctl);
+    else rs_expand_values<false><<<g, BLOCK, 0, s>>>(P, n, S, stride, at, r, out, c->ctl);
+    phase_end(c, s, PH_EXPAND0);
 }
 
 }  // namespace
@@ -1967,8 +2071,10 @@ int rs_walk_grid_current(const Plan& p) {
     return per_sm * sms;
 }
 
-RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int64_t given1, bool direct) {
+RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int64_t given1, bool direct, bool values) {
     RsLayout L;
+    values = values && p.rs_level0 == 1 && n > p.rs_small && n <= WALK_NEAR;
+    L.values = values;
     L.size[0] = n;
     // (batched lists, extra1 > 0, stay in L2 one after another at any total)
     direct = direct && p.rs_level0 == 1 && n > p.rs_small && (extra1 > 0 || n <= DIRECT_MAX);
@@ -1981,6 +2087,7 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
     // in-place walk words, the (element, rank) pairs of the read-only walk, or
     // the split mark and local-rank arrays (each 256-byte aligned)
     if (!direct) L.off_W0 = take(sizeof(uint64_t) * (size_t)n + 256);
+    if (values) L.off_P0 = take(sizeof(uint64_t) * (size_t)n);
     int64_t cur = n;
     int lvl = 0;
     while (cur > p.rs_small && lvl < MAX_LEVELS) {
@@ -2007,7 +2114,7 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
         ++lvl;
         L.size[lvl] = nb;
         L.off_R[lvl] = take(sizeof(uint64_t) * (size_t)nb);
-        if (lvl == 1 && !direct) {
+        if (lvl == 1 && !direct && !values) {
             L.off_snext = take(sizeof(int32_t) * (size_t)nb);
             L.off_sw = take(sizeof(int32_t) * (size_t)nb);
         }
@@ -2017,7 +2124,7 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
     L.levels = lvl;
     // level 1's records take over the successors and weights, which only the first level's walk reads
     for (int l = 1; l < lvl; ++l)
-        L.off_P[l] = l == 1 && !direct ? L.off_snext : take(sizeof(uint64_t) * (size_t)L.size[l]);
+        L.off_P[l] = l == 1 && !direct && !values ? L.off_snext : take(sizeof(uint64_t) * (size_t)L.size[l]);
     L.readonly = p.rs_level0 == 2 && lvl > 0 && walk_grid > 0;
     L.split = p.rs_level0 == 3 && lvl > 0;
     if (L.readonly) {
@@ -2155,10 +2262,10 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         phase_begin(c, s);
         if (vec)
             rs_select0<true><<<g, BLOCK, 0, s>>>(succ, val, n, head, W0, SN, SW, L.logD[0], L.size[1],
-                                                 seed0, ctl, given == nullptr);
+                                                 seed0, ctl, given == nullptr && !L.values);
         else
             rs_select0<false><<<g, BLOCK, 0, s>>>(succ, val, n, head, W0, SN, SW, L.logD[0], L.size[1],
-                                                  seed0, ctl, given == nullptr);
+                                                  seed0, ctl, given == nullptr && !L.values);
         if (given) {
             const int gm = stream_grid(c, given_r, (const void*)rs_mark_given);
             rs_mark_given<<<gm, BLOCK, 0, s>>>(W0, n, head, given, given_r, SN, SW, ctl);
@@ -2281,6 +2388,11 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         rs_walk_direct<<<(unsigned)((L0.nb + BLOCK - 1) / BLOCK), BLOCK, 0, s>>>(
             succ, reinterpret_cast<uint32_t*>(rank), L0, L.pbits, (int)(L.size[1] - L.fixed), R(1), ctl);
         phase_end(c, s, PH_WALK0);
+    } else if (L.values) {
+        phase_begin(c, s);
+        rs_walk_values<true><<<(unsigned)((L0.nb + BLOCK - 1) / BLOCK), BLOCK, 0, s>>>(
+            W0, reinterpret_cast<uint64_t*>(base + L.off_P0), L0, R(1), ctl);
+        phase_end(c, s, PH_WALK0);
     } else {
         walk0();
     }
@@ -2299,7 +2411,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         phase_begin(c, s);
         cudaFuncSetAttribute((const void*)rs_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         rs_final_kernel<<<1, FINAL_THREADS, smem, s>>>(R(lf), r, lf == 1 && L.direct ? (int)L.fixed : r, S(lf),
-                                                       val ? -1 : n, seed0, ctl);
+                                                       val ? -1 : n, L.values ? (unsigned long long)n : 0ull, seed0, ctl);
         phase_end(c, s, PH_FINAL);
     }
     for (int l = L.levels - 1; l >= 1; --l) {
@@ -2348,6 +2460,9 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         if (v) rs_expand_direct<true><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits);
         else rs_expand_direct<false><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits);
         phase_end(c, s, PH_EXPAND0);
+    } else if (L.values) {
+        const uint32_t* S1 = reinterpret_cast<const uint32_t*>(S(1));
+        enqueue_expand_values(c, s, reinterpret_cast<uint64_t*>(base + L.off_P0), n, S1, 1, 0, L.size[1], rank);
     } else {
         const bool v = vec && aligned16(rank);
         const void* k = v ? (const void*)rs_expand0<true> : (const void*)rs_expand0<false>;
@@ -2362,13 +2477,14 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
 }
 
 // Forest layout: walk words W0 (8 B per element), the has-predecessor bitmap,
-// then for r1_max = nb + n first-level splitters (every element could be a
-// head) their successor and weight, two word buffers and the sums. The
-// pointer-jumping form reuses W0 and the first word buffer.
+// and for r1_max = nb + n first-level splitters (every element could be a head)
+// 8 bytes for the elements' records (when they are not kept in W0), their packed
+// words and the extra splitters' elements; the layout keeps the size it had with
+// a second word buffer (37 to 40 bytes per element), which callers budget for.
 struct ForestLayout {
     int logD;
     int64_t nb, r1_max;
-    size_t off_W0, off_pred, off_snext, off_sw, off_R1, off_R1b, off_S1, bytes;
+    size_t off_W0, off_pred, off_P0, off_R1, off_R1b, off_extra, bytes;
 };
 
 ForestLayout forest_layout(int64_t n, int spacing0) {
@@ -2385,11 +2501,10 @@ ForestLayout forest_layout(int64_t n, int spacing0) {
     };
     F.off_W0 = take(sizeof(uint64_t) * (size_t)n);
     F.off_pred = take(sizeof(uint32_t) * (size_t)((n + 31) / 32));
-    F.off_snext = take(sizeof(int32_t) * (size_t)F.r1_max);
-    F.off_sw = take(sizeof(int32_t) * (size_t)F.r1_max);
+    F.off_P0 = take(sizeof(uint64_t) * (size_t)F.r1_max);
     F.off_R1 = take(sizeof(uint64_t) * (size_t)F.r1_max);
     F.off_R1b = take(sizeof(uint64_t) * (size_t)F.r1_max);
-    F.off_S1 = take(sizeof(int32_t) * (size_t)F.r1_max);
+    F.off_extra = take(sizeof(int32_t) * (size_t)F.r1_max);
     F.bytes = off;
     return F;
 }
@@ -2402,71 +2517,43 @@ lrcc_status lr_enqueue_scan_forest(Ctx* c, cudaStream_t s, const int32_t* succ, 
     char* base = static_cast<char*>(c->ws);
     uint64_t* W0 = reinterpret_cast<uint64_t*>(base + F.off_W0);
     uint32_t* pred = reinterpret_cast<uint32_t*>(base + F.off_pred);
-    int32_t* snext = reinterpret_cast<int32_t*>(base + F.off_snext);
-    int32_t* sw = reinterpret_cast<int32_t*>(base + F.off_sw);
+    uint64_t* P0 = n <= WALK_NEAR ? reinterpret_cast<uint64_t*>(base + F.off_P0) : W0;
     uint64_t* R1 = reinterpret_cast<uint64_t*>(base + F.off_R1);
-    uint64_t* R1b = reinterpret_cast<uint64_t*>(base + F.off_R1b);
-    int32_t* S1 = reinterpret_cast<int32_t*>(base + F.off_S1);
+    int32_t* extra = reinterpret_cast<int32_t*>(base + F.off_extra);
     DevCtl* ctl = c->ctl;
-    const int g = stream_grid(c, n, (const void*)ff_indeg);
-    const uint32_t seed = (uint32_t)(p.seed ^ (p.seed >> 32));
+    Level0 L0;
+    L0.n = n;
+    L0.nb = F.nb;
+    L0.logD = F.logD;
+    L0.seed = (uint32_t)(p.seed ^ (p.seed >> 32));
+    // no head among the stratified splitters: block 0 keeps its own
+    L0.bh = 0;
+    L0.head_off = (uint32_t)((uint64_t)mix32(L0.seed) * (uint64_t)std::min<int64_t>(n, int64_t(1) << F.logD) >> 32);
+    L0.extra = extra;
+    L0.extra_count = &ctl->ff_extra;
     cudaMemsetAsync(pred, 0, sizeof(uint32_t) * (size_t)((n + 31) / 32), s);
     phase_begin(c, s);
-    ff_indeg<<<g, BLOCK, 0, s>>>(succ, n, pred, ctl);
-    rs_scan_check<<<g, BLOCK, 0, s>>>(val, n, ctl);
-    ff_verdict<<<1, 1, 0, s>>>(ctl);
-    ff_select0<<<g, BLOCK, 0, s>>>(succ, val, n, pred, W0, snext, sw, F.logD, F.nb, F.r1_max, seed, ctl);
+    ff_links<<<stream_grid(c, (n + 3) / 4, (const void*)ff_links), BLOCK, 0, s>>>(succ, n, pred, ctl);
+    ff_select<<<stream_grid(c, (n + 3) / 4, (const void*)ff_select), BLOCK, 0, s>>>(succ, val, n, pred, W0, extra, L0, ctl);
     phase_end(c, s, PH_SELECT0);
     phase_begin(c, s);
-    {
-        const int gw = persistent_grid(c, (const void*)rs_walk<1>, BLOCK);
-        rs_walk<1><<<gw, BLOCK, 0, s>>>(W0, snext, sw, R1, (int)F.nb, &ctl->work[0], n, ctl, &ctl->ff_extra);
-    }
+    // (a few heads more than nb threads are left to the stride)
+    const unsigned gw = (unsigned)((F.nb + BLOCK - 1) / BLOCK);
+    if (P0 != W0) rs_walk_values<true><<<gw, BLOCK, 0, s>>>(W0, P0, L0, R1, ctl);
+    else rs_walk_values<false><<<gw, BLOCK, 0, s>>>(W0, P0, L0, R1, ctl);
     phase_end(c, s, PH_WALK0);
-    // the splitter forest by pointer jumping; rounds for the largest possible count
-    int rounds = 0;
-    while ((int64_t(1) << rounds) < F.r1_max) ++rounds;
-    const int g1 = stream_grid(c, F.nb, (const void*)fs_jump);
-    uint64_t* a = R1;
-    uint64_t* b = R1b;
-    for (int r = 0; r < rounds; ++r) {
-        phase_begin(c, s);
-        fs_jump<<<g1, BLOCK, 0, s>>>(a, b, F.nb, &ctl->ff_extra, ctl);
-        phase_end(c, s, PH_WY_JUMP);
-        std::swap(a, b);
-    }
     phase_begin(c, s);
-    fs_final<<<g1, BLOCK, 0, s>>>(a, F.nb, S1, &ctl->ff_extra, ctl);
-    phase_end(c, s, PH_FINAL);
     {
-        const bool v = aligned16(out);
-        const void* k = v ? (const void*)rs_expand0<true> : (const void*)rs_expand0<false>;
-        const int ge = stream_grid(c, (n + 3) / 4, k);
-        phase_begin(c, s);
-        if (v) rs_expand0<true><<<ge, BLOCK, 0, s>>>(W0, n, S1, F.r1_max, out, 0, ctl);
-        else rs_expand0<false><<<ge, BLOCK, 0, s>>>(W0, n, S1, F.r1_max, out, 0, ctl);
-        phase_end(c, s, PH_EXPAND0);
+        GangCtl* gc = reinterpret_cast<GangCtl*>(reinterpret_cast<char*>(ctl) + offsetof(DevCtl, gang));
+        int64_t nn = n, nb = F.nb;
+        uint64_t* words = R1;
+        void* args[] = {&words, &nn, &nb, &gc, &ctl};
+        const int blocks = (int)std::min<int64_t>(c->sms, (F.nb + GANG_THREADS - 1) / GANG_THREADS);
+        if (cudaLaunchCooperativeKernel((const void*)ff_rounds, dim3(blocks), dim3(GANG_THREADS), args, 0, s) != cudaSuccess)
+            return LRCC_ERR_CUDA;
     }
-    // values out of the first level's range: the whole forest by pointer jumping
-    // (these kernels return at once otherwise)
-    {
-        uint64_t* x = W0;
-        uint64_t* y = R1;   // r1_max >= n words
-        phase_begin(c, s);
-        fs_pack<<<g, BLOCK, 0, s>>>(succ, val, n, x, pred, ctl);
-        phase_end(c, s, PH_WY_PACK);
-        int rr = 0;
-        while ((int64_t(1) << rr) < n) ++rr;
-        for (int r = 0; r < rr; ++r) {
-            phase_begin(c, s);
-            fs_jump<<<g, BLOCK, 0, s>>>(x, y, n, nullptr, ctl);
-            phase_end(c, s, PH_WY_JUMP);
-            std::swap(x, y);
-        }
-        phase_begin(c, s);
-        fs_final<<<g, BLOCK, 0, s>>>(x, n, out, nullptr, ctl);
-        phase_end(c, s, PH_WY_FINAL);
-    }
+    phase_end(c, s, PH_WY_JUMP);
+    enqueue_expand_values(c, s, P0, n, reinterpret_cast<uint32_t*>(R1), 2, 1, F.r1_max, out);
     return cuda_status(cudaGetLastError());
 }
 

@@ -361,7 +361,7 @@ int lrcc_version(void) { return 101; }
 
 namespace {
 
-// Weighted sums: the in-place first level carries the values in packed words.
+// Weighted sums: the first level carries the values in packed words.
 // Above 2^22 elements its splitters are at least 16 apart: as fast as 8 apart
 // (15,000,000 elements: 491 us both), in 9.7 bytes per element instead of 11.3.
 Plan scan_plan(int64_t n) {
@@ -377,7 +377,8 @@ lrcc_status lr_rank_locked(Ctx* c, const int32_t* succ, int64_t n, int32_t head,
     lrcc_status st = LRCC_OK;
     const Plan p = val ? scan_plan(n) : plan_for(KIND_LR, n);
     // (a caller that ranks in place, out = succ, keeps the packed words)
-    const RsLayout L = rs_layout(n, p, rs_walk_grid(c, p), 0, 0, !val && !arrays_overlap(succ, rank, n));
+    const RsLayout L =
+        rs_layout(n, p, rs_walk_grid(c, p), 0, 0, !val && !arrays_overlap(succ, rank, n), val != nullptr);
     if (n > p.rs_small) {
         st = ensure_ws(c, L.bytes);
         if (st != LRCC_OK) return st;
@@ -479,7 +480,7 @@ lrcc_status lr_scan_forest(const int32_t* succ, const int32_t* val, int64_t n, i
     lrcc_status st = ctx_for(stream, &c);
     if (st != LRCC_OK) return st;
     std::lock_guard<std::mutex> lk(c->mu);
-    const Plan p = plan_for(KIND_LR, n);
+    const Plan p = scan_plan(n);
     st = ensure_ws(c, lr_scan_forest_ws(n, p));
     if (st != LRCC_OK) return st;
     const std::vector<uint64_t> key = {7, (uint64_t)succ, (uint64_t)val, (uint64_t)n, (uint64_t)out};
@@ -975,9 +976,9 @@ int64_t lrcc_workspace_query(int kind, int64_t n, int64_t m) {
     switch (kind) {
         case 6: {   // lr_scan: the in-place first level
             const Plan ps = scan_plan(n);
-            return n > ps.rs_small ? (int64_t)rs_layout(n, ps, rs_walk_grid_current(ps)).bytes : 0;
+            return n > ps.rs_small ? (int64_t)rs_layout(n, ps, rs_walk_grid_current(ps), 0, 0, false, true).bytes : 0;
         }
-        case 7: return (int64_t)lr_scan_forest_ws(n, p);   // lr_scan_forest
+        case 7: return (int64_t)lr_scan_forest_ws(n, scan_plan(n));   // lr_scan_forest
         case KIND_LR: {
             // the walk's block count on the current device (as on a GB300 when none can be queried)
             return n > p.rs_small ? (int64_t)rs_layout(n, p, rs_walk_grid_current(p), 0, 0, true).bytes : 0;
