@@ -68,6 +68,8 @@ def library_path() -> str:
 def load() -> ctypes.CDLL:
     """Load liblrcc.so (built in-tree by ``__graft_entry__.build()``)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -136,10 +138,18 @@ def status_str(status: int) -> str:
     return load().lrcc_status_str(int(status)).decode()
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+# The current stream's handle without a Stream object around it: small calls last
+# a few microseconds, and building the object takes three of them.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream(stream) -> int:
+    """The cudaStream_t of ``stream`` (None: the current stream of the current device)."""
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _dev_i32(t: torch.Tensor, name: str) -> torch.Tensor:
@@ -160,7 +170,7 @@ def _dev_i64(t: torch.Tensor, name: str) -> torch.Tensor:
 
 def _out(out, n, like, name):
     if out is None:
-        return torch.empty(n, dtype=torch.int32, device=like.device)
+        return like.new_empty(n)   # int32 on like's device, as like was checked to be
     _dev_i32(out, name)
     if out.numel() != n:
         raise ValueError(f"{name} must hold {n} elements")

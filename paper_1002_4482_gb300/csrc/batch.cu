@@ -712,10 +712,6 @@ __global__ void __launch_bounds__(SEG_BLOCK)
     }
 }
 
-lrcc_status set_smem(const void* k, size_t bytes) {
-    return cuda_status(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-}
-
 }  // namespace
 
 size_t lr_batched_ws(int64_t total_nodes, int64_t count) {
@@ -749,9 +745,8 @@ lrcc_status lr_batched_run(Ctx* c, const int32_t* succ, const int64_t* off, cons
     phase_end(c, s, PH_BATCH_PREP);
     auto small_k = lr_batch_kernel<BT, SMEM_ELEMS, false>;
     auto large_k = lr_batch_kernel<BT_LARGE, SMEM_ELEMS_LARGE, true>;
-    lrcc_status st = set_smem((const void*)small_k, LR_SMEM_BYTES);
-    if (st == LRCC_OK) st = set_smem((const void*)large_k, LR_SMEM_LARGE);
-    if (st != LRCC_OK) return st;
+    allow_smem(c, (const void*)small_k, LR_SMEM_BYTES);
+    allow_smem(c, (const void*)large_k, LR_SMEM_LARGE);
     int min_logD = 2;
     while (min_logD < 20 && (1 << (min_logD + 1)) <= p.rs_spacing0) ++min_logD;
     const uint32_t seed = (uint32_t)(p.seed ^ (p.seed >> 32));
@@ -877,8 +872,7 @@ lrcc_status cc_batched_run(Ctx* c, const int32_t* src, const int32_t* dst, const
     phase_end(c, s, PH_CC_LOOP);
 
     // every other graph: one block each, largest first
-    lrcc_status st = set_smem((const void*)cc_batch_kernel, CC_SMEM_BYTES);
-    if (st != LRCC_OK) return st;
+    allow_smem(c, (const void*)cc_batch_kernel, CC_SMEM_BYTES);
     const int g = (int)std::min<int64_t>(count, persistent_grid(c, (const void*)cc_batch_kernel, BT, CC_SMEM_BYTES));
     phase_begin(c, s);
     cc_batch_kernel<<<g, BT, CC_SMEM_BYTES, s>>>(src, dst, eoff, voff, count, order, label, p.cc_max_rounds, c->ctl);

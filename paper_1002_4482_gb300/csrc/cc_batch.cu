@@ -260,7 +260,7 @@ lrcc_status cc_batch_gang_run(Ctx* c, const int32_t* src, const int32_t* dst, co
     phase_end(c, s, PH_CC_LOOP);
     if (st != LRCC_OK) return st;
     phase_begin(c, s);
-    cudaFuncSetAttribute((const void*)cc_batch_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM);
+    allow_smem(c, (const void*)cc_batch_small, SMALL_SMEM);
     const int g = (int)std::min<int64_t>(count, persistent_grid(c, (const void*)cc_batch_small, SMALL_THREADS, SMALL_SMEM));
     cc_batch_small<<<g, SMALL_THREADS, SMALL_SMEM, s>>>(src, dst, eoff, voff, count, order, plan, label, c->ctl);
     phase_end(c, s, PH_CC_BATCH);

@@ -63,6 +63,7 @@ __global__ void __launch_bounds__(GANG_THREADS, 1)
         label[v] = x;
     }
     if (threadIdx.x == 0) {
+        clear_stats(ctl);   // a call of one launch has no memset before it
         ctl->rounds = 1;
         ctl->edges_read = (unsigned long long)m;
     }
@@ -183,7 +184,7 @@ GangShape gang_shape(int64_t m, int64_t n, int sms) {
 }
 
 lrcc_status launch_gang(Ctx* c, const void* kernel, GangParams& P, int blocks, size_t smem) {
-    if (smem) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (smem) allow_smem(c, kernel, smem);
     GangCtl* gc = reinterpret_cast<GangCtl*>(reinterpret_cast<char*>(c->ctl) + offsetof(DevCtl, gang));
     DevCtl* ctl = c->ctl;
     void* args[] = {&P, &gc, &ctl};
@@ -204,7 +205,7 @@ lrcc_status cc_run_gang(Ctx* c, const int32_t* src, const int32_t* dst, int64_t 
                         const Plan& p) {
     if (cc_one_block_applies(m, n)) {
         const size_t smem = sizeof(int) * (size_t)n;
-        cudaFuncSetAttribute((const void*)cc_one_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(c, (const void*)cc_one_block, sizeof(int) * ONE_MAX_N);
         phase_begin(c, c->stream);
         cc_one_block<<<1, GANG_THREADS, smem, c->stream>>>(src, dst, (int)m, (int)n, label, c->ctl);
         phase_end(c, c->stream, PH_CC_LOOP);

@@ -43,6 +43,12 @@ __device__ __forceinline__ void record_error(DevCtl* c, int code, int where = -1
     if (atomicCAS(&c->status, 0, code) == 0) c->err_where = where;
 }
 
+// What lrcc_last_stats reads, for calls that do not clear the whole block first.
+__device__ __forceinline__ void clear_stats(DevCtl* c) {
+    c->rounds = c->jump_rounds = c->ovf_next = 0;
+    c->edges_read = 0;
+}
+
 // ------------------------------------------------------------ packed words --
 
 // List ranking moves (value, pointer) pairs as one 8-byte word so that a jump

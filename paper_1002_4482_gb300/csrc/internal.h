@@ -157,6 +157,10 @@ int64_t ctx_bytes(const Ctx* c);
 lrcc_status ensure_ws(Ctx* c, size_t bytes);
 lrcc_status cuda_status(cudaError_t e);
 
+// Lets a kernel take up to `bytes` of dynamic shared memory on c's device (one
+// attribute call per kernel and size, not one per launch).
+void allow_smem(Ctx* c, const void* kernel, size_t bytes);
+
 // Persistent grid size for a kernel: SMs x resident blocks per SM.
 int persistent_grid(Ctx* c, const void* kernel, int block, size_t smem = 0);
 

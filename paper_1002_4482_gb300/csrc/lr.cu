@@ -84,7 +84,10 @@ __global__ void __launch_bounds__(FINAL_THREADS, 1)
     }
     bool whole;
     const uint2* res = block_rank<FINAL_THREADS>(W, sub, n, head, seed, &whole, ctl);
-    if (threadIdx.x == 0 && !whole) record_error(ctl, LRCC_ERR_INVALID_INPUT, head);
+    if (threadIdx.x == 0) {
+        if (!whole) record_error(ctl, LRCC_ERR_INVALID_INPUT, head);
+        clear_stats(ctl);   // a call of one launch has no memset before it
+    }
     const int bias = w ? 0 : 1;
 #pragma unroll 4
     for (int i = threadIdx.x; i < n; i += FINAL_THREADS) rank[i] = block_rank_sum<FINAL_THREADS>(W[i], res) - bias;
@@ -1995,7 +1998,7 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
 lrcc_status launch_small(Ctx* c, cudaStream_t s, const int32_t* succ, int n, int head, int32_t* rank, uint32_t seed,
                          const int32_t* val = nullptr) {
     const size_t smem = br_smem(n);
-    cudaFuncSetAttribute((const void*)lr_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(c, (const void*)lr_small_kernel, br_smem(16384));
     phase_begin(c, s);
     lr_small_kernel<<<1, FINAL_THREADS, smem, s>>>(succ, val, n, head, rank, seed, c->ctl);
     phase_end(c, s, PH_SMALL);
@@ -2007,7 +2010,7 @@ lrcc_status launch_small_wyllie(Ctx* c, cudaStream_t s, const int32_t* succ, int
     const size_t smem = 2 * sizeof(int) * per * FINAL_THREADS;
     const void* k = per == 4 ? (const void*)wy_small_kernel<4>
                   : per == 8 ? (const void*)wy_small_kernel<8> : (const void*)wy_small_kernel<16>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(c, k, smem);
     phase_begin(c, s);
     if (per == 4) wy_small_kernel<4><<<1, FINAL_THREADS, smem, s>>>(succ, n, head, rank, c->ctl);
     else if (per == 8) wy_small_kernel<8><<<1, FINAL_THREADS, smem, s>>>(succ, n, head, rank, c->ctl);
@@ -2409,7 +2412,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         const int r = (int)L.size[lf];
         const size_t smem = br_smem(r);
         phase_begin(c, s);
-        cudaFuncSetAttribute((const void*)rs_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(c, (const void*)rs_final_kernel, br_smem(16384));
         rs_final_kernel<<<1, FINAL_THREADS, smem, s>>>(R(lf), r, lf == 1 && L.direct ? (int)L.fixed : r, S(lf),
                                                        val ? -1 : n, L.values ? (unsigned long long)n : 0ull, seed0, ctl);
         phase_end(c, s, PH_FINAL);
@@ -2427,7 +2430,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     }
     if (L.readonly) {
         phase_begin(c, s);
-        cudaFuncSetAttribute((const void*)rs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SC_SMEM);
+        allow_smem(c, (const void*)rs_scatter, SC_SMEM);
         const int gs = std::min((int)L.grid, persistent_grid(c, (const void*)rs_scatter, BLOCK, SC_SMEM));
         rs_scatter<<<gs, BLOCK, SC_SMEM, s>>>(C, (int)L.grid, S(1), W0, n, ctl);
         phase_end(c, s, PH_SCATTER);

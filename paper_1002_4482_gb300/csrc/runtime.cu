@@ -207,6 +207,16 @@ int persistent_grid(Ctx* c, const void* kernel, int block, size_t smem) {
     return g;
 }
 
+void allow_smem(Ctx* c, const void* kernel, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, size_t> allowed;
+    std::lock_guard<std::mutex> lk(mu);
+    size_t& have = allowed[std::make_pair(c->device, kernel)];
+    if (bytes <= have) return;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess) have = bytes;
+    else cudaGetLastError();   // the launch reports it
+}
+
 lrcc_status ctx_for(void* stream, Ctx** out) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return LRCC_ERR_CUDA;
@@ -383,14 +393,19 @@ lrcc_status lr_rank_locked(Ctx* c, const int32_t* succ, int64_t n, int32_t head,
         st = ensure_ws(c, L.bytes);
         if (st != LRCC_OK) return st;
     }
-    std::vector<uint64_t> key = {(uint64_t)KIND_LR, (uint64_t)succ, (uint64_t)n, (uint64_t)head, (uint64_t)rank,
-                                 (uint64_t)val};
-    const auto pk = plan_key(p);
-    key.insert(key.end(), pk.begin(), pk.end());
-    st = launch_recorded(c, p, key, [&](cudaStream_t s) {
-        reset_ctl(c, s);
-        return lr_enqueue_rs(c, s, succ, n, head, rank, p, L, val);
-    });
+    if (n <= p.rs_small && !val) {
+        // one launch, which also clears the counters: no graph to record or look up
+        st = lr_enqueue_rs(c, c->stream, succ, n, head, rank, p, L);
+    } else {
+        std::vector<uint64_t> key = {(uint64_t)KIND_LR, (uint64_t)succ, (uint64_t)n, (uint64_t)head, (uint64_t)rank,
+                                     (uint64_t)val};
+        const auto pk = plan_key(p);
+        key.insert(key.end(), pk.begin(), pk.end());
+        st = launch_recorded(c, p, key, [&](cudaStream_t s) {
+            reset_ctl(c, s);
+            return lr_enqueue_rs(c, s, succ, n, head, rank, p, L, val);
+        });
+    }
     c->last_kind = val ? 6 : KIND_LR;
     c->last_levels = n > p.rs_small ? L.levels : 0;
     for (int l = 0; l < MAX_LEVELS; ++l) c->last_splitter_cap[l] = l < L.levels ? L.size[l + 1] : 0;
@@ -404,7 +419,7 @@ lrcc_status cc_label_locked(Ctx* c, const int32_t* src, const int32_t* dst, int6
     const bool gang = cc_gang_applies(p);
     lrcc_status st = ensure_ws(c, sv ? cc_sv_ws(n) : gang ? cc_gang_ws(m, n, c->sms) : cc_ws(m));
     if (st != LRCC_OK) return st;
-    reset_ctl(c, c->stream);
+    if (!(gang && cc_one_block_applies(m, n))) reset_ctl(c, c->stream);   // the one-block kernel clears its counters
     st = sv     ? cc_run_sv(c, src, dst, m, n, label, p)
          : gang ? cc_run_gang(c, src, dst, m, n, label, p)
                 : cc_run(c, src, dst, m, n, label, p);
