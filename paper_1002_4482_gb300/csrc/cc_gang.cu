@@ -11,7 +11,7 @@
 //
 // Measured against the loop of launches (us): uniform 2^20 vertices, 2^22 edges
 // 146 / 266; 1021 vertices, 2042 edges 17 / 56; paths of 8M vertices 383 / 926;
-// R-MAT scale 20, 2^24 edges 144 / 2350; scale 24, 2^28 edges 2049 / 2498 (bound by
+// R-MAT scale 20, 2^24 edges 144 / 2350; scale 24, 2^28 edges 1725 / 2498 (bound by
 // the gathers the member table does not answer, one L2 request each).
 //
 // Why no connection is lost: a hook writes p[hi] = min(p[hi], lo) where hi was
@@ -234,13 +234,16 @@ lrcc_status cc_run_gang(Ctx* c, const int32_t* src, const int32_t* dst, int64_t 
     // then holds most vertices, and the edges after the sample are mostly
     // dropped unread of their roots (2^20 vertices, 4 edges each: 142 us, 246
     // without). Below 2^19 edges a second launch costs what it saves (R-MAT scale
-    // 14: 42 us without a sample, 57 with); with 1.5 edges per vertex half the
+    // 14: 42 us without a sample, 57 with); from 16 edges per vertex and 2^22
+    // vertices up half an edge per vertex is enough (R-MAT scale 24: 1.72 ms, 1.77
+    // with one; scale 21: 314 us, 290 with one); with 1.5 edges per vertex half the
     // edges pay from 2^22 vertices on (2^24: 1111 against 1268 us; 2^20: 139
     // against 128).
     int64_t ms = m;
     if (p.cc_sample > 1) ms = m / p.cc_sample;
     else if (p.cc_sample < 0 && m >= (int64_t(1) << 19))
-        ms = m >= 2 * n ? n : n >= (int64_t(1) << 22) && 2 * m >= 3 * n ? m / 2 : m;
+        ms = m >= 16 * n && n >= (int64_t(1) << 22) ? n / 2
+             : m >= 2 * n ? n : n >= (int64_t(1) << 22) && 2 * m >= 3 * n ? m / 2 : m;
     P.ms = ms >= 4096 ? ms & ~int64_t(3) : m;
     P.first = P.ms;
     const bool sampled = P.ms < m;

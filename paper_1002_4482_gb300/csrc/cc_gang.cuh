@@ -208,8 +208,8 @@ __device__ __forceinline__ void smem_join(volatile int* p, int u, int v) {
 //         so an entry is never wrong. A warp whose vertices hit less than one
 //         time in 32 stops asking.
 // 130 KB is the best size on GB300: the rest of the 256 KB is L1, which the
-// gathers need for their lines in flight (R-MAT scale 24, filter pass: 1.43 ms
-// with 128 KB, 2.0 with 160 KB, 2.05 without a table).
+// gathers need for their lines in flight (R-MAT scale 24, filter pass: 1.4 ms with
+// 128 KB, 2.0 with 160 KB, 2.05 without a table).
 enum Table { TABLE_NONE, TABLE_BITS, TABLE_TAGS };
 constexpr int TABLE_BYTES = 130 << 10;
 constexpr int64_t BITS_MAX_N = int64_t(TABLE_BYTES) * 8;
@@ -362,6 +362,7 @@ struct GangWork {
         int32_t u[GANG_EDGES], v[GANG_EDGES];
         bool ok[GANG_EDGES];
         bool ask = TABLE != TABLE_NONE;
+        const unsigned warm = (unsigned)((hi - lo) / (12 * GANG_STEP));
         int hits = 0;
         for (int64_t i = lo; i < hi; i += GANG_STEP, ++it) {
             gang_load<VEC>(P.g, i, hi, stream_pol, u, v, ok, ctl);
@@ -397,7 +398,7 @@ struct GangWork {
                     if (!in_u) a[q] = ld_cg_hint(p + u[q], keep);
                     if (!in_v) b[q] = ld_cg_hint(p + v[q], keep);
                 }
-                const bool clear = ((it + lane()) & 7) == 0;
+                const bool clear = ((it / 16 + lane()) & 7) == 0;
                 auto learn = [&](int32_t x, uint32_t e, int32_t root) {
                     const uint32_t tag = (uint32_t)x / TAG_SLOTS;
                     unsigned char* slot = s_table + (uint32_t)x % TAG_SLOTS;
@@ -408,6 +409,9 @@ struct GangWork {
                         else if (clear) *slot = (unsigned char)(e & TAG_MASK);
                     }
                 };
+                // learning costs as much as asking: in the first twelfth of the share, then
+                // in every sixteenth iteration (1.98 -> 1.77 ms, R-MAT scale 24)
+                if (it < warm || (it & 15) == 0)
 #pragma unroll
                 for (int q = 0; q < GANG_EDGES; ++q)
                     if (ok[q]) {
