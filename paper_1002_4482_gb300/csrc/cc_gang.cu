@@ -171,11 +171,14 @@ GangShape gang_shape(int64_t m, int64_t n, int sms) {
     // a block for every 2048 edges or vertices: small graphs have cheaper barriers
     s.blocks = (int)std::max<int64_t>(1, std::min<int64_t>(sms, (std::max(m, n) + 2047) / 2048));
     const int64_t warps = (int64_t)s.blocks * GANG_WARPS;
-    // Pairs for three eighths of the edges (paths keep a third of theirs after
-    // the first passes), for a quarter above 2^26 edges; a warp that keeps more
-    // reads the rest of its share again. Only the warps that have a share count.
+    // Pairs for three quarters of the edges of a sparse graph (a uniform one of 1
+    // edge per vertex keeps two thirds after the first passes: 104 us, 128 with
+    // half the room), for three eighths where a sample leaves fewer, for a quarter
+    // above 2^26 edges; a warp that keeps more reads the rest of its share again.
+    // Only the warps that have a share count.
     const int64_t per = gang_share(m, warps);
-    s.capw = (int)(m <= (int64_t(1) << 26) ? per * 3 / 8 : per / 4) + 16;
+    s.capw = (int)(m > (int64_t(1) << 26) ? per / 4 : m < 2 * n ? per * 3 / 4 : per * 3 / 8) + 16;
+    s.capw = std::max(s.capw, GANG_STEP);   // one iteration's pairs, also of a short sample
     const int64_t used = std::min(warps, (m + GANG_STEP - 1) / GANG_STEP);   // the sample's shares are shorter
     s.off_left = align_up(sizeof(int2) * (size_t)s.capw * (size_t)std::max<int64_t>(used, 1), 256);
     s.off_bits = s.off_left + align_up(sizeof(int2) * (size_t)(warps + 1), 256);
@@ -253,7 +256,7 @@ lrcc_status cc_run_gang(Ctx* c, const int32_t* src, const int32_t* dst, int64_t 
     // us against 160), the first of which need not read the parents unless the
     // pass is long or the graph dense.
     P.sample_passes = m >= 8 * n && P.ms >= (int64_t(1) << 20) ? 1 : 3;
-    P.first_min = sampled ? P.sample_passes > 1 && P.ms < (int64_t(1) << 22) : m < 2 * n;
+    P.first_min = sampled ? P.sample_passes > 1 && P.ms < (int64_t(1) << 22) : m <= 4 * n;
     const int table = !sampled ? TABLE_NONE : n <= BITS_MAX_N ? TABLE_BITS : n <= TAGS_MAX_N ? TABLE_TAGS : TABLE_NONE;
     const bool vec = aligned16(src) && aligned16(dst);
     const bool bits = table == TABLE_BITS;
