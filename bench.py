@@ -34,8 +34,10 @@ sys.path.insert(0, ROOT)
 METRIC = "LR Mnodes/s and CC Medges/s at 1 GB300, % of HBM roofline; batched vs per-launch"
 UNIT = "M(list nodes + graph edges)/s"
 # bytes per element that the first ruling-set level moves, by layout (plan.rs_level0)
-LR_METHOD_FIRST = {1: 40, 2: 34, 3: 38}
+# (0: records in the rank array, the in-place level of lists up to 2^24)
+LR_METHOD_FIRST = {0: 16, 1: 40, 2: 34, 3: 38}
 LR_METHOD_NOTE = {
+    0: "walk 4 B read + 4 B written, expand 4 B read + 4 B written",
     1: "select 4 B read + 8 B written, walk 8 B read + 8 B written, expand 8 B read + 4 B written",
     2: "walk 4 B read + 5 B written, scatter 5 B read + 8 B written, placement 8 B read + 4 B written",
     3: "select 4 B read + 4 B written, walk 8 B read + 8 B written, expand 8 B read + 4 B written",
@@ -329,12 +331,13 @@ def chase_peak(lrcc, torch, succ, stream, chain_logs=(19, 20, 21, 22, 23)):
 
 def bench_lr_sweep(lrcc, torch, dev, stream, sizes=(16, 18, 20, 22, 24, 26, 28)):
     """List-ranking throughput against list size for the three first-level layouts
-    (in-place 8-byte words, read-only walk with chunked records, split mark and
-    local-rank arrays) and both list layouts (random, ordered = even splitters along
+    (in place: records in the rank array up to 2^24 elements, 8-byte words above;
+    read-only walk with chunked records; split mark and local-rank arrays) and both list layouts (random, ordered = even splitters along
     the list): where the rate changes as the list outgrows L2 (the paper's
     "inflection", Sec. 3.2). The paper's own comparison, the 48-bit split arrays
     (16-bit marks, so fewer than 65,535 splitters) against the packed 64-bit words
-    at the same spacing, is measured on the random layout as `paper48` / `paper64`."""
+    at the same spacing, is measured on the random layout as `paper48` / `paper64` (the
+    in-place form at that spacing: packed words above 2^24)."""
     import gen
     out = []
     base = {k: lrcc.get_plan(lrcc.KIND_LR, 1 << k) for k in sizes}
@@ -458,8 +461,8 @@ def bench_small_configs(lrcc, torch, dev, stream, hbm, reps=20):
 def bench_even_splitters(lrcc, torch, dev, stream, sizes=(16, 20, 24, 28)):
     """The paper's Table 3 on GB300 (Sec. 3.2): the same random-layout list
     ranked with random splitters and with a perfect set of even splitters (list
-    positions 0, D, 2D, ...: every sublist exactly D elements), both through the
-    in-place first level at the plan's spacing D."""
+    positions 0, D, 2D, ...: every sublist exactly D elements), both given to the
+    in-place first level of 8-byte words at the plan's spacing D."""
     import gen
     out = []
     base = {k: lrcc.get_plan(lrcc.KIND_LR, 1 << k) for k in sizes}
@@ -487,15 +490,19 @@ def bench_even_splitters(lrcc, torch, dev, stream, sizes=(16, 20, 24, 28)):
                 s_d = torch.from_numpy(succ_h).to(dev)
                 r_d = torch.empty_like(s_d)
                 even = torch.from_numpy(np.ascontiguousarray(perm[::D])).to(dev)
+                # one random element of every D consecutive ids (the head in its block), the head first
+                ids = np.arange(0, n, D) + np.random.default_rng(lg).integers(0, D, n // D)
+                ids[head // D] = head
+                rand = torch.from_numpy(np.roll(ids, -(head // D)).astype(np.int32)).to(dev)
             lrcc.set_plan(lrcc.KIND_LR, lg, lg, rs_level0=1)
-            t_rand = best_ms(lambda: lrcc.lr_rank(s_d, head, out=r_d, stream=stream))
+            t_rand = best_ms(lambda: lrcc.lr_rank_splitters(s_d, head, rand, out=r_d, stream=stream))
             t_even = best_ms(lambda: lrcc.lr_rank_splitters(s_d, head, even, out=r_d, stream=stream))
             if int(r_d[head].item()) != n - 1:
                 raise AssertionError("even splitters gave a wrong head rank")
             out.append({"log2n": lg, "spacing": D, "random_ms": t_rand, "even_ms": t_even,
                         "random_gnodes_per_s": n / t_rand / 1e6, "even_gnodes_per_s": n / t_even / 1e6,
                         "even_speedup": t_rand / t_even})
-            del s_d, r_d, even
+            del s_d, r_d, even, rand
     finally:
         for lg in sizes:
             lrcc.set_plan(lrcc.KIND_LR, lg, lg, rs_level0=base[lg]["rs_level0"])
@@ -919,7 +926,8 @@ def main():
     roofline = None
     level0 = lrcc.get_plan(lrcc.KIND_LR, n_lr)["rs_level0"]
     # bytes the method moves: per element of each ruling-set level, per edge read by a hook pass
-    lr_method = LR_METHOD_FIRST[level0] * n_lr + 44 * sum(lr_stats["splitters"])
+    lr_form = 0 if level0 == 1 and n_lr <= 1 << 24 else level0
+    lr_method = LR_METHOD_FIRST[lr_form] * n_lr + 36 * sum(lr_stats["splitters"])
     cc_method = 16 * cc_stats["edges_read"] + 8 * n_cc * cc_stats["rounds"] + 4 * n_cc
     if "rs_walk0" in phases:
         wt, wl = phases["rs_walk0"]
@@ -930,7 +938,9 @@ def main():
             # one 8-byte reduced-list word per splitter
             alg_bytes, per_elem = 9 * n_lr + 8 * r1, "9 B per element (read succ, write id + chunk header) + 8 B per splitter"
         else:
-            alg_bytes, per_elem = 16 * n_lr + 16 * r1, "16 B per element (read + write back its 8-byte word) + 16 B per splitter"
+            alg_bytes, per_elem = 8 * n_lr + 8 * r1, "8 B per element (read succ, write its record) + 8 B per splitter"
+            if lr_form == 1:
+                alg_bytes, per_elem = 16 * n_lr + 16 * r1, "16 B per element (read + write back its 8-byte word) + 16 B per splitter"
         achieved = alg_bytes / (per_launch_ms / 1e3) / 1e9
         traffic = None
         if NCU_WALK0["walk_sha1"] == walk0_sha1(os.path.join(ROOT, "paper_1002_4482_gb300", "csrc", "lr.cu")) \
@@ -980,7 +990,9 @@ def main():
                        "achieved_gbs": 16 * m_cc / (full_pass_ms / 1e3) / 1e9,
                        "frac_of_hbm": 16 * m_cc / (full_pass_ms / 1e3) / 1e9 / hbm,
                        "ceiling_ms": probe_ms, "frac_of_ceiling": probe_ms / full_pass_ms,
-                       "note": "8 B edge + two 4-byte parent gathers per edge; ceiling: the gather probe (same "
+                       "note": "rule 1 with a launch per pass (plain launches; the step itself runs all passes in one "
+                               "launch, whose filter pass leaves out the gathers its member table answers); 8 B edge + "
+                               "two 4-byte parent gathers per edge; ceiling: the gather probe (same "
                                "edge stream and gathers, no hooking), bound by the SM-to-L2 request port"})
         roofline["other_kernels"] = others
 
@@ -1178,18 +1190,19 @@ def main():
                        "problem_bytes_frac": 8 * n_lr / (lr_ms / 1e3) / 1e9 / hbm if lr_ms else None,
                        "method_bytes_per_node": lr_method / n_lr,
                        "method_bytes_frac": lr_method / (lr_ms / 1e3) / 1e9 / hbm if lr_ms else None,
-                       "method_bytes_note": "first level: " + LR_METHOD_NOTE[level0] + "; each deeper level: "
-                                            "8 B read + 8 B written by the select and the walk, 8 B read + "
-                                            "4 B written by the expand, per element of the level",
+                       "method_bytes_note": "first level: " + LR_METHOD_NOTE[lr_form] + "; each deeper level: "
+                                            "8 B written by the level before, 8 B read + 8 B written by the "
+                                            "walk, 8 B read + 4 B written by the expand, per element of the level",
                        "levels": lr_stats["levels"], "splitters": lr_stats["splitters"]},
                 "cc": {"ms": cc_ms, "medges_per_s": m_cc / cc_ms / 1e3 if cc_ms else None,
                        "problem_bytes_frac": (8 * m_cc + 4 * n_cc) / (cc_ms / 1e3) / 1e9 / hbm if cc_ms else None,
                        "rounds": cc_stats["rounds"], "edges_read": cc_stats["edges_read"],
                        "method_bytes": cc_method,
                        "method_bytes_frac": cc_method / (cc_ms / 1e3) / 1e9 / hbm if cc_ms else None,
-                       "method_bytes_note": "16 B per edge read by a hook pass (8 B of edge, two 4-byte parent "
-                                            "gathers), 8 B per vertex and shortcut pass, 4 B per vertex of init; "
-                                            "R = rounds",
+                       "method_bytes_note": "16 B per edge or kept pair read by a hook pass (8 B of ids, two 4-byte "
+                                            "parent gathers; those that the filter pass's member table answers "
+                                            "are counted too), 8 B per vertex and shortcut pass, 4 B per vertex "
+                                            "of init; R = rounds",
                        "gather_ceiling": {
                            "probe_ms_per_pass": probe_ms, "probe_gedges_per_s": m_cc / probe_ms / 1e6,
                            "edges_read": cc_stats["edges_read"],
@@ -1198,9 +1211,10 @@ def main():
                            "full_pass_ms": full_pass_ms, "full_pass_frac": probe_ms / full_pass_ms,
                            "note": "probe: the hook pass's 16-byte edge stream and two gathers per edge (L1, "
                                    "evict-last) over a 4n-byte table, no hooking (lrcc_gather_probe); ceiling: "
-                                   "every edge the hook passes read, at the probe's rate; frac = ceiling / cc ms; full_pass: the "
-                                   "loop's first pass over all edges alone (plain launches, best of 3), full_pass_frac "
-                                   "= probe / full pass"}},
+                                   "every edge the hook passes read, at the probe's rate; frac = ceiling / cc ms (above 1 "
+                                   "where the member table answers gathers the probe makes); full_pass: the "
+                                   "loop's first pass over all edges alone (plain launches, a launch per pass, best of 3), "
+                                   "full_pass_frac = probe / full pass"}},
                 "phases_ms_per_step": {k: v[0] / args.steps for k, v in phases.items()},
                 "batched": batched, "serving": serving, "cc_families": families, "lr_sweep": sweep,
                 "even_vs_random_splitters": even, "small_configs": small,
