@@ -106,3 +106,28 @@ def test_scan_of_a_list_with_a_detached_cycle(n):
     succ[b] = a
     lrcc.lr_scan(_dev(succ), _dev(np.ones(n, np.int32)), head)
     assert lrcc.last_status() == lrcc.ERR_INVALID_INPUT
+
+
+@pytest.mark.parametrize("n,lists", [((1 << 24) - 32, 1), ((1 << 24) - 16, 1), (1 << 24, 3), ((1 << 24) + 5, 1),
+                                     ((1 << 24) + 5, 20_000), (1_500_000, 1_500_000), (1_500_000, 1_200_000)])
+def test_forests_whose_splitters_jump_by_rulers(n, lists):
+    """Around 2^20 splitters (stratified ones and heads), from where one word of four jumps and the others walk to it."""
+    succ = _forest(n, lists, n + lists)
+    val = np.random.default_rng(n).integers(-(2**31), 2**31, n).astype(np.int32)
+    got = lrcc.lr_scan_forest(_dev(succ), _dev(val))
+    lrcc.check()
+    assert np.array_equal(got.cpu().numpy(), oracle.lr_scan_forest(succ, val))
+
+
+@pytest.mark.parametrize("length", [12_000_000, 64, 40, 24, 9])
+def test_cycles_among_the_rulers_words(length):
+    """A cycle of many splitters, or of a few of which some or none are rulers."""
+    n = 1 << 24
+    order = gen.permutation(n, length)
+    succ = np.empty(n, np.int32)
+    succ[order[:-1]] = order[1:]
+    succ[order[-1]] = -1
+    for start in range(0, 1 if length > 1000 else 64 * length, length):   # many short ones, or one long one
+        succ[order[start + length - 1]] = order[start]
+    lrcc.lr_scan_forest(_dev(succ), _dev(np.ones(n, np.int32)))
+    assert lrcc.last_status() == lrcc.ERR_INVALID_INPUT
