@@ -639,7 +639,7 @@ __global__ void seg_control(DevCtl* ctl, cudaGraphConditionalHandle h, int cap, 
         record_error(ctl, LRCC_ERR_NOT_CONVERGED, r);
         cont = 0;
     }
-    if (ctl->status) cont = 0;
+    if (ctl->failed) cont = 0;
     ctl->cc_stop = !cont;
     // next pass: the active buffer this pass filled (from the second pass on)
     const int sel = ctl->cc_src;
@@ -664,7 +664,7 @@ __global__ void seg_control_host(DevCtl* ctl, int cap, bool compacting) {
         record_error(ctl, LRCC_ERR_NOT_CONVERGED, r);
         cont = 0;
     }
-    if (ctl->status) cont = 0;
+    if (ctl->failed) cont = 0;
     ctl->cc_stop = !cont;
     const int sel = ctl->cc_src;
     const int out_sel = sel == 1 ? 2 : 1;

@@ -308,7 +308,7 @@ __device__ __forceinline__ void next_edges(DevCtl* ctl, bool compacting) {
 }
 
 // Loop control on the device: continue while the last hook pass joined
-// something, the round cap is not reached and no error was recorded.
+// something, the round cap is not reached and this call recorded no error.
 __global__ void cc_control(DevCtl* ctl, cudaGraphConditionalHandle h, int cap, bool compacting) {
     const int r = ++ctl->rounds;
     const int f = ctl->flag;
@@ -318,7 +318,7 @@ __global__ void cc_control(DevCtl* ctl, cudaGraphConditionalHandle h, int cap, b
         record_error(ctl, LRCC_ERR_NOT_CONVERGED, r);
         cont = 0;
     }
-    if (ctl->status) cont = 0;
+    if (ctl->failed) cont = 0;
     next_edges(ctl, compacting);
     ctl->cc_stop = !cont;
     cudaGraphSetConditional(h, cont);
@@ -334,7 +334,7 @@ __global__ void cc_control_host(DevCtl* ctl, int cap, bool compacting) {
         record_error(ctl, LRCC_ERR_NOT_CONVERGED, r);
         cont = 0;
     }
-    if (ctl->status) cont = 0;
+    if (ctl->failed) cont = 0;
     next_edges(ctl, compacting);
     ctl->cc_stop = !cont;
     ctl->pad[0] = cont;

@@ -123,7 +123,8 @@ __global__ void __launch_bounds__(GANG_THREADS, 1) cc_filter_kernel(const __grid
     extern __shared__ __align__(16) unsigned char s_table[];
     __shared__ int s_flag;
     __shared__ uint64_t s_hook[HOOK_SLOTS];
-    if (ctl->status == LRCC_ERR_TIMEOUT || (P.only >= 0 && P.giant[1] != P.only)) return;
+    // gave_up first: the sample's launch has then written neither P.giant nor P.left
+    if (ctl->gave_up || (P.only >= 0 && P.giant[1] != P.only)) return;
     for (int h = threadIdx.x; h < HOOK_SLOTS; h += GANG_THREADS) s_hook[h] = ~0ull;
     Gang G{gc, &gc->arrived[1], (int)gridDim.x, (int)blockIdx.x, 0, ctl, &s_flag};
     GangWork<VEC> w(P, G, ctl, s_hook, ctl->rounds, ctl->edges_read);

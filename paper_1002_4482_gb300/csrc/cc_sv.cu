@@ -125,7 +125,7 @@ __global__ void sv_control(DevCtl* ctl, cudaGraphConditionalHandle h, int cap) {
         record_error(ctl, LRCC_ERR_NOT_CONVERGED, r);
         cont = 0;
     }
-    if (ctl->status) cont = 0;
+    if (ctl->failed) cont = 0;
     cudaGraphSetConditional(h, cont);
 }
 
@@ -137,7 +137,7 @@ __global__ void sv_control_host(DevCtl* ctl, int cap) {
         record_error(ctl, LRCC_ERR_NOT_CONVERGED, r);
         cont = 0;
     }
-    if (ctl->status) cont = 0;
+    if (ctl->failed) cont = 0;
     ctl->pad[0] = cont;
 }
 

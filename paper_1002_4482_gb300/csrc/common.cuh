@@ -13,7 +13,8 @@ namespace lrcc {
 // Per-workspace control block in device memory. Zeroed before every call
 // except where noted.
 struct DevCtl {
-    int status;          // first device-detected error (lrcc_status), 0 = none
+    int status;          // first device-detected error (lrcc_status), 0 = none; kept until it is read
+                         // by the caller, so no kernel decides by it (failed is the call's own)
     int flag;            // component loop: some edge joined two roots this pass
     int rounds;          // component loop: hook passes so far
     int jump_rounds;     // pointer-jumping rounds (stats)
@@ -31,6 +32,8 @@ struct DevCtl {
     int seg_next_v;      // batched union path: next vertex slice of the current shortcut
     int scan_bad;        // weighted ranks: the values are outside the supported range; skip the work
     int ff_extra;        // forest ranks: list heads that became extra first-level splitters
+    int failed;          // an error was recorded by this call (status also holds those of earlier calls)
+    int gave_up;         // a gang's barrier gave up in this call: what its launch left is not to be read
     int pad[1];
     unsigned long long scan_total;   // weighted ranks: sum of the values
     unsigned long long edges_read;   // component loop: edges read by all hook passes
@@ -40,6 +43,7 @@ struct DevCtl {
 };
 
 __device__ __forceinline__ void record_error(DevCtl* c, int code, int where = -1) {
+    c->failed = 1;
     if (atomicCAS(&c->status, 0, code) == 0) c->err_where = where;
 }
 
