@@ -39,6 +39,7 @@ struct DevCtl {
     unsigned long long edges_read;   // component loop: edges read by all hook passes
     unsigned long long links, named, visited;   // weighted ranks: elements with a successor, elements
                                                 // named by one, elements the walks reached
+    unsigned long long chased[8];    // weighted ranks: elements of each deeper level its walks reached
     alignas(128) unsigned gang[64];  // gang.cuh: the GangCtl of a launch that is one gang
 };
 

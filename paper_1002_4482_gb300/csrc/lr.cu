@@ -265,42 +265,63 @@ struct CycleGuard {
 // in a pass of their own and overwrote R in place; a store to a line that was
 // just read costs the L2 far more than a store elsewhere (read-then-store runs
 // at 29-65 G/s, reads alone at 290, stores alone at 180-206).
+//
+// COUNT (weighted ranks, whose sums say nothing about how many elements they
+// cover): the elements the walks reached are added up in *chased, which rs_expand
+// compares with the level's size. That is enough: the level above is one list
+// holding all its elements (its own count, or the last level's), so the walks of
+// this one end at different splitters, cannot meet, and reach each element at
+// most once.
+static_assert(sizeof(DevCtl::chased) >= MAX_LEVELS * sizeof(unsigned long long), "a count for every level");
+template <bool COUNT>
 __global__ void __launch_bounds__(BLOCK)
     rs_chase(const uint64_t* __restrict__ R, uint32_t nl, uint64_t* __restrict__ P, uint64_t* __restrict__ Rout,
-             uint32_t r, int logD, uint32_t seed, uint32_t fixed, DevCtl* ctl) {
+             uint32_t r, int logD, uint32_t seed, uint32_t fixed, unsigned long long* chased, DevCtl* ctl) {
     if (ctl->scan_bad) return;
     const uint32_t j = blockIdx.x * BLOCK + threadIdx.x;
-    if (j >= r) return;
     const uint32_t D = 1u << logD;
     auto offset = [&](uint32_t b) {
         return b == 0 ? 0u : block_offset(b, min(D, nl - (b << logD)), seed);
     };
-    const uint32_t start = (j << logD) + offset(j);
-    if (start >= fixed && start - fixed >= (uint32_t)ctl->ff_extra) {   // an extra owner nobody took
-        Rout[j] = pack(NIL, 0);
+    // walks sublist j; the elements it reached
+    auto walk = [&]() -> uint32_t {
+        const uint32_t start = (j << logD) + offset(j);
+        if (start >= fixed && start - fixed >= (uint32_t)ctl->ff_extra) {   // an extra owner nobody took
+            Rout[j] = pack(NIL, 0);
+            return 0;
+        }
+        uint64_t w = R[start];
+        P[start] = pack(0, j);
+        uint32_t cur = lo32(w), pre = hi32(w), steps = 1;
+        CycleGuard guard(start);
+        uint32_t next = NIL;
+        while (cur != NIL) {
+            if (cur >= nl || guard.seen(cur)) {
+                record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)cur);
+                break;
+            }
+            w = R[cur];
+            const uint32_t b = cur >> logD;
+            if ((cur & (D - 1)) == offset(b)) {
+                next = b;
+                break;
+            }
+            P[cur] = pack(pre, j);
+            pre += hi32(w);
+            if (COUNT) ++steps;
+            cur = lo32(w);
+        }
+        Rout[j] = pack(next, pre);
+        return steps;
+    };
+    if (!COUNT) {
+        if (j < r) walk();
         return;
     }
-    uint64_t w = R[start];
-    P[start] = pack(0, j);
-    uint32_t cur = lo32(w), pre = hi32(w);
-    CycleGuard guard(start);
-    uint32_t next = NIL;
-    while (cur != NIL) {
-        if (cur >= nl || guard.seen(cur)) {
-            record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)cur);
-            break;
-        }
-        w = R[cur];
-        const uint32_t b = cur >> logD;
-        if ((cur & (D - 1)) == offset(b)) {
-            next = b;
-            break;
-        }
-        P[cur] = pack(pre, j);
-        pre += hi32(w);
-        cur = lo32(w);
-    }
-    Rout[j] = pack(next, pre);
+    unsigned long long reached = j < r ? walk() : 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) reached += __shfl_xor_sync(0xffffffffu, reached, o);
+    if ((threadIdx.x & 31) == 0 && reached) atomicAdd(chased, reached);
 }
 
 // Sublist walk (RS3). Each thread keeps K walks in flight so that K
@@ -1055,16 +1076,18 @@ __global__ void __launch_bounds__(BLOCK)
     }
 }
 
-// Expand at level >= 1: S[c] = S_next[owner] - prefix (RS5).
+// Expand at level >= 1: S[c] = S_next[owner] - prefix (RS5). Weighted ranks pass
+// *chased, the elements the level's walks reached: all r of one list.
 __global__ void __launch_bounds__(BLOCK)
     rs_expand(const uint64_t* __restrict__ P, uint32_t r, const int32_t* __restrict__ Snext, uint32_t rnext,
-              int32_t* __restrict__ S, DevCtl* ctl) {
+              int32_t* __restrict__ S, const unsigned long long* chased, DevCtl* ctl) {
     if (ctl->scan_bad) return;
+    if (chased && blockIdx.x == 0 && threadIdx.x == 0 && *chased != r) record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
     for (uint32_t c = blockIdx.x * BLOCK + threadIdx.x; c < r; c += gridDim.x * BLOCK) {
         const uint64_t p = P[c];
         // an element no walk reached holds an old word: its owner is checked, so
-        // that a malformed input can only give wrong values (the last level has
-        // recorded it), never an access outside Snext
+        // that a malformed input can only give wrong values, never an access outside
+        // Snext (it is recorded by the last level's total, or by the count above)
         S[c] = hi32(p) < rnext ? (int32_t)((uint32_t)Snext[hi32(p)] - lo32(p)) : 0;
     }
 }
@@ -2468,8 +2491,13 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         const uint32_t seed = mix32(seed0 + 0x9E3779B9u * (uint32_t)l);
         const unsigned g = (unsigned)((L.size[l + 1] + BLOCK - 1) / BLOCK);
         phase_begin(c, s);
-        rs_chase<<<g, BLOCK, 0, s>>>(R(l), (uint32_t)L.size[l], P(l), R(l + 1), (uint32_t)L.size[l + 1], L.logD[l], seed,
-                                     l == 1 && L.direct ? (uint32_t)L.fixed : 0xFFFFFFFFu, ctl);
+        const uint32_t fixed = l == 1 && L.direct ? (uint32_t)L.fixed : 0xFFFFFFFFu;
+        if (val)
+            rs_chase<true><<<g, BLOCK, 0, s>>>(R(l), (uint32_t)L.size[l], P(l), R(l + 1), (uint32_t)L.size[l + 1],
+                                               L.logD[l], seed, fixed, &ctl->chased[l], ctl);
+        else
+            rs_chase<false><<<g, BLOCK, 0, s>>>(R(l), (uint32_t)L.size[l], P(l), R(l + 1), (uint32_t)L.size[l + 1],
+                                                L.logD[l], seed, fixed, nullptr, ctl);
         phase_end(c, s, PH_WALK);
     }
     {
@@ -2485,7 +2513,8 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     for (int l = L.levels - 1; l >= 1; --l) {
         const int g = stream_grid(c, L.size[l], (const void*)rs_expand);
         phase_begin(c, s);
-        rs_expand<<<g, BLOCK, 0, s>>>(P(l), (uint32_t)L.size[l], S(l + 1), (uint32_t)L.size[l + 1], S(l), ctl);
+        rs_expand<<<g, BLOCK, 0, s>>>(P(l), (uint32_t)L.size[l], S(l + 1), (uint32_t)L.size[l + 1], S(l),
+                                     val ? &ctl->chased[l] : nullptr, ctl);
         phase_end(c, s, PH_EXPAND);
     }
     if (U && L.readonly) {
