@@ -49,14 +49,22 @@ constexpr int64_t CC_LARGE = int64_t(1) << 15;   // graphs above this many verti
 constexpr int SEG_BLOCK = 256;
 
 // Order instances by size class (floor(log2(size - 1))), largest first; order[count]
-// = how many have more than SMEM_ELEMS elements (they come first).
+// = how many have more than SMEM_ELEMS elements (they come first). The kernels
+// that rank lists (heads given) trust the offsets: from 0, non-decreasing, within
+// the `total` elements of the arrays and the workspace. Others are reported, and
+// no list is ranked (scan_bad).
 __global__ void __launch_bounds__(1024)
     batch_order(const int64_t* __restrict__ off_a, const int64_t* __restrict__ off_b, const int32_t* heads,
-                int64_t count, int32_t* __restrict__ order, DevCtl* ctl) {
+                int64_t count, int64_t total, int32_t* __restrict__ order, DevCtl* ctl) {
     __shared__ int s_hist[NCLASS];
     __shared__ int s_start[NCLASS];
     for (int t = threadIdx.x; t < NCLASS; t += blockDim.x) s_hist[t] = 0;
-    __syncthreads();
+    bool ok = !heads || threadIdx.x > 0 || (off_a[0] == 0 && off_a[count] <= total);
+    for (int64_t k = threadIdx.x; heads && k < count; k += blockDim.x) ok &= off_a[k] <= off_a[k + 1];
+    if (!__syncthreads_and(ok) && threadIdx.x == 0) {
+        record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
+        ctl->scan_bad = 1;
+    }
     // size class of instance k, -> class 0 when its offsets or head are invalid
     auto klass = [&](int64_t k) -> int {
         const int64_t na = off_a[k + 1] - off_a[k];
@@ -216,6 +224,7 @@ __global__ void __launch_bounds__(T)
     uint64_t* words = reinterpret_cast<uint64_t*>(lb_raw);
     uint2* sub = reinterpret_cast<uint2*>(lb_raw + sizeof(uint64_t) * CAP);
     __shared__ int s_k, s_work;
+    if (ctl->scan_bad) return;
     const int64_t first = LARGE ? 0 : *split, last = LARGE ? *split : count;
     for (;;) {
         const int64_t q = take_instance(&s_k, LARGE ? &ctl->batch_next : &ctl->seg_next, last - first);
@@ -741,7 +750,7 @@ lrcc_status lr_batched_run(Ctx* c, const int32_t* succ, const int64_t* off, cons
     int32_t* order = reinterpret_cast<int32_t*>(static_cast<char*>(c->ws) +
                                                 align_up(sizeof(uint64_t) * (size_t)std::max<int64_t>(total_nodes, 1), 256));
     phase_begin(c, s);
-    batch_order<<<1, 1024, 0, s>>>(off, nullptr, heads, count, order, c->ctl);
+    batch_order<<<1, 1024, 0, s>>>(off, nullptr, heads, count, total_nodes, order, c->ctl);
     phase_end(c, s, PH_BATCH_PREP);
     auto small_k = lr_batch_kernel<BT, SMEM_ELEMS, false>;
     auto large_k = lr_batch_kernel<BT_LARGE, SMEM_ELEMS_LARGE, true>;
@@ -786,7 +795,7 @@ lrcc_status cc_batched_run(Ctx* c, const int32_t* src, const int32_t* dst, const
     }
 
     phase_begin(c, s);
-    batch_order<<<1, 1024, 0, s>>>(voff, eoff, nullptr, count, order, c->ctl);
+    batch_order<<<1, 1024, 0, s>>>(voff, eoff, nullptr, count, 0, order, c->ctl);
     large_prep<<<1, 1024, 0, s>>>(eoff, voff, count, L);
     phase_end(c, s, PH_BATCH_PREP);
 

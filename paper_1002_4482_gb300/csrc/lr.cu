@@ -1512,6 +1512,7 @@ constexpr int BL_TILE = BLOCK * 16;
 __global__ void __launch_bounds__(BLOCK)
     bl_gsucc(const int32_t* __restrict__ succ, const int64_t* __restrict__ off, int64_t K, int64_t n,
              int32_t* __restrict__ gsucc, DevCtl* ctl) {
+    if (ctl->scan_bad) return;
     constexpr int PER = BL_TILE / BLOCK;
     __shared__ int64_t s_k;
     const uint64_t pol = policy_evict_first();
@@ -1543,8 +1544,14 @@ __global__ void __launch_bounds__(BLOCK)
     }
 }
 
+// A value of the read-only walk's work counter at which it finds no splitter left.
+constexpr int WALK_OFF = 0x7F000000;
+
 // One block: the first list's head (head_dev[0]) and the head splitter of every
-// list; head_dev[1] = the heads that became extra splitters.
+// list; head_dev[1] = the heads that became extra splitters. The kernels after it
+// trust the offsets, so they are checked here: from 0, non-decreasing, up to the n
+// elements the call names. Others are reported and every later kernel leaves the
+// arrays alone (scan_bad, and no splitters for the read-only walk).
 __global__ void __launch_bounds__(1024)
     bl_heads(const int64_t* __restrict__ off, const int32_t* __restrict__ heads, int64_t K, int64_t n, int logD,
              int64_t nb, uint32_t seed, int32_t* __restrict__ head_spl, int32_t* __restrict__ extra_elem,
@@ -1552,6 +1559,17 @@ __global__ void __launch_bounds__(1024)
     __shared__ int64_t s_first;
     __shared__ int s_warp[32];
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    bool ok = t > 0 || (off[0] == 0 && off[K] == n);
+    for (int64_t k = t; k < K; k += 1024) ok &= off[k] <= off[k + 1];
+    if (!__syncthreads_and(ok)) {
+        if (t == 0) {
+            record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
+            ctl->scan_bad = 1;
+            ctl->work[0] = WALK_OFF;
+            head_dev[0] = head_dev[1] = 0;
+        }
+        return;
+    }
     if (t == 0) {
         int64_t k0 = 0;
         while (k0 < K && off[k0 + 1] == off[k0]) ++k0;
@@ -1637,6 +1655,7 @@ __global__ void __launch_bounds__(1024)
 __global__ void __launch_bounds__(BLOCK)
     bl_link(uint64_t* __restrict__ R1, int64_t r1_max, const int64_t* __restrict__ off, int64_t K,
             const int32_t* __restrict__ head_spl, Level0 L0, DevCtl* ctl) {
+    if (ctl->scan_bad) return;
     const int64_t gh = *L0.head_dev;
     L0.bh = gh >> L0.logD;
     L0.head_off = (uint32_t)(gh - (L0.bh << L0.logD));
@@ -1664,7 +1683,9 @@ __global__ void __launch_bounds__(BLOCK)
 // correction is taken once per first-level splitter, from its suffix sum,
 // before the scatter turns suffix sums into ranks.
 __global__ void __launch_bounds__(BLOCK)
-    bl_adjust(int32_t* __restrict__ S1, const int64_t* __restrict__ off, int64_t K, int64_t n, Level0 L0) {
+    bl_adjust(int32_t* __restrict__ S1, const int64_t* __restrict__ off, int64_t K, int64_t n, Level0 L0,
+              const DevCtl* ctl) {
+    if (ctl->scan_bad) return;
     const int64_t gh = *L0.head_dev;
     L0.bh = gh >> L0.logD;
     L0.head_off = (uint32_t)(gh - (L0.bh << L0.logD));
@@ -1691,6 +1712,7 @@ __global__ void __launch_bounds__(LISTS_BLOCK)
     rs_walk_lists(const int32_t* __restrict__ succ, uint32_t* __restrict__ rec, Level0 L0,
                   const int64_t* __restrict__ off, int64_t K, const int32_t* __restrict__ head_spl, int pbits,
                   int extras, uint64_t* __restrict__ R1, DevCtl* ctl) {
+    if (ctl->scan_bad) return;
     const int64_t gh = L0.head_dev[0];
     L0.bh = gh >> L0.logD;
     L0.head_off = (uint32_t)(gh - (L0.bh << L0.logD));
@@ -1740,11 +1762,12 @@ __global__ void __launch_bounds__(LISTS_BLOCK)
 
 // Records -> local ranks: the rank along all lists less the elements of the
 // later ones. A block takes one stretch of the elements and every thread keeps
-// the list it is in.
+// the list it is in (the last one ends at n: bl_heads has checked the offsets).
 template <bool VEC>
 __global__ void __launch_bounds__(BLOCK)
     rs_expand_lists(int32_t* rank, int64_t n, const int32_t* __restrict__ S1, uint32_t r1, int pbits,
-                    const int64_t* __restrict__ off, int64_t K) {
+                    const int64_t* __restrict__ off, int64_t K, const DevCtl* ctl) {
+    if (ctl->scan_bad) return;
     const uint32_t mask = (1u << pbits) - 1;
     const int64_t per = ((n + gridDim.x - 1) / gridDim.x + 4 * BLOCK - 1) / (4 * BLOCK) * (4 * BLOCK);
     const int64_t b = per * blockIdx.x, e = min(n, b + per);
@@ -2373,9 +2396,9 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     if (U) {
         const int g = stream_grid(c, (n + BL_TILE - 1) / BL_TILE * BLOCK, (const void*)bl_gsucc);
         phase_begin(c, s);
-        if (L.readonly) bl_gsucc<<<g, BLOCK, 0, s>>>(succ, U->off, U->K, n, U->gsucc, ctl);
         bl_heads<<<1, 1024, 0, s>>>(U->off, U->heads, U->K, n, L0.logD, L0.nb, seed0, U->head_spl, U->extra_elem,
                                     U->head_dev, ctl);
+        if (L.readonly) bl_gsucc<<<g, BLOCK, 0, s>>>(succ, U->off, U->K, n, U->gsucc, ctl);
         phase_end(c, s, PH_BATCH_PREP);
         if (L.readonly) succ = U->gsucc;
         L0.head_dev = U->head_dev;
@@ -2519,7 +2542,8 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     }
     if (U && L.readonly) {
         phase_begin(c, s);
-        bl_adjust<<<stream_grid(c, L.size[1], (const void*)bl_adjust), BLOCK, 0, s>>>(S(1), U->off, U->K, n, L0);
+        bl_adjust<<<stream_grid(c, L.size[1], (const void*)bl_adjust), BLOCK, 0, s>>>(S(1), U->off, U->K, n, L0,
+                                                                                       ctl);
         phase_end(c, s, PH_BATCH_PREP);
     }
     if (L.readonly) {
@@ -2546,8 +2570,8 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         const void* k = v ? (const void*)rs_expand_lists<true> : (const void*)rs_expand_lists<false>;
         const int g = stream_grid(c, groups, k);
         phase_begin(c, s);
-        if (v) rs_expand_lists<true><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off, U->K);
-        else rs_expand_lists<false><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off, U->K);
+        if (v) rs_expand_lists<true><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off, U->K, ctl);
+        else rs_expand_lists<false><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off, U->K, ctl);
         phase_end(c, s, PH_EXPAND0);
     } else if (L.direct) {
         const bool v = aligned16(rank);
