@@ -42,15 +42,23 @@ __device__ __forceinline__ bool batch_graph(const int64_t* eoff, const int64_t* 
 // Orders the graphs by size, largest first, those for gangs in front, and
 // chooses the gang size: as many gangs as the largest graph leaves room for
 // (the call lasts at least as long as that graph on its gang), of at least 8
-// blocks. One block.
+// blocks. One block. Offsets that do not start at 0, that decrease or that pass
+// total_edges are reported and no graph is labelled (scan_bad): the labels are a
+// graph's parents in local ids, and two gangs on overlapping ones would follow
+// each other's.
 __global__ void __launch_bounds__(1024)
-    cc_batch_order(const int64_t* __restrict__ eoff, const int64_t* __restrict__ voff, int64_t count, int blocks,
-                   int32_t* __restrict__ order, BatchPlan* plan, DevCtl* ctl) {
+    cc_batch_order(const int64_t* __restrict__ eoff, const int64_t* __restrict__ voff, int64_t count,
+                   int64_t total_edges, int blocks, int32_t* __restrict__ order, BatchPlan* plan, DevCtl* ctl) {
     __shared__ int s_hist[CLASSES], s_start[CLASSES];
     __shared__ unsigned long long s_total, s_most;
     for (int t = threadIdx.x; t < CLASSES; t += blockDim.x) s_hist[t] = 0;
     if (threadIdx.x == 0) s_total = s_most = 0;
-    __syncthreads();
+    bool ok = threadIdx.x > 0 || (voff[0] == 0 && eoff[0] == 0 && eoff[count] <= total_edges);
+    for (int64_t k = threadIdx.x; k < count; k += blockDim.x) ok &= voff[k] <= voff[k + 1] && eoff[k] <= eoff[k + 1];
+    if (!__syncthreads_and(ok) && threadIdx.x == 0) {
+        record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
+        ctl->scan_bad = 1;
+    }
     auto klass = [&](int64_t k, unsigned long long* work) {
         int64_t n, m;
         *work = 0;
@@ -125,6 +133,7 @@ __global__ void __launch_bounds__(GANG_THREADS, 1)
     __shared__ int s_flag;
     __shared__ uint64_t s_hook[HOOK_SLOTS];
     __shared__ GangParams s_P;
+    if (ctl->scan_bad) return;
     const int gang = plan->gang, gangs = (int)gridDim.x / gang, id = (int)blockIdx.x / gang;
     if (id >= gangs) return;
     GangCtl* gc = gcs + id;
@@ -179,6 +188,7 @@ __global__ void __launch_bounds__(SMALL_THREADS)
     extern __shared__ int small_p[];
     __shared__ int s_q;
     volatile int* p = small_p;
+    if (ctl->scan_bad) return;
     const int first = plan->large;
     for (;;) {
         __syncthreads();   // the forest of the graph before is written out
@@ -251,7 +261,7 @@ lrcc_status cc_batch_gang_run(Ctx* c, const int32_t* src, const int32_t* dst, co
     const int blocks = c->sms;
     if (cudaMemsetAsync(gcs, 0, gcs_bytes, s) != cudaSuccess) return LRCC_ERR_CUDA;
     phase_begin(c, s);
-    cc_batch_order<<<1, 1024, 0, s>>>(eoff, voff, count, blocks, order, plan, c->ctl);
+    cc_batch_order<<<1, 1024, 0, s>>>(eoff, voff, count, total_edges, blocks, order, plan, c->ctl);
     phase_end(c, s, PH_BATCH_PREP);
     phase_begin(c, s);
     void* args[] = {&src, &dst, &eoff, &voff, &order, &plan, &gcs, &pairs, &pair_count, &label, &c->ctl};
