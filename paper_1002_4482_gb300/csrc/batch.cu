@@ -30,6 +30,7 @@
 #include "cc_device.cuh"
 #include "common.cuh"
 #include "internal.h"
+#include "list_block.cuh"
 
 namespace lrcc {
 
@@ -59,16 +60,13 @@ __global__ void __launch_bounds__(1024)
     __shared__ int s_hist[NCLASS];
     __shared__ int s_start[NCLASS];
     for (int t = threadIdx.x; t < NCLASS; t += blockDim.x) s_hist[t] = 0;
+    __syncthreads();
     bool ok = !heads || threadIdx.x > 0 || (off_a[0] == 0 && off_a[count] <= total);
-    for (int64_t k = threadIdx.x; heads && k < count; k += blockDim.x) ok &= off_a[k] <= off_a[k + 1];
-    if (!__syncthreads_and(ok) && threadIdx.x == 0) {
-        record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
-        ctl->scan_bad = 1;
-    }
     // size class of instance k, -> class 0 when its offsets or head are invalid
     auto klass = [&](int64_t k) -> int {
         const int64_t na = off_a[k + 1] - off_a[k];
         bool bad = na < 0 || na > 0x7FFFFFFELL || (k == 0 && off_a[0] != 0);
+        ok &= na >= 0 || !heads;
         int64_t size = na;
         if (off_b) {
             const int64_t nbv = off_b[k + 1] - off_b[k];
@@ -83,8 +81,12 @@ __global__ void __launch_bounds__(1024)
         return size <= 1 ? 0 : min(64 - __clzll((unsigned long long)(size - 1)), NCLASS - 1);
     };
     for (int64_t k = threadIdx.x; k < count; k += blockDim.x) atomicAdd(&s_hist[klass(k)], 1);
-    __syncthreads();
+    const bool sound = __syncthreads_and(ok);
     if (threadIdx.x == 0) {
+        if (!sound) {
+            record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
+            ctl->scan_bad = 1;
+        }
         int run = 0;
         for (int c = NCLASS - 1; c >= 0; --c) {
             s_start[c] = run;
@@ -94,13 +96,6 @@ __global__ void __launch_bounds__(1024)
     }
     __syncthreads();
     for (int64_t k = threadIdx.x; k < count; k += blockDim.x) order[atomicAdd(&s_start[klass(k)], 1)] = (int32_t)k;
-}
-
-__device__ __forceinline__ int64_t take_instance(int* s_k, int* next, int64_t count) {
-    __syncthreads();
-    if (threadIdx.x == 0) *s_k = atomicAdd(next, 1);
-    __syncthreads();
-    return *s_k < count ? *s_k : -1;
 }
 
 // ----------------------------------------------------------------- lists
@@ -122,91 +117,6 @@ __device__ void list_in_smem(const int32_t* succ, int n, int head, int32_t* rank
     if (threadIdx.x == 0 && !whole) record_error(ctl, LRCC_ERR_INVALID_INPUT, head);
 #pragma unroll 4
     for (int i = threadIdx.x; i < n; i += T) rank[i] = block_rank_sum<T>(W[i], res) - 1;
-}
-
-// Rank one larger list with a ruling set inside the block; W is the list's
-// slice of the 8-byte word workspace, R the splitters' packed words in shared
-// memory (next splitter, sublist length; before the walk: successor, 1).
-template <int T, int CAP>
-__device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_t* rank, uint64_t* W,
-                                uint64_t* R, uint2* sub, int* s_work, uint32_t seed, int min_logD, DevCtl* ctl) {
-    // spacing: a power of two, at least 2^min_logD, with at most CAP splitters
-    int logD = max(2, min_logD);
-    while (((n + (int64_t(1) << logD) - 1) >> logD) > CAP) ++logD;
-    const int64_t D = int64_t(1) << logD;
-    const int r = (int)((n + D - 1) >> logD);
-    const int64_t bh = head >> logD;
-    const uint32_t head_off = (uint32_t)(head - (bh << logD));
-    // select (RS1+RS2): walk words, and each splitter's successor in R[j]
-    for (int64_t i = threadIdx.x; i < n; i += T) {
-        const int s = succ[i];
-        const bool tail = (s == -1) | (s == i);
-        const bool bad = !tail && (s < 0 || s >= n);
-        if (bad) record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)i);
-        const uint32_t nx = (tail || bad) ? NIL : (uint32_t)s;
-        const int64_t b = i >> logD;
-        const uint32_t size = (uint32_t)min(D, n - (b << logD));
-        const uint32_t off = b == bh ? head_off : block_offset((uint32_t)b, size, seed);
-        if ((uint32_t)(i - (b << logD)) == off) {
-            const int j = (int)(b >= bh ? b - bh : b - bh + r);
-            W[i] = pack(nx | SPL, (uint32_t)j);
-            R[j] = pack(nx, 1);
-        } else {
-            W[i] = pack(nx, 1);
-        }
-    }
-    if (threadIdx.x == 0) *s_work = 0;
-    __syncthreads();
-    // walk (RS3): one sublist per thread at a time, claimed from a shared counter
-    for (;;) {
-        const int j = atomicAdd(s_work, 1);
-        if (j >= r) break;
-        uint32_t cur = lo32(R[j]);
-        uint32_t pre = 1;
-        uint32_t next = NIL;
-        int64_t steps = 0;
-        while (cur != NIL) {
-            if (cur >= n) {
-                record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)cur);
-                break;
-            }
-            const uint64_t w = W[cur];
-            const uint32_t lo = lo32(w), hi = hi32(w);
-            if (lo & SPL) {
-                next = hi;
-                break;
-            }
-            if ((hi & VIS) || ++steps > n) {
-                record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)cur);
-                break;
-            }
-            W[cur] = pack(pre, (uint32_t)j | VIS);
-            pre += hi;
-            cur = lo;
-        }
-        R[j] = pack(next == NIL ? BR_NIL : next, pre);
-    }
-    // rank the splitters (RS4) in shared memory; their suffix sums replace their words
-    bool whole;
-    const uint2* res = block_rank<T>(R, sub, r, 0, seed, &whole, ctl);
-    if (threadIdx.x == 0 && (!whole || (int64_t)res[0].y != n)) record_error(ctl, LRCC_ERR_INVALID_INPUT, -3);
-    for (int j = threadIdx.x; j < r; j += T) R[j] = (uint64_t)(uint32_t)block_rank_sum<T>(R[j], res);
-    __syncthreads();
-    // expand (RS5)
-    for (int64_t i = threadIdx.x; i < n; i += T) {
-        const uint64_t w = W[i];
-        const uint32_t lo = lo32(w), hi = hi32(w);
-        int out;
-        if (lo & SPL) {
-            out = (int)lo32(R[hi]) - 1;
-        } else if (hi & VIS) {
-            out = (int)lo32(R[hi & ~VIS]) - (int)lo - 1;
-        } else {
-            record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)i);
-            out = -1;
-        }
-        rank[i] = out;
-    }
 }
 
 // Lists of at most CAP elements in shared memory, larger ones by a ruling set

@@ -1559,17 +1559,8 @@ __global__ void __launch_bounds__(1024)
     __shared__ int64_t s_first;
     __shared__ int s_warp[32];
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    bool ok = t > 0 || (off[0] == 0 && off[K] == n);
+    bool ok = t != 32 || (off[0] == 0 && off[K] == n);
     for (int64_t k = t; k < K; k += 1024) ok &= off[k] <= off[k + 1];
-    if (!__syncthreads_and(ok)) {
-        if (t == 0) {
-            record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
-            ctl->scan_bad = 1;
-            ctl->work[0] = WALK_OFF;
-            head_dev[0] = head_dev[1] = 0;
-        }
-        return;
-    }
     if (t == 0) {
         int64_t k0 = 0;
         while (k0 < K && off[k0 + 1] == off[k0]) ++k0;
@@ -1582,7 +1573,15 @@ __global__ void __launch_bounds__(1024)
         }
         *head_dev = gh;
     }
-    __syncthreads();
+    if (!__syncthreads_and(ok)) {
+        if (t == 0) {
+            record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
+            ctl->scan_bad = 1;
+            ctl->work[0] = WALK_OFF;
+            head_dev[0] = head_dev[1] = 0;
+        }
+        return;
+    }
     const int64_t k0 = s_first;
     const int64_t gh0 = *head_dev;
     const int64_t D = int64_t(1) << logD;
