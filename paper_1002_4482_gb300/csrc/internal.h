@@ -94,6 +94,7 @@ struct BatchUnion {
     int32_t* head_spl = nullptr;
     int32_t* extra_elem = nullptr;
     int64_t* head_dev = nullptr;
+    bool again = false;   // ranked one by one when that fails together; elements may follow the last list
 };
 int rs_walk_grid(Ctx* c, const Plan& p);
 // The same grid for the current device without a workspace (152 x 8 when no

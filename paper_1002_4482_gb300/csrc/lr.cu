@@ -24,6 +24,7 @@
 #include "common.cuh"
 #include "gang.cuh"
 #include "internal.h"
+#include "list_block.cuh"
 
 namespace lrcc {
 
@@ -101,8 +102,9 @@ __global__ void __launch_bounds__(FINAL_THREADS, 1)
 // reached `visited` elements (0: walks that mark what they visit).
 __global__ void __launch_bounds__(FINAL_THREADS, 1)
     rs_final_kernel(const uint64_t* __restrict__ R, int r, int fixed, int32_t* __restrict__ S, int64_t expect,
-                    unsigned long long visited, uint32_t seed, DevCtl* ctl) {
+                    unsigned long long visited, const int64_t* expect_dev, uint32_t seed, DevCtl* ctl) {
     if (ctl->scan_bad) return;
+    if (expect_dev) expect = *expect_dev;
     if (fixed < r) r = min(r, fixed + ctl->ff_extra);   // extra owners in use (rs_walk_direct)
     extern __shared__ __align__(16) unsigned char br_raw[];
     uint2* sub = reinterpret_cast<uint2*>(br_raw);
@@ -1548,19 +1550,22 @@ __global__ void __launch_bounds__(BLOCK)
 constexpr int WALK_OFF = 0x7F000000;
 
 // One block: the first list's head (head_dev[0]) and the head splitter of every
-// list; head_dev[1] = the heads that became extra splitters. The kernels after it
-// trust the offsets, so they are checked here: from 0, non-decreasing, up to the n
-// elements the call names. Others are reported and every later kernel leaves the
-// arrays alone (scan_bad, and no splitters for the read-only walk).
+// list; head_dev[1] = the heads that became extra splitters, head_dev[2] = the
+// elements of all lists. The kernels after it trust the offsets, so they are checked
+// here: from 0, non-decreasing, up to the n elements the call names (or, with
+// pad_ok, ending before them). Others are reported and every later kernel leaves the
+// arrays alone (scan_bad, no splitters for the read-only walk, no elements for the
+// walk over the lists).
 __global__ void __launch_bounds__(1024)
     bl_heads(const int64_t* __restrict__ off, const int32_t* __restrict__ heads, int64_t K, int64_t n, int logD,
              int64_t nb, uint32_t seed, int32_t* __restrict__ head_spl, int32_t* __restrict__ extra_elem,
-             int64_t* head_dev, DevCtl* ctl) {
+             int64_t* head_dev, bool pad_ok, DevCtl* ctl) {
     __shared__ int64_t s_first;
     __shared__ int s_warp[32];
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    bool ok = t != 32 || (off[0] == 0 && off[K] == n);
-    for (int64_t k = t; k < K; k += 1024) ok &= off[k] <= off[k + 1];
+    // (the first warp looks for the first list meanwhile)
+    bool ok = t != 32 || (off[0] == 0 && (off[K] == n || (pad_ok && off[K] < n)));
+    for (int64_t k = t - 32; t >= 32 && k < K; k += 1024 - 32) ok &= off[k] <= off[k + 1];
     if (t == 0) {
         int64_t k0 = 0;
         while (k0 < K && off[k0 + 1] == off[k0]) ++k0;
@@ -1578,7 +1583,7 @@ __global__ void __launch_bounds__(1024)
             record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
             ctl->scan_bad = 1;
             ctl->work[0] = WALK_OFF;
-            head_dev[0] = head_dev[1] = 0;
+            head_dev[0] = head_dev[1] = head_dev[2] = 0;
         }
         return;
     }
@@ -1645,6 +1650,7 @@ __global__ void __launch_bounds__(1024)
     if (t == 0) {
         ctl->ff_extra = total;
         head_dev[1] = total;
+        head_dev[2] = off[K];
     }
 }
 
@@ -1711,7 +1717,6 @@ __global__ void __launch_bounds__(LISTS_BLOCK)
     rs_walk_lists(const int32_t* __restrict__ succ, uint32_t* __restrict__ rec, Level0 L0,
                   const int64_t* __restrict__ off, int64_t K, const int32_t* __restrict__ head_spl, int pbits,
                   int extras, uint64_t* __restrict__ R1, DevCtl* ctl) {
-    if (ctl->scan_bad) return;
     const int64_t gh = L0.head_dev[0];
     L0.bh = gh >> L0.logD;
     L0.head_off = (uint32_t)(gh - (L0.bh << L0.logD));
@@ -1719,6 +1724,10 @@ __global__ void __launch_bounds__(LISTS_BLOCK)
     uint32_t j = blockIdx.x * LISTS_BLOCK + threadIdx.x;
     if (j >= g.nb + (uint32_t)L0.head_dev[1]) return;
     uint32_t cur = splitter_node32(j, g, L0.extra), pos = 0;
+    if (cur >= L0.head_dev[2]) {   // behind the last list
+        R1[j] = pack(NIL, 0);
+        return;
+    }
     int64_t k = find_list(off, K, cur);
     const uint32_t base = (uint32_t)off[k], len = (uint32_t)(off[k + 1] - off[k]);
     int32_t x = __ldg(succ + cur);
@@ -1761,22 +1770,47 @@ __global__ void __launch_bounds__(LISTS_BLOCK)
 
 // Records -> local ranks: the rank along all lists less the elements of the
 // later ones. A block takes one stretch of the elements and every thread keeps
-// the list it is in (the last one ends at n: bl_heads has checked the offsets).
-template <bool VEC>
+// the list it is in (bl_heads has checked the offsets; elements behind the last
+// list are left alone).
+//
+// AGAIN: when an error was recorded, the blocks take the lists one by one instead,
+// each in global memory (W: 8 bytes per element), so that a list that is none
+// spoils only its own ranks. A kernel of its own after this one for it costs every
+// call 4 to 6 us of 70 to 90.
+constexpr int AGAIN_CAP = 1024;   // splitters of a list ranked that way
+template <bool VEC, bool AGAIN>
 __global__ void __launch_bounds__(BLOCK)
     rs_expand_lists(int32_t* rank, int64_t n, const int32_t* __restrict__ S1, uint32_t r1, int pbits,
-                    const int64_t* __restrict__ off, int64_t K, const DevCtl* ctl) {
-    if (ctl->scan_bad) return;
+                    const int64_t* __restrict__ off, int64_t K, const int64_t* __restrict__ end_dev,
+                    const int32_t* __restrict__ succ, const int32_t* __restrict__ heads, uint64_t* W, uint32_t seed,
+                    DevCtl* ctl) {
+    const int64_t elems = min(n, *end_dev);   // 0: offsets that name no lists
+    const int failed = AGAIN ? ctl->failed : 0;
     const uint32_t mask = (1u << pbits) - 1;
     const int64_t per = ((n + gridDim.x - 1) / gridDim.x + 4 * BLOCK - 1) / (4 * BLOCK) * (4 * BLOCK);
-    const int64_t b = per * blockIdx.x, e = min(n, b + per);
-    if (b >= e) return;
+    const int64_t b = per * blockIdx.x, e = min(elems, b + per);
     int64_t k = find_list(off, K, min(b + (int64_t)threadIdx.x * 4, n - 1));
     int64_t end = off[k + 1];
+    if constexpr (AGAIN) {
+        if (failed && elems > 0) {
+            __shared__ uint64_t s_words[AGAIN_CAP];
+            __shared__ uint2 s_sub[2 * BLOCK];
+            __shared__ int s_k, s_work;
+            for (;;) {
+                const int64_t k = take_instance(&s_k, &ctl->batch_next, K);
+                if (k < 0) return;
+                const int64_t b = off[k], len = off[k + 1] - b;
+                if (len == 0 || heads[k] < 0 || heads[k] >= len) continue;   // (a head outside is recorded already)
+                list_ruling_set<BLOCK, AGAIN_CAP>(succ + b, len, heads[k], rank + b, W + b, s_words, s_sub, &s_work,
+                                                  seed ^ (uint32_t)k, 2, ctl);
+            }
+        }
+    }
+    if (b >= e) return;
     auto rank_of = [&](int64_t i, int32_t v) {
         while (i >= end) end = off[++k + 1];
         const uint32_t o = (uint32_t)v >> pbits;
-        return o < r1 ? (int32_t)((uint32_t)S1[o] - 1u - ((uint32_t)v & mask) - (uint32_t)(n - end)) : -1;
+        return o < r1 ? (int32_t)((uint32_t)S1[o] - 1u - ((uint32_t)v & mask) - (uint32_t)(elems - end)) : -1;
     };
     for (int64_t i = b + threadIdx.x * 4; i < e; i += 4 * BLOCK) {
         if (VEC && i + 3 < e) {
@@ -2291,8 +2325,13 @@ BatchMode lr_batch_mode(int64_t total, int64_t K, const Plan& batch_plan, bool o
     return total >= UNION_READONLY_MIN ? BATCH_READONLY : BATCH_BLOCKS;
 }
 
+// Up to this total the lists are ranked one by one when that fails together (one of
+// them is none), and elements may follow the last; a larger total keeps no room for it.
+constexpr int64_t UNION_AGAIN_MAX = int64_t(1) << 24;
+
 struct UnionPlan {
     Plan p;
+    bool again;
     RsLayout L;
     size_t off_gsucc, off_head_spl, off_extra, off_head_dev, bytes;
 };
@@ -2311,6 +2350,9 @@ UnionPlan union_plan(int walk_grid, int64_t total, int64_t K, BatchMode mode) {
     off = align_up(off + sizeof(int32_t) * (size_t)K, 256);
     U.off_extra = off;
     off = align_up(off + sizeof(int32_t) * (size_t)K, 256);
+    U.again = direct && total <= UNION_AGAIN_MAX;
+    // (the words of lists ranked one by one lie in front: blocks that start later still read it)
+    if (U.again) off = std::max(off, align_up(sizeof(uint64_t) * (size_t)total, 256));
     U.off_head_dev = off;
     U.bytes = off + 256;
     return U;
@@ -2333,6 +2375,7 @@ lrcc_status lr_batched_union(Ctx* c, cudaStream_t s, const int32_t* succ, const 
     U.head_spl = reinterpret_cast<int32_t*>(base + P.off_head_spl);
     U.extra_elem = reinterpret_cast<int32_t*>(base + P.off_extra);
     U.head_dev = reinterpret_cast<int64_t*>(base + P.off_head_dev);
+    U.again = P.again;
     return lr_enqueue_rs(c, s, succ, total, 0, rank, P.p, P.L, nullptr, &U);
 }
 
@@ -2396,7 +2439,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         const int g = stream_grid(c, (n + BL_TILE - 1) / BL_TILE * BLOCK, (const void*)bl_gsucc);
         phase_begin(c, s);
         bl_heads<<<1, 1024, 0, s>>>(U->off, U->heads, U->K, n, L0.logD, L0.nb, seed0, U->head_spl, U->extra_elem,
-                                    U->head_dev, ctl);
+                                    U->head_dev, U->again, ctl);
         if (L.readonly) bl_gsucc<<<g, BLOCK, 0, s>>>(succ, U->off, U->K, n, U->gsucc, ctl);
         phase_end(c, s, PH_BATCH_PREP);
         if (L.readonly) succ = U->gsucc;
@@ -2529,7 +2572,8 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         phase_begin(c, s);
         allow_smem(c, (const void*)rs_final_kernel, br_smem(16384));
         rs_final_kernel<<<1, FINAL_THREADS, smem, s>>>(R(lf), r, lf == 1 && L.direct ? (int)L.fixed : r, S(lf),
-                                                       val ? -1 : n, L.values ? (unsigned long long)n : 0ull, seed0, ctl);
+                                                       val ? -1 : n, L.values ? (unsigned long long)n : 0ull,
+                                                       U ? U->head_dev + 2 : nullptr, seed0, ctl);
         phase_end(c, s, PH_FINAL);
     }
     for (int l = L.levels - 1; l >= 1; --l) {
@@ -2565,13 +2609,18 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         }
         phase_end(c, s, PH_EXPAND0);
     } else if (L.direct && U) {
-        const bool v = aligned16(rank);
-        const void* k = v ? (const void*)rs_expand_lists<true> : (const void*)rs_expand_lists<false>;
-        const int g = stream_grid(c, groups, k);
-        phase_begin(c, s);
-        if (v) rs_expand_lists<true><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off, U->K, ctl);
-        else rs_expand_lists<false><<<g, BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off, U->K, ctl);
-        phase_end(c, s, PH_EXPAND0);
+        auto expand = [&](auto v, auto again) {
+            auto k = rs_expand_lists<decltype(v)::value, decltype(again)::value>;
+            phase_begin(c, s);
+            k<<<stream_grid(c, groups, (const void*)k), BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off,
+                                                                       U->K, U->head_dev + 2, succ, U->heads,
+                                                                       static_cast<uint64_t*>(c->ws), seed0, ctl);
+            phase_end(c, s, PH_EXPAND0);
+        };
+        if (aligned16(rank))
+            U->again ? expand(std::true_type(), std::true_type()) : expand(std::true_type(), std::false_type());
+        else
+            U->again ? expand(std::false_type(), std::true_type()) : expand(std::false_type(), std::false_type());
     } else if (L.direct) {
         const bool v = aligned16(rank);
         const void* k = v ? (const void*)rs_expand_direct<true> : (const void*)rs_expand_direct<false>;
