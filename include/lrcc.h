@@ -197,7 +197,7 @@ lrcc_status cc_label_host(const int32_t* src, const int32_t* dst, int64_t m, int
  * Batched list ranking: num_lists independent lists in one launch (a
  * persistent kernel takes the lists from a device work queue, largest first;
  * each list is ranked by one thread block), or, when the lists are long on
- * average (2^12 elements) or many (2^25 in all) and the batched plan's rs_level0
+ * average (2^12 elements) or many (more than 2^24 in all) and the batched plan's rs_level0
  * is 2, by the whole GPU as one list.
  * List k owns elements [node_off[k], node_off[k+1]) of succ and rank;
  * succ values and heads[k] are LOCAL ids (0-based within list k), and the

@@ -2308,26 +2308,30 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
 // for all of them; the host only knows the total and the count, so the mean
 // decides: lists of 2^12 elements on average go together (16 lists of up to 2^17:
 // 62 us, 269 by blocks; 64 of up to 2^20: 166 against 2618), of 2^13 when they
-// total less than 2^17, shorter ones by blocks (2000 of up to 2^14: 83 us), and a
-// large total is not left to single blocks. Lists of 2^22 elements and less on
-// average keep their records in the rank array, longer ones outgrow L2 and take
-// the read-only first level (chunks, scatter, placement) when they total 2^25.
+// total less than 2^17, shorter ones by blocks (2000 of up to 2^14: 83 us). A total
+// above 2^24 is never left to single blocks, where one long list among many short
+// ones lasts as long as it does alone (5000 lists of 256 elements and one of 2^24: 64.7
+// ms by blocks, 0.64 together), although short lists alone are faster
+// there (12,000 of 1500: 232 us by blocks, 336 together). Lists of 2^22
+// elements and less on average keep their records in the rank array, longer ones (and
+// those ranked in place) outgrow L2 and take the read-only first level (chunks,
+// scatter, placement) above 2^24 in all (3 lists of 2^23: 884 us, 40.7 ms by blocks).
 constexpr int64_t UNION_MIN = int64_t(1) << 15;
 constexpr int64_t UNION_DIRECT_MEAN = int64_t(1) << 22;
-constexpr int64_t UNION_READONLY_MIN = int64_t(1) << 25;
+constexpr int64_t UNION_LARGE = int64_t(1) << 24;
 constexpr int64_t UNION_MAX = int64_t(0x7FFFFFFE);   // global ids are int32
 
 BatchMode lr_batch_mode(int64_t total, int64_t K, const Plan& batch_plan, bool overlap) {
     if (batch_plan.rs_level0 != 2 || total < UNION_MIN || total > UNION_MAX - K) return BATCH_BLOCKS;
     const int64_t min_mean = int64_t(1) << (total < (int64_t(1) << 17) ? 13 : 12);
     if (total <= UNION_DIRECT_MEAN * K && !overlap)
-        return total >= min_mean * K || total >= UNION_READONLY_MIN ? BATCH_DIRECT : BATCH_BLOCKS;
-    return total >= UNION_READONLY_MIN ? BATCH_READONLY : BATCH_BLOCKS;
+        return total >= min_mean * K || total > UNION_LARGE ? BATCH_DIRECT : BATCH_BLOCKS;
+    return total > UNION_LARGE ? BATCH_READONLY : BATCH_BLOCKS;
 }
 
 // Up to this total the lists are ranked one by one when that fails together (one of
 // them is none), and elements may follow the last; a larger total keeps no room for it.
-constexpr int64_t UNION_AGAIN_MAX = int64_t(1) << 24;
+constexpr int64_t UNION_AGAIN_MAX = UNION_LARGE;
 
 struct UnionPlan {
     Plan p;
