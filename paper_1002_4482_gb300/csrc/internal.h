@@ -94,6 +94,7 @@ struct BatchUnion {
     int32_t* head_spl = nullptr;
     int32_t* extra_elem = nullptr;
     int64_t* head_dev = nullptr;
+    int form = 0;         // BatchMode
     bool again = false;   // ranked one by one when that fails together; elements may follow the last list
 };
 int rs_walk_grid(Ctx* c, const Plan& p);
@@ -217,7 +218,8 @@ lrcc_status cc_batch_gang_run(Ctx* c, const int32_t* src, const int32_t* dst, co
 size_t lr_batched_ws(int64_t total_nodes, int64_t count);
 // How batched lists are ranked: one block per list, all of them together as one
 // list with records in the rank array, or together by the read-only first level.
-enum BatchMode { BATCH_BLOCKS, BATCH_DIRECT, BATCH_READONLY };
+// BATCH_EITHER: the second or the third, as the device finds the sizes.
+enum BatchMode { BATCH_BLOCKS, BATCH_DIRECT, BATCH_READONLY, BATCH_EITHER };
 BatchMode lr_batch_mode(int64_t total, int64_t K, const Plan& batch_plan, bool overlap);
 size_t lr_batched_union_ws(int walk_grid, int64_t total, int64_t K, BatchMode mode);
 lrcc_status lr_batched_union(Ctx* c, cudaStream_t s, const int32_t* succ, const int64_t* off, const int32_t* heads,

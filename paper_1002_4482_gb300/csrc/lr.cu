@@ -579,6 +579,7 @@ __global__ void __launch_bounds__(BLOCK)
     rs_walk0c(const int32_t* __restrict__ succ, Level0 L0, Chunks C, uint64_t* __restrict__ R1, int* work,
               DevCtl* ctl) {
     if (L0.head_dev) {
+        if (!L0.head_dev[3]) return;   // batched lists that this form does not rank
         const int64_t gh = *L0.head_dev;
         L0.bh = gh >> L0.logD;
         L0.head_off = (uint32_t)(gh - (L0.bh << L0.logD));
@@ -737,7 +738,7 @@ __global__ void __launch_bounds__(BLOCK)
 // block per bucket; the row total goes to totals[bucket]. The start of each
 // bucket (a scan over NBK totals) is formed by the scatter blocks themselves.
 constexpr int SCAN_THREADS = 256;
-__global__ void __launch_bounds__(SCAN_THREADS) rs_scan_counts(int* counts, int G, int* totals) {
+__device__ __forceinline__ void scan_counts(int* counts, int G, int* totals) {
     __shared__ int s_warp[SCAN_THREADS / 32];
     int* row = counts + (int64_t)blockIdx.x * G;
     const int per = (G + SCAN_THREADS - 1) / SCAN_THREADS;
@@ -770,6 +771,9 @@ __global__ void __launch_bounds__(SCAN_THREADS) rs_scan_counts(int* counts, int 
         run += c;
     }
     if (threadIdx.x == SCAN_THREADS - 1) totals[blockIdx.x] = run;
+}
+__global__ void __launch_bounds__(SCAN_THREADS) rs_scan_counts(int* counts, int G, int* totals) {
+    scan_counts(counts, G, totals);
 }
 
 // Chunks of walk block g -> (element, rank) pairs at block g's offsets of
@@ -871,6 +875,7 @@ __global__ void __launch_bounds__(BLOCK, LRCC_SC_MINB)
     {
         int all = 0;
         bstart = block_scan(C.totals[t], &all);
+        if (all == 0) return;   // nothing was walked (and ctl->pairs is 0)
         if (blockIdx.x == 0 && t == 0) ctl->pairs = all;
     }
     s.cnt[t] = 0;
@@ -1506,67 +1511,32 @@ __device__ __forceinline__ int64_t find_list(const int64_t* __restrict__ off, in
     return lo;
 }
 
-constexpr int BL_TILE = BLOCK * 16;
-
-// Global successors; one binary search per tile of elements. Each thread
-// loads its 16 elements of the tile first, so that 16 streaming reads are in
-// flight, then converts them.
-__global__ void __launch_bounds__(BLOCK)
-    bl_gsucc(const int32_t* __restrict__ succ, const int64_t* __restrict__ off, int64_t K, int64_t n,
-             int32_t* __restrict__ gsucc, DevCtl* ctl) {
-    if (ctl->scan_bad) return;
-    constexpr int PER = BL_TILE / BLOCK;
-    __shared__ int64_t s_k;
-    const uint64_t pol = policy_evict_first();
-    for (int64_t t0 = (int64_t)blockIdx.x * BL_TILE; t0 < n; t0 += (int64_t)gridDim.x * BL_TILE) {
-        if (threadIdx.x == 0) s_k = find_list(off, K, t0);
-        __syncthreads();
-        int64_t k = s_k;
-        __syncthreads();
-        const int64_t tend = min(t0 + BL_TILE, n);
-        int32_t sx[PER];
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            const int64_t i = t0 + threadIdx.x + (int64_t)q * BLOCK;
-            sx[q] = i < tend ? ld_stream(succ + i, pol) : -1;
-        }
-#pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            const int64_t i = t0 + threadIdx.x + (int64_t)q * BLOCK;
-            if (i >= tend) break;
-            while (k + 1 < K && off[k + 1] <= i) ++k;
-            const int64_t base = off[k], len = off[k + 1] - base;
-            int32_t g = -1;
-            if (sx[q] != -1 && sx[q] != i - base) {
-                if (sx[q] < 0 || sx[q] >= len) record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)i);
-                else g = (int32_t)(base + sx[q]);
-            }
-            gsucc[i] = g;
-        }
-    }
-}
-
-// A value of the read-only walk's work counter at which it finds no splitter left.
-constexpr int WALK_OFF = 0x7F000000;
+constexpr int64_t LONG_LIST = int64_t(1) << 24;   // succ and rank of a longer one outgrow L2
 
 // One block: the first list's head (head_dev[0]) and the head splitter of every
 // list; head_dev[1] = the heads that became extra splitters, head_dev[2] = the
-// elements of all lists. The kernels after it trust the offsets, so they are checked
-// here: from 0, non-decreasing, up to the n elements the call names (or, with
-// pad_ok, ending before them). Others are reported and every later kernel leaves the
-// arrays alone (scan_bad, no splitters for the read-only walk, no elements for the
-// walk over the lists).
+// elements of all lists, head_dev[3] and [4] = whether the read-only first level or
+// the one with records in the rank array ranks them, head_dev[5] = the first list's
+// length. Where the call left the form open (BATCH_EITHER) it is the read-only one
+// when lists of more than LONG_LIST elements, which L2 does not hold, have most of
+// the elements (one of 2^27 among 63 short ones: 4.5 ms, 8.3 with records; one of
+// 2^26 and 63 of 2^20, a little over half: 3.5 and 4.1; one of 2^25 and 64 of 2^20, a third: 2.4
+// with records, 2.7 read-only).
+// The kernels after it trust the offsets, so they are checked here: from 0,
+// non-decreasing, up to the n elements the call names (or, with pad_ok, ending
+// before them). Others are reported and every later kernel leaves the arrays alone
+// (scan_bad; no form ranks them).
 __global__ void __launch_bounds__(1024)
     bl_heads(const int64_t* __restrict__ off, const int32_t* __restrict__ heads, int64_t K, int64_t n, int logD,
              int64_t nb, uint32_t seed, int32_t* __restrict__ head_spl, int32_t* __restrict__ extra_elem,
-             int64_t* head_dev, bool pad_ok, DevCtl* ctl) {
+             int64_t* head_dev, int form, bool pad_ok, DevCtl* ctl) {
+    __shared__ unsigned long long s_long;
     __shared__ int64_t s_first;
     __shared__ int s_warp[32];
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    // (the first warp looks for the first list meanwhile)
     bool ok = t != 32 || (off[0] == 0 && (off[K] == n || (pad_ok && off[K] < n)));
-    for (int64_t k = t - 32; t >= 32 && k < K; k += 1024 - 32) ok &= off[k] <= off[k + 1];
     if (t == 0) {
+        s_long = 0;
         int64_t k0 = 0;
         while (k0 < K && off[k0 + 1] == off[k0]) ++k0;
         s_first = k0;
@@ -1578,15 +1548,7 @@ __global__ void __launch_bounds__(1024)
         }
         *head_dev = gh;
     }
-    if (!__syncthreads_and(ok)) {
-        if (t == 0) {
-            record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
-            ctl->scan_bad = 1;
-            ctl->work[0] = WALK_OFF;
-            head_dev[0] = head_dev[1] = head_dev[2] = 0;
-        }
-        return;
-    }
+    __syncthreads();
     const int64_t k0 = s_first;
     const int64_t gh0 = *head_dev;
     const int64_t D = int64_t(1) << logD;
@@ -1605,13 +1567,18 @@ __global__ void __launch_bounds__(1024)
         *strat = b != bh && (uint32_t)(h - (b << logD)) == block_offset((uint32_t)b, size, seed);
     };
     int cnt = 0;
+    unsigned long long in_long = 0;
     for (int64_t k = kb; k < ke; ++k) {
-        if (k == k0 || off[k + 1] == off[k]) continue;
+        const int64_t len = off[k + 1] - off[k];
+        ok &= len >= 0;
+        if (len > LONG_LIST) in_long += (unsigned long long)len;
+        if (k == k0 || len == 0) continue;
         int64_t gh;
         bool strat;
         head_of(k, &gh, &strat);
         cnt += !strat;
     }
+    if (in_long) atomicAdd(&s_long, in_long);
     int incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1619,7 +1586,14 @@ __global__ void __launch_bounds__(1024)
         if (lane >= o) incl += x;
     }
     if (lane == 31) s_warp[wid] = incl;
-    __syncthreads();
+    if (!__syncthreads_and(ok)) {   // (up to here the offsets were only counted with)
+        if (t == 0) {
+            record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
+            ctl->scan_bad = 1;
+            for (int i = 0; i < 6; ++i) head_dev[i] = 0;
+        }
+        return;
+    }
     int before = 0, total = 0;
     for (int w = 0; w < 32; ++w) {
         before += w < wid ? s_warp[w] : 0;
@@ -1651,55 +1625,90 @@ __global__ void __launch_bounds__(1024)
         ctl->ff_extra = total;
         head_dev[1] = total;
         head_dev[2] = off[K];
+        const bool readonly = form == BATCH_READONLY || (form == BATCH_EITHER && 2 * s_long > (unsigned long long)n);
+        head_dev[3] = readonly;
+        head_dev[4] = !readonly;
+        head_dev[5] = k0 < K ? off[k0 + 1] - off[k0] : 0;
     }
 }
 
-// After the first-level walk: the splitter that ends list k (its word names no
-// next splitter) is linked to the next non-empty list's head splitter; the
-// unused extra slots become a chain of empty splitters after the last list.
-__global__ void __launch_bounds__(BLOCK)
-    bl_link(uint64_t* __restrict__ R1, int64_t r1_max, const int64_t* __restrict__ off, int64_t K,
-            const int32_t* __restrict__ head_spl, Level0 L0, DevCtl* ctl) {
-    if (ctl->scan_bad) return;
+// What the read-only form of batched lists reads beside the walk's own arrays.
+struct ListsGlobal {
+    int32_t* gsucc;          // successors as global ids
+    uint32_t* vis;           // the walk's marks and counts, to be cleared
+    int* counts;
+    int64_t ncounts;
+};
+
+// The read-only form's part of the first launch over the elements: block b's
+// `tile` elements' successors as global ids, and its share of what has to be cleared.
+template <int T>
+__device__ void lists_to_global(const int32_t* __restrict__ succ, const int64_t* __restrict__ off, int64_t K, int64_t n,
+                                int64_t tile, const ListsGlobal& G, DevCtl* ctl) {
+    for (int64_t i = (int64_t)blockIdx.x * T + threadIdx.x; i < G.ncounts; i += (int64_t)gridDim.x * T) G.counts[i] = 0;
+    const int64_t b = (int64_t)blockIdx.x * tile, e = min(n, b + tile);
+    if (b >= e) return;
+    for (int64_t w = (b >> 5) + threadIdx.x; w < (e + 31) >> 5; w += T) G.vis[w] = 0;   // tile: a multiple of 32
+    const uint64_t pol = policy_evict_first();
+    int64_t k = find_list(off, K, min(b + (int64_t)threadIdx.x, n - 1));
+    constexpr int U = 8;   // loads in flight
+    for (int64_t i0 = b + threadIdx.x; i0 < e; i0 += U * T) {
+        int32_t sx[U];
+#pragma unroll
+        for (int q = 0; q < U; ++q) sx[q] = i0 + q * T < e ? ld_stream(succ + i0 + q * T, pol) : -1;
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+            const int64_t i = i0 + q * T;
+            if (i >= e) break;
+            while (off[k + 1] <= i) ++k;
+            const int64_t base = off[k], len = off[k + 1] - base;
+            int32_t g = -1;
+            if (sx[q] != -1 && sx[q] != i - base) {
+                if (sx[q] < 0 || sx[q] >= len) record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)i);
+                else g = (int32_t)(base + sx[q]);
+            }
+            G.gsucc[i] = g;
+        }
+    }
+}
+
+// The next non-empty list after list k, or K, and the word of a splitter that ends
+// list k with `pos` elements: on to that list's head, with that list's length taken
+// off its weight, so that every sum from there back is list k's own. (The sum from the
+// first list's head is then that list's length if and only if all lists' elements were
+// met: the lengths taken off are those of all the others.)
+__device__ __forceinline__ uint64_t list_end(const int64_t* __restrict__ off, int64_t K, const int32_t* __restrict__ head_spl,
+                                             int64_t k, uint32_t pos) {
+    for (++k; k < K && off[k + 1] == off[k];) ++k;
+    return k < K ? pack((uint32_t)head_spl[k], pos - (uint32_t)(off[k + 1] - off[k])) : pack(NIL, pos);
+}
+
+// After the read-only walk, whose words of the last sublists name no next splitter.
+// Runs in blocks of the launch that scans the walk's counts (blocks first ..).
+__device__ void lists_link(uint64_t* __restrict__ R1, const int64_t* __restrict__ off, int64_t K,
+                           const int32_t* __restrict__ head_spl, Level0 L0, int first) {
     const int64_t gh = *L0.head_dev;
     L0.bh = gh >> L0.logD;
     L0.head_off = (uint32_t)(gh - (L0.bh << L0.logD));
     const int64_t r_real = L0.nb + *L0.extra_count;
-    for (int64_t j = (int64_t)blockIdx.x * BLOCK + threadIdx.x; j < r1_max; j += (int64_t)gridDim.x * BLOCK) {
-        if (j >= r_real) {
-            R1[j] = pack(j + 1 < r1_max ? (uint32_t)(j + 1) : NIL, 0);
-            continue;
-        }
+    const int64_t stride = (int64_t)(gridDim.x - first) * blockDim.x;
+    for (int64_t j = (int64_t)(blockIdx.x - first) * blockDim.x + threadIdx.x; j < r_real; j += stride) {
         const uint64_t w = R1[j];
         if (lo32(w) != NIL) continue;
-        const int64_t e = splitter_node0(j, L0);
-        int64_t k = find_list(off, K, e) + 1;
-        while (k < K && off[k + 1] == off[k]) ++k;
-        uint32_t nx = NIL;
-        if (k < K) nx = (uint32_t)head_spl[k];
-        else if (r_real < r1_max) nx = (uint32_t)r_real;
-        R1[j] = pack(nx, hi32(w));
+        R1[j] = list_end(off, K, head_spl, find_list(off, K, splitter_node0(j, L0)), hi32(w));
     }
 }
 
-// Global ranks -> local ranks: every element of list k is ahead of the
-// n - off[k + 1] elements of the later lists, which its local rank does not
-// count. A sublist never leaves its list (each list ends in a tail), so the
-// correction is taken once per first-level splitter, from its suffix sum,
-// before the scatter turns suffix sums into ranks.
-__global__ void __launch_bounds__(BLOCK)
-    bl_adjust(int32_t* __restrict__ S1, const int64_t* __restrict__ off, int64_t K, int64_t n, Level0 L0,
-              const DevCtl* ctl) {
-    if (ctl->scan_bad) return;
-    const int64_t gh = *L0.head_dev;
-    L0.bh = gh >> L0.logD;
-    L0.head_off = (uint32_t)(gh - (L0.bh << L0.logD));
-    const int64_t r_real = L0.nb + *L0.extra_count;   // the empty tail splitters own nothing
-    for (int64_t j = (int64_t)blockIdx.x * BLOCK + threadIdx.x; j < r_real; j += (int64_t)gridDim.x * BLOCK) {
-        const int64_t e = splitter_node0(j, L0);
-        if (e < 0 || e >= n) continue;
-        const int64_t k = find_list(off, K, e);
-        S1[j] = (int32_t)((uint32_t)S1[j] - (uint32_t)(n - off[k + 1]));
+__global__ void __launch_bounds__(SCAN_THREADS)
+    bl_scan_link(int* counts, int G, int* totals, uint64_t* __restrict__ R1, const int64_t* __restrict__ off, int64_t K,
+                 const int32_t* __restrict__ head_spl, Level0 L0) {
+    const bool run = L0.head_dev[3];
+    if (blockIdx.x >= NBK) {
+        if (run) lists_link(R1, off, K, head_spl, L0, NBK);
+    } else if (run) {
+        scan_counts(counts, G, totals);
+    } else if (threadIdx.x == 0) {   // nothing was walked
+        totals[blockIdx.x] = 0;
     }
 }
 
@@ -1708,15 +1717,20 @@ __global__ void __launch_bounds__(BLOCK)
 // walkers take the splitters in id order, so those in flight stay in a few
 // lists whose successors and records are in L2. The walk reads the local ids
 // itself, and the splitter that ends a list is linked to the next list's head
-// on the spot. 2048 lists of 2^8 to 2^20 elements: 3.58 ms, against 5.87 through
+// on the spot. 2048 lists of 2^8 to 2^20 elements: 3.46 ms, against 5.87 through
 // global successors, chunks, scatter and placement; the walk (2.6 ms, 96 G
 // steps/s) is bound by its two L2 requests per element, the expansion (0.8 ms) by
-// one gather each.
+// one gather each. Its 34 registers leave 12 of 16 blocks on an SM, which is better
+// than all: held to 32 registers the same lists take 3.65 ms.
 constexpr int LISTS_BLOCK = 128;   // short blocks: one lasts as long as its longest sublist
 __global__ void __launch_bounds__(LISTS_BLOCK)
     rs_walk_lists(const int32_t* __restrict__ succ, uint32_t* __restrict__ rec, Level0 L0,
                   const int64_t* __restrict__ off, int64_t K, const int32_t* __restrict__ head_spl, int pbits,
-                  int extras, uint64_t* __restrict__ R1, DevCtl* ctl) {
+                  int extras, uint64_t* __restrict__ R1, ListsGlobal LG, DevCtl* ctl) {
+    if (!L0.head_dev[4]) {
+        if (L0.head_dev[3]) lists_to_global<LISTS_BLOCK>(succ, off, K, L0.n, (int64_t)LISTS_BLOCK << L0.logD, LG, ctl);
+        return;
+    }
     const int64_t gh = L0.head_dev[0];
     L0.bh = gh >> L0.logD;
     L0.head_off = (uint32_t)(gh - (L0.bh << L0.logD));
@@ -1732,15 +1746,13 @@ __global__ void __launch_bounds__(LISTS_BLOCK)
     const uint32_t base = (uint32_t)off[k], len = (uint32_t)(off[k + 1] - off[k]);
     int32_t x = __ldg(succ + cur);
     CycleGuard guard(cur);
-    uint32_t next = NIL;
+    uint64_t last = NIL;   // the word's next splitter, and what goes off its weight
     for (;;) {
         // cur (a global id) belongs to owner j at position pos, x is its local successor
         rec[cur] = (j << pbits) | pos;
         ++pos;
         if (x == -1 || (uint32_t)x == cur - base) {
-            // the end of list k: on to the next list's head
-            for (++k; k < K && off[k + 1] == off[k];) ++k;
-            if (k < K) next = (uint32_t)head_spl[k];
+            last = list_end(off, K, head_spl, k, 0);   // on to the next list's head
             break;
         }
         if ((uint32_t)x >= len || guard.seen(base + (uint32_t)x)) {
@@ -1751,7 +1763,7 @@ __global__ void __launch_bounds__(LISTS_BLOCK)
         x = __ldg(succ + cur);   // on its way while cur is tested
         const int sj = splitter_index32(cur, g);
         if (sj >= 0) {
-            next = (uint32_t)sj;
+            last = (uint32_t)sj;
             break;
         }
         if (pos >> pbits) {
@@ -1765,13 +1777,11 @@ __global__ void __launch_bounds__(LISTS_BLOCK)
             pos = 0;
         }
     }
-    R1[j] = pack(next, pos);
+    R1[j] = pack(lo32(last), pos + hi32(last));
 }
 
-// Records -> local ranks: the rank along all lists less the elements of the
-// later ones. A block takes one stretch of the elements and every thread keeps
-// the list it is in (bl_heads has checked the offsets; elements behind the last
-// list are left alone).
+// Records -> local ranks, as rs_expand_direct (list_end makes the owners' sums the
+// lists' own). Elements behind the last list are left alone.
 //
 // AGAIN: when an error was recorded, the blocks take the lists one by one instead,
 // each in global memory (W: 8 bytes per element), so that a list that is none
@@ -1781,18 +1791,14 @@ constexpr int AGAIN_CAP = 1024;   // splitters of a list ranked that way
 template <bool VEC, bool AGAIN>
 __global__ void __launch_bounds__(BLOCK)
     rs_expand_lists(int32_t* rank, int64_t n, const int32_t* __restrict__ S1, uint32_t r1, int pbits,
-                    const int64_t* __restrict__ off, int64_t K, const int64_t* __restrict__ end_dev,
+                    const int64_t* __restrict__ off, int64_t K, const int64_t* __restrict__ head_dev,
                     const int32_t* __restrict__ succ, const int32_t* __restrict__ heads, uint64_t* W, uint32_t seed,
                     DevCtl* ctl) {
-    const int64_t elems = min(n, *end_dev);   // 0: offsets that name no lists
     const int failed = AGAIN ? ctl->failed : 0;
+    n = head_dev[4] ? min(n, head_dev[2]) : 0;   // 0: not ranked in this form
     const uint32_t mask = (1u << pbits) - 1;
-    const int64_t per = ((n + gridDim.x - 1) / gridDim.x + 4 * BLOCK - 1) / (4 * BLOCK) * (4 * BLOCK);
-    const int64_t b = per * blockIdx.x, e = min(elems, b + per);
-    int64_t k = find_list(off, K, min(b + (int64_t)threadIdx.x * 4, n - 1));
-    int64_t end = off[k + 1];
     if constexpr (AGAIN) {
-        if (failed && elems > 0) {
+        if (failed && n > 0) {
             __shared__ uint64_t s_words[AGAIN_CAP];
             __shared__ uint2 s_sub[2 * BLOCK];
             __shared__ int s_k, s_work;
@@ -1806,25 +1812,21 @@ __global__ void __launch_bounds__(BLOCK)
             }
         }
     }
-    if (b >= e) return;
-    auto rank_of = [&](int64_t i, int32_t v) {
-        while (i >= end) end = off[++k + 1];
+    auto rank_of = [&](int32_t v) {
         const uint32_t o = (uint32_t)v >> pbits;
-        return o < r1 ? (int32_t)((uint32_t)S1[o] - 1u - ((uint32_t)v & mask) - (uint32_t)(elems - end)) : -1;
+        return o < r1 ? (int32_t)((uint32_t)S1[o] - 1u - ((uint32_t)v & mask)) : -1;
     };
+    // a block takes one stretch of the elements: its owners stay in few lists
+    const int64_t per = ((n + gridDim.x - 1) / gridDim.x + 4 * BLOCK - 1) / (4 * BLOCK) * (4 * BLOCK);
+    const int64_t b = per * blockIdx.x, e = min(n, b + per);
     for (int64_t i = b + threadIdx.x * 4; i < e; i += 4 * BLOCK) {
         if (VEC && i + 3 < e) {
             int4* p = reinterpret_cast<int4*>(rank + i);
             const int4 v = __ldcs(p);
-            int4 r;
-            r.x = rank_of(i, v.x);
-            r.y = rank_of(i + 1, v.y);
-            r.z = rank_of(i + 2, v.z);
-            r.w = rank_of(i + 3, v.w);
-            __stcs(p, r);
+            __stcs(p, make_int4(rank_of(v.x), rank_of(v.y), rank_of(v.z), rank_of(v.w)));
         } else {
             for (int q = 0; q < 4; ++q)
-                if (i + q < e) rank[i + q] = rank_of(i + q, rank[i + q]);
+                if (i + q < e) rank[i + q] = rank_of(rank[i + q]);
         }
     }
 }
@@ -2224,7 +2226,7 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
     L.values = values;
     L.size[0] = n;
     // (batched lists, extra1 > 0, stay in L2 one after another at any total)
-    direct = direct && p.rs_level0 == 1 && n > p.rs_small && (extra1 > 0 || n <= DIRECT_MAX);
+    direct = direct && n > p.rs_small && (extra1 > 0 || (p.rs_level0 == 1 && n <= DIRECT_MAX));
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const size_t o = off;
@@ -2233,7 +2235,7 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
     };
     // in-place walk words, the (element, rank) pairs of the read-only walk, or
     // the split mark and local-rank arrays (each 256-byte aligned)
-    if (!direct) L.off_W0 = take(sizeof(uint64_t) * (size_t)n + 256);
+    if (!direct || p.rs_level0 == 2) L.off_W0 = take(sizeof(uint64_t) * (size_t)n + 256);
     if (values) L.off_P0 = take(sizeof(uint64_t) * (size_t)n);
     int64_t cur = n;
     int lvl = 0;
@@ -2247,11 +2249,11 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
         // level 1 may hold extra splitters (the heads of batched lists ranked as one list)
         int64_t nb = ((cur + (int64_t(1) << logD) - 1) >> logD) + (lvl == 0 ? extra1 : 0);
         if (lvl == 0 && given1 > 0) nb = given1;   // first-level splitters chosen by the caller
+        if (lvl == 0 && (direct || extra1 > 0)) L.fixed = nb - extra1;
         if (lvl == 0 && direct) {
             // as many position bits as the owners leave, extra owners included
             const int64_t heads = nb;   // with the heads of batched lists
             L.direct = true;
-            L.fixed = nb - extra1;
             for (L.pbits = 31; L.pbits > 0; --L.pbits) {
                 nb = heads + (n >> L.pbits);
                 if (nb <= (int64_t(1) << (32 - L.pbits))) break;
@@ -2316,16 +2318,23 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
 // elements and less on average keep their records in the rank array, longer ones (and
 // those ranked in place) outgrow L2 and take the read-only first level (chunks,
 // scatter, placement) above 2^24 in all (3 lists of 2^23: 884 us, 40.7 ms by blocks).
+// The mean says little where a few long lists have most of the elements: from 2^25 on,
+// where a list can outgrow L2, the device chooses between the two (bl_heads); the
+// launches of the other one end at once (16 us: 40 lists of 2^20 743 -> 756, 100 of
+// them 1633 -> 1629).
 constexpr int64_t UNION_MIN = int64_t(1) << 15;
 constexpr int64_t UNION_DIRECT_MEAN = int64_t(1) << 22;
 constexpr int64_t UNION_LARGE = int64_t(1) << 24;
+constexpr int64_t UNION_EITHER_MIN = int64_t(1) << 25;
 constexpr int64_t UNION_MAX = int64_t(0x7FFFFFFE);   // global ids are int32
 
 BatchMode lr_batch_mode(int64_t total, int64_t K, const Plan& batch_plan, bool overlap) {
     if (batch_plan.rs_level0 != 2 || total < UNION_MIN || total > UNION_MAX - K) return BATCH_BLOCKS;
     const int64_t min_mean = int64_t(1) << (total < (int64_t(1) << 17) ? 13 : 12);
     if (total <= UNION_DIRECT_MEAN * K && !overlap)
-        return total >= min_mean * K || total > UNION_LARGE ? BATCH_DIRECT : BATCH_BLOCKS;
+        return total >= UNION_EITHER_MIN                        ? BATCH_EITHER
+               : total >= min_mean * K || total > UNION_LARGE ? BATCH_DIRECT
+                                                              : BATCH_BLOCKS;
     return total > UNION_LARGE ? BATCH_READONLY : BATCH_BLOCKS;
 }
 
@@ -2342,14 +2351,14 @@ struct UnionPlan {
 
 UnionPlan union_plan(int walk_grid, int64_t total, int64_t K, BatchMode mode) {
     UnionPlan U;
-    const bool direct = mode == BATCH_DIRECT;
+    const bool direct = mode != BATCH_READONLY;
     U.p = plan_for(KIND_LR, total);
-    U.p.rs_level0 = direct ? 1 : 2;
+    U.p.rs_level0 = mode == BATCH_DIRECT ? 1 : 2;
     U.p.rs_small = std::min(U.p.rs_small, 16384);
     U.L = rs_layout(total, U.p, walk_grid, K, 0, direct);
     size_t off = align_up(U.L.bytes, 256);
     U.off_gsucc = off;
-    if (!direct) off = align_up(off + sizeof(int32_t) * (size_t)total, 256);
+    if (mode != BATCH_DIRECT) off = align_up(off + sizeof(int32_t) * (size_t)total, 256);
     U.off_head_spl = off;
     off = align_up(off + sizeof(int32_t) * (size_t)K, 256);
     U.off_extra = off;
@@ -2379,6 +2388,7 @@ lrcc_status lr_batched_union(Ctx* c, cudaStream_t s, const int32_t* succ, const 
     U.head_spl = reinterpret_cast<int32_t*>(base + P.off_head_spl);
     U.extra_elem = reinterpret_cast<int32_t*>(base + P.off_extra);
     U.head_dev = reinterpret_cast<int64_t*>(base + P.off_head_dev);
+    U.form = mode;
     U.again = P.again;
     return lr_enqueue_rs(c, s, succ, total, 0, rank, P.p, P.L, nullptr, &U);
 }
@@ -2440,13 +2450,10 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     L0.head_off = (uint32_t)(head - (L0.bh << L0.logD));
     L0.seed = seed0;
     if (U) {
-        const int g = stream_grid(c, (n + BL_TILE - 1) / BL_TILE * BLOCK, (const void*)bl_gsucc);
         phase_begin(c, s);
         bl_heads<<<1, 1024, 0, s>>>(U->off, U->heads, U->K, n, L0.logD, L0.nb, seed0, U->head_spl, U->extra_elem,
-                                    U->head_dev, U->again, ctl);
-        if (L.readonly) bl_gsucc<<<g, BLOCK, 0, s>>>(succ, U->off, U->K, n, U->gsucc, ctl);
+                                    U->head_dev, U->form, U->again, ctl);
         phase_end(c, s, PH_BATCH_PREP);
-        if (L.readonly) succ = U->gsucc;
         L0.head_dev = U->head_dev;
         L0.extra = U->extra_elem;
         L0.extra_count = &ctl->ff_extra;
@@ -2500,25 +2507,35 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         }
         phase_end(c, s, PH_WALK0);
     };
+    // overflow units' counts are accumulated with atomics (own units are stored whole)
+    const int64_t ncounts = (int64_t)NBK * L.units;
+    if (U) {
+        // the walk over the lists, or the global successors of the read-only one
+        phase_begin(c, s);
+        rs_walk_lists<<<(unsigned)((L0.nb + U->K + LISTS_BLOCK - 1) / LISTS_BLOCK), LISTS_BLOCK, 0, s>>>(
+            succ, reinterpret_cast<uint32_t*>(rank), L0, U->off, U->K, U->head_spl, L.pbits, (int)(L.size[1] - L.fixed),
+            R(1), ListsGlobal{U->gsucc, C.vis, C.counts, L.readonly ? ncounts : 0}, ctl);
+        phase_end(c, s, L.direct ? PH_WALK0 : PH_BATCH_PREP);
+    }
     if (L.readonly) {
-        cudaMemsetAsync(C.vis, 0, sizeof(uint32_t) * (size_t)((n + 31) / 32), s);
-        // overflow units' counts are accumulated with atomics (own units are stored whole)
-        cudaMemsetAsync(C.counts, 0, sizeof(int) * (size_t)NBK * (size_t)L.units, s);
+        if (!U) {
+            cudaMemsetAsync(C.vis, 0, sizeof(uint32_t) * (size_t)((n + 31) / 32), s);
+            cudaMemsetAsync(C.counts, 0, sizeof(int) * (size_t)ncounts, s);
+        }
+        const int32_t* next = U ? U->gsucc : succ;
         const int G = (int)L.grid;
         phase_begin(c, s);
-        if (p.rs_chains >= 4) rs_walk0c<4><<<G, BLOCK, 0, s>>>(succ, L0, C, R(1), &ctl->work[0], ctl);
-        else if (p.rs_chains == 2) rs_walk0c<2><<<G, BLOCK, 0, s>>>(succ, L0, C, R(1), &ctl->work[0], ctl);
-        else rs_walk0c<1><<<G, BLOCK, 0, s>>>(succ, L0, C, R(1), &ctl->work[0], ctl);
+        if (p.rs_chains >= 4) rs_walk0c<4><<<G, BLOCK, 0, s>>>(next, L0, C, R(1), &ctl->work[0], ctl);
+        else if (p.rs_chains == 2) rs_walk0c<2><<<G, BLOCK, 0, s>>>(next, L0, C, R(1), &ctl->work[0], ctl);
+        else rs_walk0c<1><<<G, BLOCK, 0, s>>>(next, L0, C, R(1), &ctl->work[0], ctl);
         phase_end(c, s, PH_WALK0);
         phase_begin(c, s);
-        rs_scan_counts<<<NBK, SCAN_THREADS, 0, s>>>(C.counts, L.units, C.totals);
+        if (U)
+            bl_scan_link<<<NBK + 4 * c->sms, SCAN_THREADS, 0, s>>>(C.counts, L.units, C.totals, R(1), U->off, U->K,
+                                                                  U->head_spl, L0);
+        else
+            rs_scan_counts<<<NBK, SCAN_THREADS, 0, s>>>(C.counts, L.units, C.totals);
         phase_end(c, s, PH_SCAN);
-        if (U) {
-            phase_begin(c, s);
-            bl_link<<<stream_grid(c, L.size[1], (const void*)bl_link), BLOCK, 0, s>>>(R(1), L.size[1], U->off, U->K,
-                                                                                    U->head_spl, L0, ctl);
-            phase_end(c, s, PH_BATCH_PREP);
-        }
     } else if (L.split) {
         auto walk0s = [&](auto mt, auto k) {
             using MT = decltype(mt);
@@ -2537,13 +2554,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
             else walk0s(uint32_t(), std::integral_constant<int, 1>());
         }
         phase_end(c, s, PH_WALK0);
-    } else if (L.direct && U) {
-        phase_begin(c, s);
-        rs_walk_lists<<<(unsigned)((L0.nb + U->K + LISTS_BLOCK - 1) / LISTS_BLOCK), LISTS_BLOCK, 0, s>>>(
-            succ, reinterpret_cast<uint32_t*>(rank), L0, U->off, U->K, U->head_spl, L.pbits, (int)(L.size[1] - L.fixed),
-            R(1), ctl);
-        phase_end(c, s, PH_WALK0);
-    } else if (L.direct) {
+    } else if (L.direct && !U) {
         phase_begin(c, s);
         rs_walk_direct<<<(unsigned)((L0.nb + BLOCK - 1) / BLOCK), BLOCK, 0, s>>>(
             succ, reinterpret_cast<uint32_t*>(rank), L0, L.pbits, (int)(L.size[1] - L.fixed), R(1), ctl);
@@ -2553,14 +2564,14 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         rs_walk_values<true><<<(unsigned)((L0.nb + BLOCK - 1) / BLOCK), BLOCK, 0, s>>>(
             W0, reinterpret_cast<uint64_t*>(base + L.off_P0), L0, R(1), ctl);
         phase_end(c, s, PH_WALK0);
-    } else {
+    } else if (!U) {
         walk0();
     }
     for (int l = 1; l < L.levels; ++l) {
         const uint32_t seed = mix32(seed0 + 0x9E3779B9u * (uint32_t)l);
         const unsigned g = (unsigned)((L.size[l + 1] + BLOCK - 1) / BLOCK);
         phase_begin(c, s);
-        const uint32_t fixed = l == 1 && L.direct ? (uint32_t)L.fixed : 0xFFFFFFFFu;
+        const uint32_t fixed = l == 1 && L.fixed > 0 ? (uint32_t)L.fixed : 0xFFFFFFFFu;
         if (val)
             rs_chase<true><<<g, BLOCK, 0, s>>>(R(l), (uint32_t)L.size[l], P(l), R(l + 1), (uint32_t)L.size[l + 1],
                                                L.logD[l], seed, fixed, &ctl->chased[l], ctl);
@@ -2575,9 +2586,9 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         const size_t smem = br_smem(r);
         phase_begin(c, s);
         allow_smem(c, (const void*)rs_final_kernel, br_smem(16384));
-        rs_final_kernel<<<1, FINAL_THREADS, smem, s>>>(R(lf), r, lf == 1 && L.direct ? (int)L.fixed : r, S(lf),
+        rs_final_kernel<<<1, FINAL_THREADS, smem, s>>>(R(lf), r, lf == 1 && L.fixed > 0 ? (int)L.fixed : r, S(lf),
                                                        val ? -1 : n, L.values ? (unsigned long long)n : 0ull,
-                                                       U ? U->head_dev + 2 : nullptr, seed0, ctl);
+                                                       U ? U->head_dev + 5 : nullptr, seed0, ctl);
         phase_end(c, s, PH_FINAL);
     }
     for (int l = L.levels - 1; l >= 1; --l) {
@@ -2586,12 +2597,6 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         rs_expand<<<g, BLOCK, 0, s>>>(P(l), (uint32_t)L.size[l], S(l + 1), (uint32_t)L.size[l + 1], S(l),
                                      val ? &ctl->chased[l] : nullptr, ctl);
         phase_end(c, s, PH_EXPAND);
-    }
-    if (U && L.readonly) {
-        phase_begin(c, s);
-        bl_adjust<<<stream_grid(c, L.size[1], (const void*)bl_adjust), BLOCK, 0, s>>>(S(1), U->off, U->K, n, L0,
-                                                                                       ctl);
-        phase_end(c, s, PH_BATCH_PREP);
     }
     if (L.readonly) {
         phase_begin(c, s);
@@ -2613,18 +2618,7 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         }
         phase_end(c, s, PH_EXPAND0);
     } else if (L.direct && U) {
-        auto expand = [&](auto v, auto again) {
-            auto k = rs_expand_lists<decltype(v)::value, decltype(again)::value>;
-            phase_begin(c, s);
-            k<<<stream_grid(c, groups, (const void*)k), BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off,
-                                                                       U->K, U->head_dev + 2, succ, U->heads,
-                                                                       static_cast<uint64_t*>(c->ws), seed0, ctl);
-            phase_end(c, s, PH_EXPAND0);
-        };
-        if (aligned16(rank))
-            U->again ? expand(std::true_type(), std::true_type()) : expand(std::true_type(), std::false_type());
-        else
-            U->again ? expand(std::false_type(), std::true_type()) : expand(std::false_type(), std::false_type());
+        // (below)
     } else if (L.direct) {
         const bool v = aligned16(rank);
         const void* k = v ? (const void*)rs_expand_direct<true> : (const void*)rs_expand_direct<false>;
@@ -2645,6 +2639,20 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
         if (v) rs_expand0<true><<<g, BLOCK, 0, s>>>(W0, n, S(1), L.size[1], rank, bias, ctl);
         else rs_expand0<false><<<g, BLOCK, 0, s>>>(W0, n, S(1), L.size[1], rank, bias, ctl);
         phase_end(c, s, PH_EXPAND0);
+    }
+    if (L.direct && U) {
+        auto expand = [&](auto v, auto again) {
+            auto k = rs_expand_lists<decltype(v)::value, decltype(again)::value>;
+            phase_begin(c, s);
+            k<<<stream_grid(c, groups, (const void*)k), BLOCK, 0, s>>>(rank, n, S(1), (uint32_t)L.size[1], L.pbits, U->off,
+                                                                       U->K, U->head_dev, succ, U->heads,
+                                                                       static_cast<uint64_t*>(c->ws), seed0, ctl);
+            phase_end(c, s, PH_EXPAND0);
+        };
+        if (aligned16(rank))
+            U->again ? expand(std::true_type(), std::true_type()) : expand(std::true_type(), std::false_type());
+        else
+            U->again ? expand(std::false_type(), std::true_type()) : expand(std::false_type(), std::false_type());
     }
     return cuda_status(cudaGetLastError());
 }

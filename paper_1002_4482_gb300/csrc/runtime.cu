@@ -607,10 +607,14 @@ lrcc_status lr_rank_batched_sized(const int32_t* succ, const int64_t* node_off, 
     // the batched plan is looked up by the total element count: its first-level
     // mode decides between one block per list and the lists ranked as one list
     const Plan p = plan_for(KIND_LR_BATCH, total_nodes);
-    const BatchMode mode = lr_batch_mode(total_nodes, num_lists, p, arrays_overlap(succ, rank, total_nodes));
+    BatchMode mode = lr_batch_mode(total_nodes, num_lists, p, arrays_overlap(succ, rank, total_nodes));
     if (mode != BATCH_BLOCKS) {
         const int grid = rs_walk_grid(c, plan_for(KIND_LR, total_nodes));
         st = ensure_ws(c, lr_batched_union_ws(grid, total_nodes, num_lists, mode));
+        if (st == LRCC_ERR_NOMEM && mode == BATCH_EITHER) {
+            mode = BATCH_DIRECT;   // a fifth of the workspace, and slower only for lists that outgrow L2
+            st = ensure_ws(c, lr_batched_union_ws(grid, total_nodes, num_lists, mode));
+        }
         if (st != LRCC_OK) return st;
         reset_ctl(c, c->stream);
         st = lr_batched_union(c, c->stream, succ, node_off, heads, num_lists, total_nodes, rank, mode);
