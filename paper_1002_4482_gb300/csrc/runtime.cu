@@ -999,8 +999,12 @@ int64_t lrcc_workspace_query(int kind, int64_t n, int64_t m) {
         }
         case 7: return (int64_t)lr_scan_forest_ws(n, scan_plan(n));   // lr_scan_forest
         case KIND_LR: {
-            // the walk's block count on the current device (as on a GB300 when none can be queried)
-            return n > p.rs_small ? (int64_t)rs_layout(n, p, rs_walk_grid_current(p), 0, 0, true).bytes : 0;
+            // the walk's block count on the current device (as on a GB300 when none can be
+            // queried); the most that a call takes (one with rank = succ keeps 8-byte words
+            // where others keep their records in the rank array)
+            if (n <= p.rs_small) return 0;
+            const int grid = rs_walk_grid_current(p);
+            return (int64_t)std::max(rs_layout(n, p, grid, 0, 0, true).bytes, rs_layout(n, p, grid).bytes);
         }
         case KIND_LR_WYLLIE: return n > p.rs_small ? (int64_t)lr_wyllie_ws(n, p) : 0;
         case KIND_CC:
