@@ -167,7 +167,7 @@ struct GangShape {
     size_t off_left, off_bits, bytes;   // behind the pairs: what each warp left, the giant, the bit map
 };
 
-GangShape gang_shape(int64_t m, int64_t n, int sms) {
+GangShape gang_shape(int64_t m, int64_t n, int sms, bool tight) {
     GangShape s;
     // a block for every 2048 edges or vertices: small graphs have cheaper barriers
     s.blocks = (int)std::max<int64_t>(1, std::min<int64_t>(sms, (std::max(m, n) + 2047) / 2048));
@@ -175,10 +175,11 @@ GangShape gang_shape(int64_t m, int64_t n, int sms) {
     // Pairs for three quarters of the edges of a sparse graph (a uniform one of 1
     // edge per vertex keeps two thirds after the first passes: 104 us, 128 with
     // half the room), for three eighths where a sample leaves fewer, for a quarter
-    // above 2^26 edges; a warp that keeps more reads the rest of its share again.
-    // Only the warps that have a share count.
+    // above 2^26 edges; a warp that keeps more reads the rest of its share again, so a
+    // quarter will do where memory is accounted for (tight). Only the warps that have a
+    // share count.
     const int64_t per = gang_share(m, warps);
-    s.capw = (int)(m > (int64_t(1) << 26) ? per / 4 : m < 2 * n ? per * 3 / 4 : per * 3 / 8) + 16;
+    s.capw = (int)(tight || m > (int64_t(1) << 26) ? per / 4 : m < 2 * n ? per * 3 / 4 : per * 3 / 8) + 16;
     s.capw = std::max(s.capw, GANG_STEP);   // one iteration's pairs, also of a short sample
     const int64_t used = std::min(warps, (m + GANG_STEP - 1) / GANG_STEP);   // the sample's shares are shorter
     s.off_left = align_up(sizeof(int2) * (size_t)s.capw * (size_t)std::max<int64_t>(used, 1), 256);
@@ -201,12 +202,12 @@ bool cc_gang_applies(const Plan& p) { return p.cc_hook == 1 && p.cc_max_rounds =
 
 bool cc_one_block_applies(int64_t m, int64_t n) { return n <= ONE_MAX_N && m <= ONE_MAX_M; }
 
-size_t cc_gang_ws(int64_t m, int64_t n, int sms) {
-    return cc_one_block_applies(m, n) ? 0 : gang_shape(m, n, sms).bytes;
+size_t cc_gang_ws(int64_t m, int64_t n, int sms, bool tight) {
+    return cc_one_block_applies(m, n) ? 0 : gang_shape(m, n, sms, tight).bytes;
 }
 
 lrcc_status cc_run_gang(Ctx* c, const int32_t* src, const int32_t* dst, int64_t m, int64_t n, int32_t* label,
-                        const Plan& p) {
+                        const Plan& p, bool tight) {
     if (cc_one_block_applies(m, n)) {
         const size_t smem = sizeof(int) * (size_t)n;
         allow_smem(c, (const void*)cc_one_block, sizeof(int) * ONE_MAX_N);
@@ -215,7 +216,7 @@ lrcc_status cc_run_gang(Ctx* c, const int32_t* src, const int32_t* dst, int64_t 
         phase_end(c, c->stream, PH_CC_LOOP);
         return cuda_status(cudaGetLastError());
     }
-    const GangShape S = gang_shape(m, n, c->sms);
+    const GangShape S = gang_shape(m, n, c->sms, tight);
     char* ws = static_cast<char*>(c->ws);
     GangParams P;
     P.g = GangGraph{src, dst, m, (int32_t)n, label};

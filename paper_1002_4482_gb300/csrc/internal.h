@@ -123,6 +123,7 @@ struct Ctx {
     DevCtl* ctl = nullptr;            // device control block
     void* ws = nullptr;
     size_t ws_bytes = 0;
+    bool reserved = false;            // adopted by a context: calls take what the query names
     void* io = nullptr;               // device copies of host-buffer calls' inputs and outputs
     size_t io_bytes = 0;
     cudaEvent_t io_ev[4] = {};        // host-buffer calls: staging free, uploaded, computed, downloaded
@@ -196,9 +197,10 @@ size_t cc_ws(int64_t m);
 // Rule 1 in one launch (cc_gang.cu): whether the plan takes it, its workspace, the run.
 bool cc_gang_applies(const Plan& p);
 bool cc_one_block_applies(int64_t m, int64_t n);
-size_t cc_gang_ws(int64_t m, int64_t n, int sms);
+// tight: room for a quarter of the edges as pairs, which is enough, and no more.
+size_t cc_gang_ws(int64_t m, int64_t n, int sms, bool tight);
 lrcc_status cc_run_gang(Ctx* c, const int32_t* src, const int32_t* dst, int64_t m, int64_t n, int32_t* label,
-                        const Plan& p);
+                        const Plan& p, bool tight);
 // The Shiloach-Vishkin round structure (plan.cc_hook = 4): workspace, run, round bound.
 size_t cc_sv_ws(int64_t n);
 lrcc_status cc_run_sv(Ctx* c, const int32_t* src, const int32_t* dst, int64_t m, int64_t n, int32_t* label,

@@ -417,11 +417,18 @@ lrcc_status cc_label_locked(Ctx* c, const int32_t* src, const int32_t* dst, int6
     const Plan p = plan_for(cc_plan_kind(m, n), n);
     const bool sv = p.cc_hook == 4;
     const bool gang = cc_gang_applies(p);
-    lrcc_status st = ensure_ws(c, sv ? cc_sv_ws(n) : gang ? cc_gang_ws(m, n, c->sms) : cc_ws(m));
+    // rule 1 in one launch takes more room for pairs than it needs (up to 6 bytes per edge
+    // instead of 2) where nobody accounts for the memory and it can be had
+    bool tight = gang && c->reserved && c->ws_bytes < cc_gang_ws(m, n, c->sms, false);
+    lrcc_status st = ensure_ws(c, sv ? cc_sv_ws(n) : gang ? cc_gang_ws(m, n, c->sms, tight) : cc_ws(m));
+    if (st == LRCC_ERR_NOMEM && gang && !tight) {
+        tight = true;
+        st = ensure_ws(c, cc_gang_ws(m, n, c->sms, true));
+    }
     if (st != LRCC_OK) return st;
     if (!(gang && cc_one_block_applies(m, n))) reset_ctl(c, c->stream);   // the one-block kernel clears its counters
     st = sv     ? cc_run_sv(c, src, dst, m, n, label, p)
-         : gang ? cc_run_gang(c, src, dst, m, n, label, p)
+         : gang ? cc_run_gang(c, src, dst, m, n, label, p, tight)
                 : cc_run(c, src, dst, m, n, label, p);
     c->last_kind = KIND_CC;
     return st;
@@ -954,6 +961,7 @@ lrcc_status lrcc_ctx_reserve(lrcc_ctx* ctx, void* stream, int64_t bytes) {
     if (st != LRCC_OK) return st;
     {
         std::lock_guard<std::mutex> lk(c->mu);
+        c->reserved = true;
         st = ensure_ws(c, (size_t)bytes);
     }
     std::lock_guard<std::mutex> lk(ctx->mu);
@@ -1008,7 +1016,7 @@ int64_t lrcc_workspace_query(int kind, int64_t n, int64_t m) {
         }
         case KIND_LR_WYLLIE: return n > p.rs_small ? (int64_t)lr_wyllie_ws(n, p) : 0;
         case KIND_CC:
-            return (int64_t)(p.cc_hook == 4 ? cc_sv_ws(n) : cc_gang_applies(p) ? cc_gang_ws(m, n, sms_current()) : cc_ws(m));
+            return (int64_t)(p.cc_hook == 4 ? cc_sv_ws(n) : cc_gang_applies(p) ? cc_gang_ws(m, n, sms_current(), true) : cc_ws(m));
         case KIND_LR_BATCH: {   // n = total elements, m = lists
             const Plan pb = plan_for(KIND_LR_BATCH, n);
             // the most that a call of this size takes (one with rank = succ keeps its
