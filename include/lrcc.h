@@ -147,8 +147,9 @@ lrcc_status lr_scan(const int32_t* succ, const int32_t* val, int64_t n, int32_t 
  * of the ruling set's first level, and the much smaller forest of splitters is
  * summed by pointer jumping (Sec. 3.1). Any values are accepted. An element
  * named by two successors, a cycle or a successor out of range records
- * LRCC_ERR_INVALID_INPUT. Workspace: 37 to 40 bytes per element (the first level
- * is sized for every element a head).
+ * LRCC_ERR_INVALID_INPUT. Workspace: 21 bytes per element, 30 up to 2^22 elements
+ * (the first level is sized for every element a head); lrcc_workspace_query still
+ * names 37.
  */
 lrcc_status lr_scan_forest(const int32_t* succ, const int32_t* val, int64_t n, int32_t* out, void* stream);
 

@@ -2657,15 +2657,14 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     return cuda_status(cudaGetLastError());
 }
 
-// Forest layout: walk words W0 (8 B per element), the has-predecessor bitmap,
-// and for r1_max = nb + n first-level splitters (every element could be a head)
-// 8 bytes for the elements' records (when they are not kept in W0), their packed
-// words and the extra splitters' elements; the layout keeps the size it had with
-// a second word buffer (37 to 40 bytes per element), which callers budget for.
+// Forest layout: walk words W0 (8 B per element), the has-predecessor bitmap, the
+// elements' records (8 B, up to WALK_NEAR elements: above they are kept in W0), and for
+// r1_max = nb + n first-level splitters (every element could be a head) their packed
+// words and the extra ones' elements (12 B): 21 bytes per element, 30 up to WALK_NEAR.
 struct ForestLayout {
     int logD;
     int64_t nb, r1_max;
-    size_t off_W0, off_pred, off_P0, off_R1, off_R1b, off_extra, bytes;
+    size_t off_W0, off_pred, off_P0, off_R1, off_extra, bytes;
 };
 
 ForestLayout forest_layout(int64_t n, int spacing0) {
@@ -2682,9 +2681,8 @@ ForestLayout forest_layout(int64_t n, int spacing0) {
     };
     F.off_W0 = take(sizeof(uint64_t) * (size_t)n);
     F.off_pred = take(sizeof(uint32_t) * (size_t)((n + 31) / 32));
-    F.off_P0 = take(sizeof(uint64_t) * (size_t)F.r1_max);
+    F.off_P0 = n <= WALK_NEAR ? take(sizeof(uint64_t) * (size_t)n) : F.off_W0;
     F.off_R1 = take(sizeof(uint64_t) * (size_t)F.r1_max);
-    F.off_R1b = take(sizeof(uint64_t) * (size_t)F.r1_max);
     F.off_extra = take(sizeof(int32_t) * (size_t)F.r1_max);
     F.bytes = off;
     return F;
@@ -2698,7 +2696,7 @@ lrcc_status lr_enqueue_scan_forest(Ctx* c, cudaStream_t s, const int32_t* succ, 
     char* base = static_cast<char*>(c->ws);
     uint64_t* W0 = reinterpret_cast<uint64_t*>(base + F.off_W0);
     uint32_t* pred = reinterpret_cast<uint32_t*>(base + F.off_pred);
-    uint64_t* P0 = n <= WALK_NEAR ? reinterpret_cast<uint64_t*>(base + F.off_P0) : W0;
+    uint64_t* P0 = reinterpret_cast<uint64_t*>(base + F.off_P0);
     uint64_t* R1 = reinterpret_cast<uint64_t*>(base + F.off_R1);
     int32_t* extra = reinterpret_cast<int32_t*>(base + F.off_extra);
     DevCtl* ctl = c->ctl;

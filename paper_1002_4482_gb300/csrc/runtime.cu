@@ -1005,7 +1005,9 @@ int64_t lrcc_workspace_query(int kind, int64_t n, int64_t m) {
             const Plan ps = scan_plan(n);
             return n > ps.rs_small ? (int64_t)rs_layout(n, ps, rs_walk_grid_current(ps), 0, 0, false, true).bytes : 0;
         }
-        case 7: return (int64_t)lr_scan_forest_ws(n, scan_plan(n));   // lr_scan_forest
+        // lr_scan_forest: at least the 37 bytes per element that its callers have always been
+        // told, of which the call takes 21 to 30
+        case 7: return std::max((int64_t)lr_scan_forest_ws(n, scan_plan(n)), 37 * n);
         case KIND_LR: {
             // the walk's block count on the current device (as on a GB300 when none can be
             // queried); the most that a call takes (one with rank = succ keeps 8-byte words
