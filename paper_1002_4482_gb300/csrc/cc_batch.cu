@@ -53,17 +53,14 @@ __global__ void __launch_bounds__(1024)
     __shared__ unsigned long long s_total, s_most;
     for (int t = threadIdx.x; t < CLASSES; t += blockDim.x) s_hist[t] = 0;
     if (threadIdx.x == 0) s_total = s_most = 0;
+    __syncthreads();
     bool ok = threadIdx.x > 0 || (voff[0] == 0 && eoff[0] == 0 && eoff[count] <= total_edges);
-    for (int64_t k = threadIdx.x; k < count; k += blockDim.x) ok &= voff[k] <= voff[k + 1] && eoff[k] <= eoff[k + 1];
-    if (!__syncthreads_and(ok) && threadIdx.x == 0) {
-        record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
-        ctl->scan_bad = 1;
-    }
     auto klass = [&](int64_t k, unsigned long long* work) {
         int64_t n, m;
         *work = 0;
         if (!batch_graph(eoff, voff, k, &n, &m)) {
             record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)k);
+            ok &= n >= 0 && m >= 0;
             return 0;
         }
         const int c = n + m <= 1 ? 0 : 63 - __clzll((unsigned long long)(n + m));
@@ -79,8 +76,12 @@ __global__ void __launch_bounds__(1024)
     }
     atomicAdd(&s_total, total);
     atomicMax(&s_most, most);
-    __syncthreads();
+    const bool sound = __syncthreads_and(ok);
     if (threadIdx.x == 0) {
+        if (!sound) {
+            record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
+            ctl->scan_bad = 1;
+        }
         int run = 0;
         for (int c = CLASSES - 1; c >= 0; --c) {
             if (c == 39) plan->large = run;
