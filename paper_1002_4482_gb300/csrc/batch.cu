@@ -50,10 +50,9 @@ constexpr int64_t CC_LARGE = int64_t(1) << 15;   // graphs above this many verti
 constexpr int SEG_BLOCK = 256;
 
 // Order instances by size class (floor(log2(size - 1))), largest first; order[count]
-// = how many have more than SMEM_ELEMS elements (they come first). The kernels
-// that rank lists (heads given) trust the offsets: from 0, non-decreasing, within
-// the `total` elements of the arrays and the workspace. Others are reported, and
-// no list is ranked (scan_bad).
+// = how many have more than SMEM_ELEMS elements (they come first). A list (heads
+// given) whose offsets do not lie within the `total` elements of the arrays and the
+// workspace is reported, and left out by the kernels that rank the others.
 __global__ void __launch_bounds__(1024)
     batch_order(const int64_t* __restrict__ off_a, const int64_t* __restrict__ off_b, const int32_t* heads,
                 int64_t count, int64_t total, int32_t* __restrict__ order, DevCtl* ctl) {
@@ -61,12 +60,11 @@ __global__ void __launch_bounds__(1024)
     __shared__ int s_start[NCLASS];
     for (int t = threadIdx.x; t < NCLASS; t += blockDim.x) s_hist[t] = 0;
     __syncthreads();
-    bool ok = !heads || threadIdx.x > 0 || (off_a[0] == 0 && off_a[count] <= total);
     // size class of instance k, -> class 0 when its offsets or head are invalid
     auto klass = [&](int64_t k) -> int {
         const int64_t na = off_a[k + 1] - off_a[k];
         bool bad = na < 0 || na > 0x7FFFFFFELL || (k == 0 && off_a[0] != 0);
-        ok &= na >= 0 || !heads;
+        if (heads) bad |= !list_in_range(off_a[k], na, total);
         int64_t size = na;
         if (off_b) {
             const int64_t nbv = off_b[k + 1] - off_b[k];
@@ -81,12 +79,8 @@ __global__ void __launch_bounds__(1024)
         return size <= 1 ? 0 : min(64 - __clzll((unsigned long long)(size - 1)), NCLASS - 1);
     };
     for (int64_t k = threadIdx.x; k < count; k += blockDim.x) atomicAdd(&s_hist[klass(k)], 1);
-    const bool sound = __syncthreads_and(ok);
+    __syncthreads();
     if (threadIdx.x == 0) {
-        if (!sound) {
-            record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
-            ctl->scan_bad = 1;
-        }
         int run = 0;
         for (int c = NCLASS - 1; c >= 0; --c) {
             s_start[c] = run;
@@ -129,19 +123,18 @@ template <int T, int CAP, bool LARGE>
 __global__ void __launch_bounds__(T)
     lr_batch_kernel(const int32_t* __restrict__ succ, const int64_t* __restrict__ off, const int32_t* __restrict__ heads,
                     int64_t count, const int32_t* __restrict__ order, const int32_t* __restrict__ split,
-                    int32_t* __restrict__ rank, uint64_t* W, uint32_t seed, int min_logD, DevCtl* ctl) {
+                    int64_t total, int32_t* __restrict__ rank, uint64_t* W, uint32_t seed, int min_logD, DevCtl* ctl) {
     extern __shared__ __align__(16) unsigned char lb_raw[];
     uint64_t* words = reinterpret_cast<uint64_t*>(lb_raw);
     uint2* sub = reinterpret_cast<uint2*>(lb_raw + sizeof(uint64_t) * CAP);
     __shared__ int s_k, s_work;
-    if (ctl->scan_bad) return;
     const int64_t first = LARGE ? 0 : *split, last = LARGE ? *split : count;
     for (;;) {
         const int64_t q = take_instance(&s_k, LARGE ? &ctl->batch_next : &ctl->seg_next, last - first);
         if (q < 0) break;
         const int64_t k = order[first + q];
         const int64_t b = off[k], n = off[k + 1] - b;
-        if (n <= 0 || n > 0x7FFFFFFELL) continue;
+        if (n <= 0 || n > 0x7FFFFFFELL || !list_in_range(b, n, total)) continue;
         const int head = heads[k];
         if (head < 0 || head >= n) continue;
         if (n <= CAP)
@@ -673,11 +666,12 @@ lrcc_status lr_batched_run(Ctx* c, const int32_t* succ, const int64_t* off, cons
     if (total_nodes > SMEM_ELEMS) {
         const int64_t most = std::min<int64_t>(count, total_nodes / SMEM_ELEMS);   // lists above SMEM_ELEMS at most
         const int g = (int)std::min<int64_t>(most, persistent_grid(c, (const void*)large_k, BT_LARGE, LR_SMEM_LARGE));
-        large_k<<<g, BT_LARGE, LR_SMEM_LARGE, s>>>(succ, off, heads, count, order, order + count, rank, W, seed, min_logD,
+        large_k<<<g, BT_LARGE, LR_SMEM_LARGE, s>>>(succ, off, heads, count, order, order + count, total_nodes, rank, W, seed, min_logD,
                                                    c->ctl);
     }
     const int g = (int)std::min<int64_t>(count, persistent_grid(c, (const void*)small_k, BT, LR_SMEM_BYTES));
-    small_k<<<g, BT, LR_SMEM_BYTES, s>>>(succ, off, heads, count, order, order + count, rank, W, seed, min_logD, c->ctl);
+    small_k<<<g, BT, LR_SMEM_BYTES, s>>>(succ, off, heads, count, order, order + count, total_nodes, rank, W, seed, min_logD,
+                                            c->ctl);
     phase_end(c, s, PH_LR_BATCH);
     return cuda_status(cudaGetLastError());
 }

@@ -33,19 +33,21 @@ struct BatchPlan {
     int gang;       // blocks per gang
 };
 
-__device__ __forceinline__ bool batch_graph(const int64_t* eoff, const int64_t* voff, int64_t k, int64_t* n, int64_t* m) {
+// Sizes of graph k; whether its offsets are those of a graph.
+__device__ __forceinline__ bool batch_graph(const int64_t* eoff, const int64_t* voff, int64_t k, int64_t total_edges,
+                                            int64_t* n, int64_t* m) {
     *n = voff[k + 1] - voff[k];
     *m = eoff[k + 1] - eoff[k];
-    return *n >= 0 && *n <= 0x7FFFFFFELL && *m >= 0 && *m <= 0x7FFFFFFFFFLL && (k > 0 || (voff[0] == 0 && eoff[0] == 0));
+    return *n >= 0 && *n <= 0x7FFFFFFELL && *m >= 0 && *m <= 0x7FFFFFFFFFLL && voff[k] >= 0 && eoff[k] >= 0 &&
+           eoff[k + 1] <= total_edges && (k > 0 || (voff[0] == 0 && eoff[0] == 0));
 }
 
 // Orders the graphs by size, largest first, those for gangs in front, and
 // chooses the gang size: as many gangs as the largest graph leaves room for
 // (the call lasts at least as long as that graph on its gang), of at least 8
-// blocks. One block. Offsets that do not start at 0, that decrease or that pass
-// total_edges are reported and no graph is labelled (scan_bad): the labels are a
-// graph's parents in local ids, and two gangs on overlapping ones would follow
-// each other's.
+// blocks. One block. A graph whose offsets are none (not from 0, decreasing, past
+// total_edges) is reported and left out. scan_bad = 1 when vertex offsets decrease,
+// so that graphs may overlap.
 __global__ void __launch_bounds__(1024)
     cc_batch_order(const int64_t* __restrict__ eoff, const int64_t* __restrict__ voff, int64_t count,
                    int64_t total_edges, int blocks, int32_t* __restrict__ order, BatchPlan* plan, DevCtl* ctl) {
@@ -54,13 +56,12 @@ __global__ void __launch_bounds__(1024)
     for (int t = threadIdx.x; t < CLASSES; t += blockDim.x) s_hist[t] = 0;
     if (threadIdx.x == 0) s_total = s_most = 0;
     __syncthreads();
-    bool ok = threadIdx.x > 0 || (voff[0] == 0 && eoff[0] == 0 && eoff[count] <= total_edges);
     auto klass = [&](int64_t k, unsigned long long* work) {
         int64_t n, m;
         *work = 0;
-        if (!batch_graph(eoff, voff, k, &n, &m)) {
+        if (!batch_graph(eoff, voff, k, total_edges, &n, &m)) {
             record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)k);
-            ok &= n >= 0 && m >= 0;
+            if (n < 0) ctl->scan_bad = 1;
             return 0;
         }
         const int c = n + m <= 1 ? 0 : 63 - __clzll((unsigned long long)(n + m));
@@ -76,12 +77,8 @@ __global__ void __launch_bounds__(1024)
     }
     atomicAdd(&s_total, total);
     atomicMax(&s_most, most);
-    const bool sound = __syncthreads_and(ok);
+    __syncthreads();
     if (threadIdx.x == 0) {
-        if (!sound) {
-            record_error(ctl, LRCC_ERR_INVALID_INPUT, -9);
-            ctl->scan_bad = 1;
-        }
         int run = 0;
         for (int c = CLASSES - 1; c >= 0; --c) {
             if (c == 39) plan->large = run;
@@ -96,6 +93,14 @@ __global__ void __launch_bounds__(1024)
     __syncthreads();
     for (int64_t k = threadIdx.x; k < count; k += blockDim.x)
         order[atomicAdd(&s_start[klass(k, &w)], 1)] = (int32_t)k;
+}
+
+// Whether graph k shares label entries with another graph (the whole block calls it).
+__device__ bool overlaps(const int64_t* __restrict__ voff, int64_t count, int64_t k) {
+    const int64_t b = voff[k], e = voff[k + 1];
+    bool hit = false;
+    for (int64_t i = threadIdx.x; i < count; i += blockDim.x) hit |= i != k && max(b, voff[i]) < min(e, voff[i + 1]);
+    return __syncthreads_or(hit);
 }
 
 // One graph by the gang; false when a barrier gave up.
@@ -128,13 +133,12 @@ __device__ bool gang_label(const GangParams& P, Gang& G, DevCtl* ctl, volatile u
 
 __global__ void __launch_bounds__(GANG_THREADS, 1)
     cc_batch_gangs(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, const int64_t* __restrict__ eoff,
-                   const int64_t* __restrict__ voff, const int32_t* __restrict__ order,
-                   const BatchPlan* __restrict__ plan, GangCtl* gcs, int2* pairs, int64_t pair_count, int32_t* label,
-                   DevCtl* ctl) {
+                   const int64_t* __restrict__ voff, int64_t count, int64_t total_edges,
+                   const int32_t* __restrict__ order, const BatchPlan* __restrict__ plan, GangCtl* gcs, int2* pairs,
+                   int64_t pair_count, int32_t* label, DevCtl* ctl) {
     __shared__ int s_flag;
     __shared__ uint64_t s_hook[HOOK_SLOTS];
     __shared__ GangParams s_P;
-    if (ctl->scan_bad) return;
     const int gang = plan->gang, gangs = (int)gridDim.x / gang, id = (int)blockIdx.x / gang;
     if (id >= gangs) return;
     GangCtl* gc = gcs + id;
@@ -149,10 +153,16 @@ __global__ void __launch_bounds__(GANG_THREADS, 1)
         if (!G.sync()) return;   // also: every block is done with the graph before
         const int q = (int)*(volatile unsigned*)&gc->instance;
         if (q >= large) return;
+        // a graph's labels are its parents in local ids: gangs on graphs that share some
+        // would follow each other's out of range
+        if (ctl->scan_bad && overlaps(voff, count, order[q])) {
+            if (!G.sync()) return;   // every block has read the instance
+            continue;
+        }
         if (threadIdx.x == 0) {
             const int64_t k = order[q];
             int64_t n, m;
-            batch_graph(eoff, voff, k, &n, &m);
+            batch_graph(eoff, voff, k, total_edges, &n, &m);
             GangParams& P = s_P;
             P.g = GangGraph{src + eoff[k], dst + eoff[k], m, (int32_t)n, label + voff[k]};
             // A sample of 7/8 edge per vertex from 2 edges per vertex up. The first
@@ -184,12 +194,12 @@ __global__ void __launch_bounds__(GANG_THREADS, 1)
 // The other graphs, one block each, largest first, in shared memory.
 __global__ void __launch_bounds__(SMALL_THREADS)
     cc_batch_small(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, const int64_t* __restrict__ eoff,
-                   const int64_t* __restrict__ voff, int64_t count, const int32_t* __restrict__ order,
-                   const BatchPlan* __restrict__ plan, int32_t* __restrict__ label, DevCtl* ctl) {
+                   const int64_t* __restrict__ voff, int64_t count, int64_t total_edges,
+                   const int32_t* __restrict__ order, const BatchPlan* __restrict__ plan, int32_t* __restrict__ label,
+                   DevCtl* ctl) {
     extern __shared__ int small_p[];
     __shared__ int s_q;
     volatile int* p = small_p;
-    if (ctl->scan_bad) return;
     const int first = plan->large;
     for (;;) {
         __syncthreads();   // the forest of the graph before is written out
@@ -199,7 +209,7 @@ __global__ void __launch_bounds__(SMALL_THREADS)
         if (q >= count) return;
         const int64_t k = order[q];
         int64_t n64, m64;
-        if (!batch_graph(eoff, voff, k, &n64, &m64) || n64 == 0) continue;
+        if (!batch_graph(eoff, voff, k, total_edges, &n64, &m64) || n64 == 0) continue;
         const int n = (int)n64, m = (int)m64;
         const int32_t* s = src + eoff[k];
         const int32_t* d = dst + eoff[k];
@@ -265,7 +275,7 @@ lrcc_status cc_batch_gang_run(Ctx* c, const int32_t* src, const int32_t* dst, co
     cc_batch_order<<<1, 1024, 0, s>>>(eoff, voff, count, total_edges, blocks, order, plan, c->ctl);
     phase_end(c, s, PH_BATCH_PREP);
     phase_begin(c, s);
-    void* args[] = {&src, &dst, &eoff, &voff, &order, &plan, &gcs, &pairs, &pair_count, &label, &c->ctl};
+    void* args[] = {&src, &dst, &eoff, &voff, &count, &total_edges, &order, &plan, &gcs, &pairs, &pair_count, &label, &c->ctl};
     const lrcc_status st = cuda_status(cudaLaunchCooperativeKernel((const void*)cc_batch_gangs, dim3(blocks),
                                                                    dim3(GANG_THREADS), args, 0, s));
     phase_end(c, s, PH_CC_LOOP);
@@ -273,7 +283,7 @@ lrcc_status cc_batch_gang_run(Ctx* c, const int32_t* src, const int32_t* dst, co
     phase_begin(c, s);
     allow_smem(c, (const void*)cc_batch_small, SMALL_SMEM);
     const int g = (int)std::min<int64_t>(count, persistent_grid(c, (const void*)cc_batch_small, SMALL_THREADS, SMALL_SMEM));
-    cc_batch_small<<<g, SMALL_THREADS, SMALL_SMEM, s>>>(src, dst, eoff, voff, count, order, plan, label, c->ctl);
+    cc_batch_small<<<g, SMALL_THREADS, SMALL_SMEM, s>>>(src, dst, eoff, voff, count, total_edges, order, plan, label, c->ctl);
     phase_end(c, s, PH_CC_BATCH);
     return cuda_status(cudaGetLastError());
 }

@@ -30,7 +30,8 @@ struct DevCtl {
     int cc_stop;         // component loop: the last pass joined nothing
     int seg_next;        // batched union path: next edge slice of the current pass
     int seg_next_v;      // batched union path: next vertex slice of the current shortcut
-    int scan_bad;        // skip the work (values outside the supported range, offsets that name no lists or graphs)
+    int scan_bad;        // lists: skip the work (values outside the supported range, offsets that name no lists);
+                         // batched graphs: some may overlap
     int ff_extra;        // forest ranks: list heads that became extra first-level splitters
     int failed;          // an error was recorded by this call (status also holds those of earlier calls)
     int gave_up;         // a gang's barrier gave up in this call: what its launch left is not to be read

@@ -15,9 +15,16 @@ __device__ __forceinline__ int64_t take_instance(int* s_k, int* next, int64_t co
     return *s_k < count ? *s_k : -1;
 }
 
+// Whether a list of n elements from element b on lies in a call's `total` elements.
+__device__ __forceinline__ bool list_in_range(int64_t b, int64_t n, int64_t total) {
+    return b >= 0 && n >= 0 && b <= total && n <= total - b;
+}
+
 // Rank one larger list with a ruling set inside the block; W is the list's
 // slice of the 8-byte word workspace, R the splitters' packed words in shared
-// memory (next splitter, sublist length; before the walk: successor, 1).
+// memory (next splitter, sublist length; before the walk: successor, 1). Indices
+// read back from W are checked: offsets that overlap (reported) put two blocks on
+// the same words.
 template <int T, int CAP>
 __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_t* rank, uint64_t* W,
                                 uint64_t* R, uint2* sub, int* s_work, uint32_t seed, int min_logD, DevCtl* ctl) {
@@ -64,7 +71,7 @@ __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_
             const uint64_t w = W[cur];
             const uint32_t lo = lo32(w), hi = hi32(w);
             if (lo & SPL) {
-                next = hi;
+                if (hi < (uint32_t)r) next = hi;
                 break;
             }
             if ((hi & VIS) || ++steps > n) {
@@ -88,9 +95,9 @@ __device__ void list_ruling_set(const int32_t* succ, int64_t n, int head, int32_
         const uint64_t w = W[i];
         const uint32_t lo = lo32(w), hi = hi32(w);
         int out;
-        if (lo & SPL) {
+        if ((lo & SPL) && hi < (uint32_t)r) {
             out = (int)lo32(R[hi]) - 1;
-        } else if (hi & VIS) {
+        } else if (!(lo & SPL) && (hi & VIS) && (hi & ~VIS) < (uint32_t)r) {
             out = (int)lo32(R[hi & ~VIS]) - (int)lo - 1;
         } else {
             record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)i);

@@ -1524,8 +1524,7 @@ constexpr int64_t LONG_LIST = int64_t(1) << 24;   // succ and rank of a longer o
 // with records, 2.7 read-only).
 // The kernels after it trust the offsets, so they are checked here: from 0,
 // non-decreasing, up to the n elements the call names (or, with pad_ok, ending
-// before them). Others are reported and every later kernel leaves the arrays alone
-// (scan_bad; no form ranks them).
+// before them). Others are reported and no form ranks the lists together (scan_bad).
 __global__ void __launch_bounds__(1024)
     bl_heads(const int64_t* __restrict__ off, const int32_t* __restrict__ heads, int64_t K, int64_t n, int logD,
              int64_t nb, uint32_t seed, int32_t* __restrict__ head_spl, int32_t* __restrict__ extra_elem,
@@ -1795,10 +1794,11 @@ __global__ void __launch_bounds__(BLOCK)
                     const int32_t* __restrict__ succ, const int32_t* __restrict__ heads, uint64_t* W, uint32_t seed,
                     DevCtl* ctl) {
     const int failed = AGAIN ? ctl->failed : 0;
+    const int64_t total = n;
     n = head_dev[4] ? min(n, head_dev[2]) : 0;   // 0: not ranked in this form
     const uint32_t mask = (1u << pbits) - 1;
     if constexpr (AGAIN) {
-        if (failed && n > 0) {
+        if (failed) {
             __shared__ uint64_t s_words[AGAIN_CAP];
             __shared__ uint2 s_sub[2 * BLOCK];
             __shared__ int s_k, s_work;
@@ -1806,7 +1806,11 @@ __global__ void __launch_bounds__(BLOCK)
                 const int64_t k = take_instance(&s_k, &ctl->batch_next, K);
                 if (k < 0) return;
                 const int64_t b = off[k], len = off[k + 1] - b;
-                if (len == 0 || heads[k] < 0 || heads[k] >= len) continue;   // (a head outside is recorded already)
+                if (len == 0) continue;
+                if (!list_in_range(b, len, total) || (k == 0 && b != 0) || heads[k] < 0 || heads[k] >= len) {
+                    if (threadIdx.x == 0) record_error(ctl, LRCC_ERR_INVALID_INPUT, (int)k);
+                    continue;
+                }
                 list_ruling_set<BLOCK, AGAIN_CAP>(succ + b, len, heads[k], rank + b, W + b, s_words, s_sub, &s_work,
                                                   seed ^ (uint32_t)k, 2, ctl);
             }

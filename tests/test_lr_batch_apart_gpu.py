@@ -65,3 +65,30 @@ def test_elements_behind_the_last_list(mix, pad, shift):
     assert status == lrcc.OK
     assert np.array_equal(got[:total], oracle.lr_rank_batched(succ, off, heads))
     assert (got[total:] == -7).all()
+
+
+@pytest.mark.parametrize("sizes,k", [([300, 9000, 24_577, 77, 500, 30_000, 900] + [100] * 5, 3),  # one block per list
+                                     ([40_000, 24_576, 60_000, 24_577, 30_000, 50_000], 2)])      # together
+@pytest.mark.parametrize("case", ["decreasing", "overlapping", "past_the_end", "first_not_zero", "negative"])
+def test_one_bad_offset(sizes, k, case):
+    succ, off, heads = (a.astype(t) for a, t in zip(gen.list_batch(np.asarray(sizes, np.int64), 8),
+                                                    (np.int32, np.int64, np.int32)))
+    want, good = oracle.lr_rank_batched(succ, off, heads), off.copy()
+    touched = {k - 1, k}                          # the lists that the offset bounds
+    if case == "decreasing":
+        off[k] = good[k - 1] - 9                  # list k also runs over the end of list k - 2
+        touched.add(k - 2)
+    elif case == "overlapping":
+        off[k] = good[k + 1] + 5                  # list k - 1 runs into list k + 1
+        touched.add(k + 1)
+    elif case == "past_the_end":
+        off[k] = good[-1] + 1000
+    elif case == "first_not_zero":
+        off[0] = 2
+        touched = {0}
+    else:
+        off[k] = -5
+    status, got = _call(succ, off, heads)
+    assert status == lrcc.ERR_INVALID_INPUT
+    for i in set(range(len(sizes))) - touched:
+        assert np.array_equal(got[good[i]:good[i + 1]], want[good[i]:good[i + 1]]), i
