@@ -7,10 +7,13 @@
 // first passes only roots are chased and a full shortcut over all vertices
 // happens once at the end instead of once per round. And the pairs stay in
 // stretches private to a warp, so nothing is appended through a shared counter
-// and a round with few edges costs one barrier.
+// and a round with few edges costs one barrier. Labelling a part of the edges
+// first and leaving out what lies inside the largest tree after it is the idea of
+// Afforest (Sutton, Ben-Nun, Barak, "Optimizing Parallel Graph Connectivity
+// Computation via Subgraph Sampling", IPDPS 2018).
 //
 // Measured against the loop of launches (us): uniform 2^20 vertices, 2^22 edges
-// 146 / 266; 1021 vertices, 2042 edges 17 / 56; paths of 8M vertices 383 / 926;
+// 146 / 266; 1021 vertices, 2042 edges 11-15 / 50-56; paths of 8M vertices 383 / 926;
 // R-MAT scale 20, 2^24 edges 144 / 2350; scale 24, 2^28 edges 1725 / 2498 (bound by
 // the gathers the member table does not answer, one L2 request each).
 //

@@ -2,16 +2,19 @@
 // sparse ruling set / random splitter method (Sec. 3.2, Algorithms 2 and 3).
 //
 // Ruling set, as built here for sm_103a:
-//   select   (RS1+RS2) one streaming pass packs succ into 8-byte words
-//            W[i] = (next | splitter flag, splitter index or weight 1); one
-//            random splitter per block of D indices, the head is splitter 0;
-//   walk     (RS3) every splitter's sublist is walked once; each visited
-//            word is overwritten IN PLACE with (prefix weight, owner | VIS),
-//            so a step costs one random sector read plus its write-back;
+//   select   (RS1+RS2) one random splitter per block of D indices, at a hashed
+//            offset, so a walk recognises it without a mark; the head is
+//            splitter 0;
+//   walk     (RS3) every splitter's sublist is walked once. Up to 2^24 elements
+//            the walk reads succ and writes a 4-byte record (owner, position)
+//            into the rank array (rs_walk_direct, rs_walk_lists), above it writes
+//            what it visits as 32-byte chunks (rs_walk0c); weighted ranks walk
+//            packed 8-byte words (rs_walk_values, rs_walk), split arrays are a
+//            plan option (rs_walk0s);
 //   recurse  (RS4) the list of splitters, weighted by sublist size, is again
 //            cut by splitters and walked (rs_chase) until it fits one thread
 //            block, which ranks it in shared memory (block_rank.cuh);
-//   expand   (RS5) streaming passes turn (prefix, owner) into ranks.
+//   expand   (RS5) streaming passes turn (owner, position) into ranks.
 // Every level stores the inclusive suffix weight S (elements from a node to
 // the tail, itself included); the final rank is S - 1.
 #include <algorithm>
@@ -1717,9 +1720,9 @@ __global__ void __launch_bounds__(SCAN_THREADS)
 // lists whose successors and records are in L2. The walk reads the local ids
 // itself, and the splitter that ends a list is linked to the next list's head
 // on the spot. 2048 lists of 2^8 to 2^20 elements: 3.46 ms, against 5.87 through
-// global successors, chunks, scatter and placement; the walk (2.6 ms, 96 G
-// steps/s) is bound by its two L2 requests per element, the expansion (0.8 ms) by
-// one gather each. Its 34 registers leave 12 of 16 blocks on an SM, which is better
+// global successors, chunks, scatter and placement; the walk (2.5 ms, 100 G
+// steps/s) is bound by its L2 requests (2.6 per element), the expansion (0.73 ms)
+// by one gather each. Its 34 registers leave 12 of 16 blocks on an SM, which is better
 // than all: held to 32 registers the same lists take 3.65 ms.
 constexpr int LISTS_BLOCK = 128;   // short blocks: one lasts as long as its longest sublist
 __global__ void __launch_bounds__(LISTS_BLOCK)
