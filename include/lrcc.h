@@ -205,7 +205,9 @@ lrcc_status cc_label_host(const int32_t* src, const int32_t* dst, int64_t m, int
  * List k owns elements [node_off[k], node_off[k+1]) of succ and rank;
  * succ values and heads[k] are LOCAL ids (0-based within list k), and the
  * ranks are local too. node_off is int64[num_lists + 1] on the device,
- * non-decreasing, node_off[0] = 0. Every list must be valid.
+ * non-decreasing, node_off[0] = 0. Every list must be valid; one that is not is
+ * reported, and the others are ranked all the same in a call of at most 2^24
+ * elements.
  */
 lrcc_status lr_rank_batched(const int32_t* succ, const int64_t* node_off, const int32_t* heads,
                             int64_t num_lists, int32_t* rank, void* stream);
