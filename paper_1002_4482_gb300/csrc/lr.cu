@@ -1719,18 +1719,21 @@ __global__ void __launch_bounds__(SCAN_THREADS)
 // walkers take the splitters in id order, so those in flight stay in a few
 // lists whose successors and records are in L2. The walk reads the local ids
 // itself, and the splitter that ends a list is linked to the next list's head
-// on the spot. 2048 lists of 2^8 to 2^20 elements: 3.46 ms, against 5.87 through
-// global successors, chunks, scatter and placement; the walk (2.5 ms, 100 G
+// on the spot. 2048 lists of 2^8 to 2^20 elements: 3.30 ms, against 5.87 through
+// global successors, chunks, scatter and placement; the walk (2.4 ms, 104 G
 // steps/s) is bound by its L2 requests (2.6 per element), the expansion (0.73 ms)
-// by one gather each. Its 34 registers leave 12 of 16 blocks on an SM, which is better
-// than all: held to 32 registers the same lists take 3.65 ms.
+// by one gather each. Fewer warps keep more of the lists in flight in L2: with 44
+// registers 10 of 16 blocks fit an SM (EITHER: both forms in the kernel), 3.46 ms with
+// 12, 3.65 with all. Without the other form 38 registers, 12 blocks (14 lists of 2^20:
+// walk 155 us, 161 with all).
 constexpr int LISTS_BLOCK = 128;   // short blocks: one lasts as long as its longest sublist
-__global__ void __launch_bounds__(LISTS_BLOCK)
+template <bool EITHER>
+__global__ void __launch_bounds__(LISTS_BLOCK, 1)
     rs_walk_lists(const int32_t* __restrict__ succ, uint32_t* __restrict__ rec, Level0 L0,
                   const int64_t* __restrict__ off, int64_t K, const int32_t* __restrict__ head_spl, int pbits,
                   int extras, uint64_t* __restrict__ R1, ListsGlobal LG, DevCtl* ctl) {
     if (!L0.head_dev[4]) {
-        if (L0.head_dev[3]) lists_to_global<LISTS_BLOCK>(succ, off, K, L0.n, (int64_t)LISTS_BLOCK << L0.logD, LG, ctl);
+        if (EITHER && L0.head_dev[3]) lists_to_global<LISTS_BLOCK>(succ, off, K, L0.n, (int64_t)LISTS_BLOCK << L0.logD, LG, ctl);
         return;
     }
     const int64_t gh = L0.head_dev[0];
@@ -1789,7 +1792,7 @@ __global__ void __launch_bounds__(LISTS_BLOCK)
 // each in global memory (W: 8 bytes per element), so that a list that is none
 // spoils only its own ranks. A kernel of its own after this one for it costs every
 // call 4 to 6 us of 70 to 90.
-constexpr int AGAIN_CAP = 1024;   // splitters of a list ranked that way
+constexpr int AGAIN_CAP = 256;   // splitters of a list ranked that way (L1 for the gathers, not speed there)
 template <bool VEC, bool AGAIN>
 __global__ void __launch_bounds__(BLOCK)
     rs_expand_lists(int32_t* rank, int64_t n, const int32_t* __restrict__ S1, uint32_t r1, int pbits,
@@ -2327,8 +2330,7 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
 // scatter, placement) above 2^24 in all (3 lists of 2^23: 884 us, 40.7 ms by blocks).
 // The mean says little where a few long lists have most of the elements: from 2^25 on,
 // where a list can outgrow L2, the device chooses between the two (bl_heads); the
-// launches of the other one end at once (16 us: 40 lists of 2^20 743 -> 756, 100 of
-// them 1633 -> 1629).
+// launches of the other one end at once (16 us of 735 for 40 lists of 2^20).
 constexpr int64_t UNION_MIN = int64_t(1) << 15;
 constexpr int64_t UNION_DIRECT_MEAN = int64_t(1) << 22;
 constexpr int64_t UNION_LARGE = int64_t(1) << 24;
@@ -2519,7 +2521,8 @@ lrcc_status lr_enqueue_rs(Ctx* c, cudaStream_t s, const int32_t* succ, int64_t n
     if (U) {
         // the walk over the lists, or the global successors of the read-only one
         phase_begin(c, s);
-        rs_walk_lists<<<(unsigned)((L0.nb + U->K + LISTS_BLOCK - 1) / LISTS_BLOCK), LISTS_BLOCK, 0, s>>>(
+        auto walk = L.readonly ? rs_walk_lists<true> : rs_walk_lists<false>;
+        walk<<<(unsigned)((L0.nb + U->K + LISTS_BLOCK - 1) / LISTS_BLOCK), LISTS_BLOCK, 0, s>>>(
             succ, reinterpret_cast<uint32_t*>(rank), L0, U->off, U->K, U->head_spl, L.pbits, (int)(L.size[1] - L.fixed),
             R(1), ListsGlobal{U->gsucc, C.vis, C.counts, L.readonly ? ncounts : 0}, ctl);
         phase_end(c, s, L.direct ? PH_WALK0 : PH_BATCH_PREP);
