@@ -2323,11 +2323,11 @@ RsLayout rs_layout(int64_t n, const Plan& p, int walk_grid, int64_t extra1, int6
 // total less than 2^17, shorter ones by blocks (2000 of up to 2^14: 83 us). A total
 // above 2^24 is never left to single blocks, where one long list among many short
 // ones lasts as long as it does alone (5000 lists of 256 elements and one of 2^24: 64.7
-// ms by blocks, 0.64 together), although short lists alone are faster
-// there (12,000 of 1500: 232 us by blocks, 336 together). Lists of 2^22
+// ms by blocks, 0.67 together), although short lists alone are faster
+// there (12,000 of 1500: 232 us by blocks, 323 together). Lists of 2^22
 // elements and less on average keep their records in the rank array, longer ones (and
 // those ranked in place) outgrow L2 and take the read-only first level (chunks,
-// scatter, placement) above 2^24 in all (3 lists of 2^23: 884 us, 40.7 ms by blocks).
+// scatter, placement) above 2^24 in all (3 lists of 2^23: 858 us, 40.7 ms by blocks).
 // The mean says little where a few long lists have most of the elements: from 2^25 on,
 // where a list can outgrow L2, the device chooses between the two (bl_heads); the
 // launches of the other one end at once (16 us of 735 for 40 lists of 2^20).
